@@ -33,7 +33,7 @@ def _nvcc() -> str:
 
 def _sources():
     return [os.path.join(CSRC, s) for s in SOURCES_CU + SOURCES_CPP] + \
-        [os.path.join(CSRC, "plan.hpp"), os.path.join(INC, "stc.h")]
+        [os.path.join(CSRC, "plan.hpp"), os.path.join(CSRC, "splitmm.cuh"), os.path.join(INC, "stc.h")]
 
 
 def stale() -> bool:

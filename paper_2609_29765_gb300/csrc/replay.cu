@@ -26,6 +26,7 @@
 #include <stdexcept>
 
 #include "plan.hpp"
+#include "splitmm.cuh"
 
 namespace stc {
 namespace {
@@ -54,6 +55,8 @@ constexpr int kRStage = kRKc * kRStLd;
 constexpr int kRPacked = kNbMax * (kNbMax + 1) / 2;
 constexpr int kRCbuf = (kRLd * kNbMax > kRPacked ? kRLd * kNbMax : kRPacked) + 16;
 constexpr size_t kRSmemBytes = (size_t)(kRCbuf + 2 * kRStage + kNbMax) * sizeof(double);
+static_assert(kRKc == kSpK && kSpDoubles <= kRStage && kRCbuf % 2 == 0 && kRStage % 2 == 0,
+              "a staging buffer holds the digits of one chunk, 16-byte aligned");
 
 // packed lower triangle of an nb x nb tile, column-major: (r, c), r >= c
 __host__ __device__ __forceinline__ int pk(int nb, int r, int c) { return c * nb - (c * (c + 1)) / 2 + r; }
@@ -1877,9 +1880,16 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                 if (!s_ok) break;
                 for (int k0 = 0; k0 < u.klen; k0 += kRKc) {
                     const int K = min(kRKc, u.klen - k0);
-                    sn_stage(S0, kRStLd, F, A, 0, A.h, k0, K);
-                    __syncthreads();
-                    mma_scatter<true, true>(C, 0, A.h, A.h, S0, kRStLd, S0, kRStLd, K, s_rm, s_rm, w);
+                    const double* ga = F + A.off + (size_t)k0 * A.ld;
+                    if (sp_worth(A.h * A.h / 2, K) &&
+                        sp_stage_a(S0, A.h, [&](int r, int k) { return __ldcg(ga + r + (size_t)k * A.ld); }, K)) {
+                        sp_product<true>(S0, A.h, S0, A.h,
+                                         [&](int r, int c, double v) { C[pk(w, s_rm[r], s_rm[c])] -= v; });
+                    } else {
+                        sn_stage(S0, kRStLd, F, A, 0, A.h, k0, K);
+                        __syncthreads();
+                        mma_scatter<true, true>(C, 0, A.h, A.h, S0, kRStLd, S0, kRStLd, K, s_rm, s_rm, w);
+                    }
                     __syncthreads();
                 }
             }
@@ -1915,10 +1925,19 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                 if (!s_ok) break;
                 for (int k0 = 0; k0 < u.klen; k0 += kRKc) {
                     const int K = min(kRKc, u.klen - k0);
-                    sn_stage(S0, kRStLd, F, A, u.ar0, Ra, k0, K);
-                    sn_stage(S1, kRStLd, F, B, 0, B.h, k0, K);
-                    __syncthreads();
-                    mma_scatter<false, false>(C, kRLd, Ra, B.h, S0, kRStLd, S1, kRStLd, K, s_rm, s_cm, 0);
+                    const double* ga = F + A.off + u.ar0 + (size_t)k0 * A.ld;
+                    const double* gb = F + B.off + (size_t)k0 * B.ld;
+                    if (sp_worth(Ra * B.h, K) &&
+                        sp_stage_ab(S0, Ra, [&](int r, int k) { return __ldcg(ga + r + (size_t)k * A.ld); }, S1, B.h,
+                                    [&](int r, int k) { return __ldcg(gb + r + (size_t)k * B.ld); }, K)) {
+                        sp_product<false>(S0, Ra, S1, B.h,
+                                          [&](int r, int c, double v) { C[s_rm[r] + s_cm[c] * kRLd] -= v; });
+                    } else {
+                        sn_stage(S0, kRStLd, F, A, u.ar0, Ra, k0, K);
+                        sn_stage(S1, kRStLd, F, B, 0, B.h, k0, K);
+                        __syncthreads();
+                        mma_scatter<false, false>(C, kRLd, Ra, B.h, S0, kRStLd, S1, kRStLd, K, s_rm, s_cm, 0);
+                    }
                     __syncthreads();
                 }
             }
@@ -1945,12 +1964,20 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                         if (Cn <= 0) continue;
                         for (int k0 = p; k0 < pn; k0 += kRKc) {
                             const int K = min(kRKc, pn - k0);
-                            const int Cp = ((Cn + 3) & ~3) + 4;
-                            for_rc(Cp, K, [&](int c, int k) {
-                                S1[c + k * kRStLd] = c < Cn ? __ldcg(DT + pn + c + (size_t)(k0 + k) * D.ld) : 0.0;
-                            });
-                            __syncthreads();
-                            mma_sub<false>(C + pn * kRLd, kRLd, R, Cn, C + k0 * kRLd, kRLd, S1, kRStLd, K);
+                            const double *X = C + k0 * kRLd, *gb = DT + pn + (size_t)k0 * D.ld;
+                            double* Y = C + pn * kRLd;
+                            if (sp_worth(R * Cn, K) &&
+                                sp_stage_ab(S0, R, [&](int r, int k) { return X[r + k * kRLd]; }, S1, Cn,
+                                            [&](int c, int k) { return __ldcg(gb + c + (size_t)k * D.ld); }, K)) {
+                                sp_product<false>(S0, R, S1, Cn, [&](int r, int c, double v) { Y[r + c * kRLd] -= v; });
+                            } else {
+                                const int Cp = ((Cn + 3) & ~3) + 4;
+                                for_rc(Cp, K, [&](int c, int k) {
+                                    S1[c + k * kRStLd] = c < Cn ? __ldcg(gb + c + (size_t)k * D.ld) : 0.0;
+                                });
+                                __syncthreads();
+                                mma_sub<false>(Y, kRLd, R, Cn, X, kRLd, S1, kRStLd, K);
+                            }
                             __syncthreads();
                         }
                     }
