@@ -291,6 +291,9 @@ struct SnPlan {
     int64_t item_doubles() const { return (poff() + nsn() + 31) / 32 * 32; }
 };
 
+// Device queue order of a supernodal plan's factorization tasks, scheduled on `procs` CTAs.
+std::vector<int32_t> sn_queue_order(const SnPlan& S, int procs);
+
 // Device copies of a supernodal plan (uploaded on first use per device).
 struct SnDev {
     SnDevCell* cells = nullptr;
@@ -309,6 +312,7 @@ struct SnDev {
     SnSCon* scons = nullptr;
     int32_t* rows = nullptr;        // the supernodes' row lists (permuted indices)
     int32_t* cell_rowoff = nullptr;
+    int32_t* order = nullptr;       // task of each queue position (sn_queue_order)
     int device = -1;
 };
 

@@ -21,6 +21,7 @@
 #include <functional>
 #include <memory>
 #include <mutex>
+#include <queue>
 #include <stdexcept>
 #include <vector>
 
@@ -358,4 +359,80 @@ void stc_plan::build_device_form(stc::SnPlan& S, const vector<int32_t>& snof,
             }
         }
     }
+}
+
+// Device queue order of the factorization tasks for `procs` CTAs: list scheduling of the
+// task DAG under a cost model, tasks in order of their modelled start (a topological order:
+// a task starts once every cell it reads is final).  Among ready tasks the longest path to
+// the end goes first.  Costs in microseconds, from per-phase clocks on the GB300: a
+// 16-column chunk of an update 1.2 + 0.3 per eight 16 x 8 units, a TRSM panel of 32 columns
+// 5, POTRF 1.3 per column, 3 per task.
+vector<int32_t> stc::sn_queue_order(const stc::SnPlan& S, int procs) {
+    const int32_t nt = (int32_t)S.dtasks.size(), nc = (int32_t)S.dcells.size();
+    vector<double> cost(nt), bl(nt, 0.0);
+    vector<int32_t> deps(nt, 0), left(nc, 0);
+    // readers of a cell (an update reads two cells, an off-diagonal task its diagonal cell)
+    vector<int64_t> rbeg(nc + 1, 0);
+    auto each_source = [&](int32_t t, auto&& f) {
+        const stc::SnDevTask& k = S.dtasks[t];
+        for (int32_t u = k.ubeg; u < k.uend; ++u) {
+            f(S.dupds[u].a);
+            if (S.dupds[u].b != S.dupds[u].a) f(S.dupds[u].b);
+        }
+        if (k.kind != stc::SN_T_DIAG) f(k.diag);
+    };
+    for (int32_t t = 0; t < nt; ++t) {
+        const stc::SnDevTask& k = S.dtasks[t];
+        const int32_t w = S.dcells[k.cell].w;
+        double c = 3.0;
+        for (int32_t u = k.ubeg; u < k.uend; ++u) {
+            const stc::SnDevUpd& x = S.dupds[u];
+            const int32_t ra = (x.ar1 - x.ar0 + 15) / 16, cb = (S.dcells[x.b].h + 7) / 8;
+            const int32_t units = k.kind == stc::SN_T_DIAG ? ra * (ra + 1) : ra * cb;
+            c += ((x.klen + 15) / 16) * (1.2 + 0.3 * ((units + 7) / 8));
+        }
+        c += k.kind == stc::SN_T_DIAG ? 1.3 * w : 5.0 * ((w + 31) / 32);
+        cost[t] = c;
+        ++left[k.cell];
+        each_source(t, [&](int32_t s) { ++rbeg[s + 1]; ++deps[t]; });
+    }
+    for (int32_t c = 0; c < nc; ++c) rbeg[c + 1] += rbeg[c];
+    vector<int32_t> readers(rbeg[nc]);
+    {
+        vector<int64_t> at(rbeg.begin(), rbeg.end() - 1);
+        for (int32_t t = 0; t < nt; ++t) each_source(t, [&](int32_t s) { readers[at[s]++] = t; });
+    }
+    // the tasks are stored in a topological order: longest paths in one backward sweep
+    vector<double> cbl(nc, 0.0);  // largest path of a cell's readers
+    for (int32_t t = nt - 1; t >= 0; --t) {
+        bl[t] = cost[t] + cbl[S.dtasks[t].cell];
+        each_source(t, [&](int32_t s) { cbl[s] = std::max(cbl[s], bl[t]); });
+    }
+    typedef std::pair<double, int32_t> E;
+    std::priority_queue<E> ready;                                      // longest path first
+    std::priority_queue<E, vector<E>, std::greater<E>> running;       // earliest finish first
+    for (int32_t t = 0; t < nt; ++t)
+        if (!deps[t]) ready.push(E(bl[t], -t));
+    vector<int32_t> order;
+    order.reserve(nt);
+    int idle = std::max(procs, 1);
+    double now = 0.0;
+    while (!ready.empty() || !running.empty()) {
+        while (idle > 0 && !ready.empty()) {
+            const int32_t t = -ready.top().second;
+            ready.pop();
+            order.push_back(t);
+            running.push(E(now + cost[t], t));
+            --idle;
+        }
+        const int32_t t = running.top().second, c = S.dtasks[t].cell;
+        now = running.top().first;
+        running.pop();
+        ++idle;
+        if (--left[c] == 0)
+            for (int64_t q = rbeg[c]; q < rbeg[c + 1]; ++q)
+                if (--deps[readers[q]] == 0) ready.push(E(bl[readers[q]], -readers[q]));
+    }
+    if ((int32_t)order.size() != nt) throw std::logic_error("supernodal task set: a dependency cycle");
+    return order;
 }
