@@ -151,7 +151,9 @@ __device__ __forceinline__ double sp_double(long long T, int E) {
     const int lz = __clzll((long long)mag);
     const unsigned long long nrm = mag << lz;
     // biased exponent of the leading bit: 1023 + 63 - lz + E - 2102; the hidden bit adds one
-    const unsigned long long bits = ((unsigned long long)(unsigned)(E - 1016 - lz - 1) << 52) + ((nrm + 0x400ull) >> 11);
+    // (rounded after the shift: a mantissa of ones carries into the exponent)
+    const unsigned long long bits =
+        ((unsigned long long)(unsigned)(E - 1016 - lz - 1) << 52) + (nrm >> 11) + ((nrm >> 10) & 1ull);
     return __longlong_as_double((long long)(bits | ((unsigned long long)T & 0x8000000000000000ull)));
 }
 

@@ -71,3 +71,13 @@ def test_graded_pivots(route):
 def test_ragged_dense(route, n):
     Ap, Ai, Ax = I.random_spd(n, 0.6, seed=n)
     _check(n, Ap, Ai, Ax, None, 128, route, ordering="natural")
+
+
+# tau = 2 makes sums of products that end just below a power of two (53 leading ones): the
+# rounding of an exact sum has to carry into the exponent
+@pytest.mark.parametrize("route", ["supernodal", "semisparse", "dense"])
+@pytest.mark.parametrize("theta", [(2.0, 0.6, 0.7), (0.5, 0.5, 1.0), (8.0, 0.25, 1.0)])
+def test_sums_below_powers_of_two(route, theta):
+    dims = (14, 12, 8, 0)
+    Ap, Ai, coords = I.stcov_pattern(*dims)
+    _check(len(Ap) - 1, Ap, Ai, I.stcov_values(theta, *dims), coords, 32, route)
