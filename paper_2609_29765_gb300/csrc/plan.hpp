@@ -251,6 +251,17 @@ struct SnSCon {
     int32_t mode;      // SN_SC_*
     int32_t pad;
 };
+constexpr int kSnSolveRows = 256;
+struct SnSolveNode {   // one supernode as the solve sees it
+    int64_t off;       // arena offset of its panel
+    int64_t uoff;      // its update vector (also its place in srel)
+    int64_t poff;      // its backward partials, (chunks - 1) x w
+    int32_t first, w;  // first column, columns
+    int32_t ld;        // panel rows
+    int32_t roff;      // its rows below the diagonal block in the row lists
+    int32_t kbeg, kend;  // children
+    int32_t chunk, nchunk;  // its chunks (at least one)
+};
 struct SnPlan {
     std::vector<int32_t> first;
     std::vector<int64_t> rptr;
@@ -285,6 +296,17 @@ struct SnPlan {
     std::vector<SnSTask> stasks;     // selected inverse, reverse supernode order
     std::vector<SnSCon> scons;
     std::vector<int32_t> cell_rowoff;  // per cell: offset in rows of its first row
+    // Solve: the supernodal elimination tree.  A supernode's rows below its own columns are
+    // rows of its parent; step J leaves an update vector over them, cut into chunks of
+    // kSnSolveRows rows (a device task each; the first also solves J's diagonal block).
+    std::vector<SnSolveNode> snodes;
+    std::vector<int32_t> skids;        // children of each supernode, ascending
+    std::vector<int32_t> srel;         // per below row: its position in the parent's rows
+    std::vector<int32_t> schunk_own;   // per chunk: row supernode that owns its first row
+    std::vector<int32_t> sfwd, sbwd;   // queue order, two per task: supernode, chunk
+    int64_t nu = 0, npart = 0;         // doubles of the update vectors, of the backward partials
+    int32_t nchunks = 0;
+    int32_t wmax = 0;                  // widest supernode
     int32_t nsn() const { return (int32_t)first.size() - 1; }
     // item layout of the supernodal route: the arena, then one logdet partial per supernode
     int64_t poff() const { return (arena + 31) / 32 * 32; }
@@ -293,6 +315,9 @@ struct SnPlan {
 
 // Device queue order of a supernodal plan's factorization tasks, scheduled on `procs` CTAs.
 std::vector<int32_t> sn_queue_order(const SnPlan& S, int procs);
+
+// The solve's part of a supernodal plan (called at the end of its construction).
+void sn_build_solve(SnPlan& S);
 
 // Device copies of a supernodal plan (uploaded on first use per device).
 struct SnDev {
@@ -312,6 +337,8 @@ struct SnDev {
     SnSCon* scons = nullptr;
     int32_t* rows = nullptr;        // the supernodes' row lists (permuted indices)
     int32_t* cell_rowoff = nullptr;
+    SnSolveNode* snodes = nullptr;
+    int32_t *skids = nullptr, *srel = nullptr, *schunk_own = nullptr, *sfwd = nullptr, *sbwd = nullptr;
     int32_t* order = nullptr;       // task of each queue position (sn_queue_order)
     int device = -1;
 };

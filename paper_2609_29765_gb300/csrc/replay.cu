@@ -1337,73 +1337,6 @@ static_assert(kNbMax <= 128 && kThreads == 256, "the solve's register prefetch c
 // diagonal tile (>= (nb + 1) nb and (kd + 1) nb doubles) + four 32 x 33 panel triangles
 constexpr size_t kSolveSmem = ((size_t)kLdc * kNbMax + 4 * 32 * 33) * sizeof(double);
 
-// Diagonal-block substitution with the unit lower triangular M = L diag(L)^{-1} (Ls
-// holds M, its columns scaled beforehand, off the dependency chain), panels of 32: warp 0
-// solves the panel's 32x32 triangle with its rows (forward) or columns (backward) in
-// registers, one lane per row/column, values broadcast by shuffle, so a step of the chain
-// is one shuffle and one FMA; the rows below (forward) or above (backward) the panel are
-// then updated with one thread per row.  Forward: v <- M^{-1} v (the caller scales by
-// diag(L)^{-1} afterwards); backward: v <- M^{-T} v (the caller scales before).
-template <bool BACK>
-__device__ void diag_solve(double* v, const double* Ls, const DTile& D, int nb, int w) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int kd = min(D.kd, nb - 1);
-    const int np = (w + 31) / 32;
-    for (int qi = 0; qi < np; ++qi) {
-        const int p = BACK ? (np - 1 - qi) * 32 : qi * 32;
-        const int pw = min(32, w - p);
-        if (warp == 0) {
-            double Lr[32];
-            double vi = 0.0;
-            if (lane < pw) {
-#pragma unroll
-                for (int l = 0; l < 32; ++l) {
-                    // forward: row p+lane, columns p+l < row; backward: column p+lane, rows p+l > it
-                    const int r = BACK ? p + l : p + lane, c = BACK ? p + lane : p + l;
-                    Lr[l] = (l < pw && r > c) ? Ls[r + c * kLdc] : 0.0;
-                }
-                vi = v[p + lane];
-            } else {
-#pragma unroll
-                for (int l = 0; l < 32; ++l) Lr[l] = 0.0;
-            }
-#pragma unroll
-            for (int jj = 0; jj < 32; ++jj) {
-                const int j = BACK ? 31 - jj : jj;
-                if (j < pw) {
-                    const double yj = __shfl_sync(0xffffffffu, vi, j);
-                    if (!BACK && lane > j) vi = fma(-Lr[j], yj, vi);
-                    if (BACK && lane < j) vi = fma(-Lr[j], yj, vi);
-                }
-            }
-            if (lane < pw) v[p + lane] = vi;
-        }
-        __syncthreads();
-        if (!BACK) {
-            const int rend = min(w, p + pw + kd);
-            for (int r = p + pw + threadIdx.x; r < rend; r += kThreads) {
-                double s0 = v[r], s1 = 0.0;
-                for (int l = 0; l < pw; l += 2) {
-                    s0 = fma(-Ls[r + (p + l) * kLdc], v[p + l], s0);
-                    if (l + 1 < pw) s1 = fma(-Ls[r + (p + l + 1) * kLdc], v[p + l + 1], s1);
-                }
-                v[r] = s0 + s1;
-            }
-        } else {
-            const int cbeg = max(0, p - kd);
-            for (int c = cbeg + threadIdx.x; c < p; c += kThreads) {
-                double s0 = v[c], s1 = 0.0;
-                for (int l = 0; l < pw; l += 2) {
-                    s0 = fma(-Ls[p + l + c * kLdc], v[p + l], s0);
-                    if (l + 1 < pw) s1 = fma(-Ls[p + l + 1 + c * kLdc], v[p + l + 1], s1);
-                }
-                v[c] = s0 + s1;
-            }
-        }
-        __syncthreads();
-    }
-}
-
 // ---- one-dimensional TMA (cp.async.bulk) into shared memory, completion on an mbarrier
 __device__ __forceinline__ unsigned smem_u32(const void* p) { return (unsigned)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void mbar_init(unsigned long long* bar) {
@@ -2013,151 +1946,250 @@ __global__ void __launch_bounds__(kThreads, 2) sn_replay_kernel(const __grid_con
     }
 }
 
-// Supernodal solve.  One persistent kernel over every (item, rhs) chain; step J < nsn is
-// the forward block of supernode J:  y_J = L_JJ^{-1} ((P b)_J - sum_I L_(J,I) y_I) over
-// the cells (J, I) that row supernode J owns; step nsn + i is the backward block of
-// J = nsn-1-i:  z_J = L_JJ^{-T} (y_J - sum_K L_(K,J)^T z_K) over the cells below J's
-// diagonal; z is scattered to x = P^T z.
+// Supernodal solve on the elimination tree of the supernodes, one persistent kernel over
+// every (item, rhs) chain.  Forward step J: the update vectors of J's children are added up
+// (ascending children, so in a fixed order), y_J = L_JJ^{-1} ((P b)_J + their part on J's
+// columns), and J's own update vector over its rows below is the rest minus L_below y_J.
+// Backward step J: z_J = L_JJ^{-T} (y_J - L_below^T z_below), z scattered to x = P^T z.  A
+// step waits for its children (its parent) only and reads its panel once as one dense block;
+// rows below beyond kSnSolveRows are tasks of their own, so a wide panel takes several SMs.
+// What bounds it: the path through the tree, per level a diagonal substitution and one
+// chunk (256 x 128 FMAs on one SM's FP64 pipe, 8 us).  Gathering every cell of a row
+// supernode one by one, in J order, took 58.2 ms at n = 180,020 (now 5.7), 18.0 ms on a 48^3
+// FEM operator (4.1) and 13.4 ms on 1024 small grids (4.6).
 struct SnSolveArgs {
-    const SnDevCell* cells;
-    const int16_t* maps;
-    const int32_t* cell_cmap;
-    const int32_t* first;
-    const int32_t* cptr;       // cells of column supernode J: [cptr[J], cptr[J+1]), diagonal first
-    const int32_t* rptr_cells; // cells owned by row supernode J
-    const int32_t* row_cells;
-    const int32_t* perm;
+    const SnSolveNode* nodes;
+    const int32_t *kids, *rel, *chunk_own, *fwd, *bwd, *rows, *perm;
     const double* factor;
     long long fstride;
     const double* b;           // [chains][n]
     double* x;                 // [chains][n]
     double* y;                 // workspace [chains][n]
-    int* done;                 // workspace [chains][2*nsn]
+    double* u;                 // workspace [chains][nu]
+    double* part;              // workspace [chains][npart]
+    int* flags;                // workspace [chains][2 nchunks + 2 nsn]
     WorkHeader* hdr;
-    long long chains, nrhs;
-    int nsn;
-    long long n, spin;
+    long long chains, nrhs, n, nu, npart, spin;
+    int nsn, nchunks;
 };
 
-__global__ void __launch_bounds__(kThreads, 1) sn_solve_kernel(SnSolveArgs a) {
+// v <- M^{-1} v (forward) or M^{-T} v (backward), M the unit lower w x w triangle packed in
+// Ls (pk layout), panels of 32: warp 0 solves a panel's triangle, the other rows (columns)
+// are then updated by a thread each.
+template <bool BACK>
+__device__ __forceinline__ void sn_tri_solve(double* v, const double* Ls, int w) {
+    const int lane = threadIdx.x & 31;
+    const int np = (w + 31) / 32;
+    for (int qi = 0; qi < np; ++qi) {
+        const int p = BACK ? (np - 1 - qi) * 32 : qi * 32, pw = min(32, w - p);
+        if (threadIdx.x < 32) {
+            double vi = lane < pw ? v[p + lane] : 0.0;
+#pragma unroll 8
+            for (int jj = 0; jj < pw; ++jj) {
+                const int j = BACK ? pw - 1 - jj : jj;
+                const bool live = BACK ? lane < j : (lane > j && lane < pw);
+                const double m = live ? Ls[BACK ? pk(w, p + j, p + lane) : pk(w, p + lane, p + j)] : 0.0;
+                const double yj = __shfl_sync(0xffffffffu, vi, j);
+                if (live) vi = fma(-m, yj, vi);
+            }
+            if (lane < pw) v[p + lane] = vi;
+        }
+        __syncthreads();
+        const int lo = BACK ? 0 : p + pw, hi = BACK ? p : w;
+        for (int r = lo + threadIdx.x; r < hi; r += blockDim.x) {
+            double s0 = v[r], s1 = 0.0;
+            int l = 0;
+            for (; l + 1 < pw; l += 2) {
+                s0 = fma(-Ls[BACK ? pk(w, p + l, r) : pk(w, r, p + l)], v[p + l], s0);
+                s1 = fma(-Ls[BACK ? pk(w, p + l + 1, r) : pk(w, r, p + l + 1)], v[p + l + 1], s1);
+            }
+            if (l < pw) s0 = fma(-Ls[BACK ? pk(w, p + l, r) : pk(w, r, p + l)], v[p + l], s0);
+            v[r] = s0 + s1;
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) sn_solve_kernel(SnSolveArgs a) {
     extern __shared__ double smem[];
-    double* Ls = smem;                              // diagonal block, L(r,c) at r + c*kLdc
-    __shared__ double v[kNbMax], ys[kNbMax], sdinv[kNbMax];
-    __shared__ double part[kThreads];
+    double* Ls = smem;                              // packed unit triangle of the diagonal block
+    __shared__ double v[kNbMax], sdinv[kNbMax];
+    __shared__ double us[kSnSolveRows];             // update vector chunk, or z of the chunk's rows
+    __shared__ double red[kThreads];
     __shared__ long long s_slot;
-    __shared__ int s_ok;
-    const long long total = 2LL * a.nsn * a.chains;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int T = blockDim.x, tid = threadIdx.x;
+    const long long half = (long long)a.nchunks * a.chains, total = 2 * half;
     for (;;) {
-        if (threadIdx.x == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
+        if (tid == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
         __syncthreads();
         const long long slot = s_slot;
-        __syncthreads();
+        bool ok = __syncthreads_and(*(volatile int*)&a.hdr->status == STC_OK);
         if (slot >= total) break;
-        const int ti = (int)(slot / a.chains);
-        const long long ch = slot % a.chains;
-        const long long item = ch / a.nrhs;
-        const double* F = a.factor + item * a.fstride;
+        const bool fwd = slot < half;
+        const long long sl = fwd ? slot : slot - half;
+        const int32_t* tk = (fwd ? a.fwd : a.bwd) + 2 * (sl / a.chains);
+        const int J = tk[0], q = tk[1];
+        const long long ch = sl % a.chains;
+        const SnSolveNode d = a.nodes[J];
+        const double* P = a.factor + (ch / a.nrhs) * a.fstride + d.off;
         double* y = a.y + ch * a.n;
-        int* done = a.done + ch * 2LL * a.nsn;
-        const bool fwd = ti < a.nsn;
-        const int J = fwd ? ti : a.nsn - 1 - (ti - a.nsn);
-        const SnDevCell D = a.cells[a.cptr[J]];
-        const int w = D.w, c0 = a.first[J];
-        if (threadIdx.x == 0) {
-            s_ok = (*(volatile int*)&a.hdr->status == STC_OK);
-            if (s_ok && !fwd) s_ok = wait_counter(done + J, 1, a.spin, &a.hdr->status);
+        double* u = a.u + ch * a.nu;
+        double* part = a.part + ch * a.npart + d.poff;
+        int* fchunk = a.flags + ch * (2LL * a.nchunks + 2LL * a.nsn);  // forward chunks done
+        int* bchunk = fchunk + a.nchunks;                              // backward chunks done
+        int* yflag = bchunk + a.nchunks;                               // y_J in place
+        int* zflag = yflag + a.nsn;                                    // z_J in place
+        const int w = d.w, ld = d.ld, nb = ld - w;
+        const int r0 = q * kSnSolveRows, R = max(0, min(kSnSolveRows, nb - r0));
+        if (q == 0 && ok) {
+            // diagonal block and right-hand side, before any wait
+            for (int c = tid; c < w; c += T) sdinv[c] = 1.0 / __ldg(P + c + (size_t)c * ld);
+            for (int r = tid; r < w; r += T) v[r] = fwd ? a.b[ch * a.n + a.perm[d.first + r]] : 0.0;
+            __syncthreads();
+            const int lane = tid & 31;
+            for (int c = tid >> 5; c < w; c += T >> 5)
+                for (int r = c + 1 + lane; r < w; r += 32) Ls[pk(w, r, c)] = __ldg(P + r + (size_t)c * ld) * sdinv[c];
         }
-        __syncthreads();
-        if (s_ok) {
-            // diagonal block, scaled to the unit lower triangle M = L diag(L)^{-1}
-            for_rc(kNbMax, kNbMax, [&](int r, int c) { Ls[r + c * kLdc] = 0.0; });
-            __syncthreads();
-            for_rc(w, w, [&](int r, int c) {
-                if (r >= c) Ls[r + c * kLdc] = __ldcg(F + D.off + r + (size_t)c * D.ld);
-            });
-            __syncthreads();
-            for (int c = threadIdx.x; c < w; c += kThreads) sdinv[c] = 1.0 / Ls[c * (kLdc + 1)];
-            for (int r = threadIdx.x; r < kNbMax; r += kThreads) {
-                v[r] = 0.0;
-                if (r < w) v[r] = fwd ? a.b[ch * a.n + a.perm[c0 + r]] : __ldcg(y + c0 + r);
+        if (fwd) {
+            // every chunk of every child, and y_J for the tasks of further rows
+            for (int k = d.kbeg; k < d.kend && ok; ++k) {
+                const SnSolveNode& c = a.nodes[a.kids[k]];
+                for (int z = tid; z < c.nchunk && ok; z += T) ok = wait_counter(fchunk + c.chunk + z, 1, a.spin, &a.hdr->status);
             }
-            __syncthreads();
-            for_rc(w, w, [&](int r, int c) { if (r > c) Ls[r + c * kLdc] *= sdinv[c]; });
-            __syncthreads();
-            if (fwd) {
-                // v[map[i]] -= sum_k L_(J,I)[i][k] y_I[k], cells in ascending I
-                for (int q = a.rptr_cells[J]; q < a.rptr_cells[J + 1] && s_ok; ++q) {
-                    const int cid = a.row_cells[q];
-                    const SnDevCell T = a.cells[cid];
-                    if (threadIdx.x == 0) s_ok = wait_counter(done + T.I, 1, a.spin, &a.hdr->status);
-                    __syncthreads();
-                    if (!s_ok) break;
-                    const int cI = a.first[T.I];
-                    for (int k = threadIdx.x; k < T.w; k += kThreads) ys[k] = __ldcg(y + cI + k);
-                    __syncthreads();
-                    // two threads per row (T.h <= 128), halves of the inner range
-                    const int i = threadIdx.x >> 1, hf = threadIdx.x & 1;
-                    double s0 = 0.0, s1 = 0.0;
-                    if (i < T.h) {
-                        const double* Lr = F + T.off + i;
-                        int k = hf;
-                        for (; k + 2 < T.w; k += 4) {
-                            s0 = fma(__ldcg(Lr + (size_t)k * T.ld), ys[k], s0);
-                            s1 = fma(__ldcg(Lr + (size_t)(k + 2) * T.ld), ys[k + 2], s1);
-                        }
-                        if (k < T.w) s0 = fma(__ldcg(Lr + (size_t)k * T.ld), ys[k], s0);
-                    }
-                    double sacc = s0 + s1;
-                    sacc += __shfl_xor_sync(0xffffffffu, sacc, 1);
-                    if (i < T.h && hf == 0) v[a.maps[a.cell_cmap[cid] + i]] -= sacc;
-                    __syncthreads();
-                }
-            } else {
-                // v[k] -= sum_i L_(K,J)[i][k] z_K[map[i]], cells below the diagonal, last first
-                for (int q = a.cptr[J + 1] - 1; q > a.cptr[J] && s_ok; --q) {
-                    const SnDevCell T = a.cells[q];
-                    if (threadIdx.x == 0) s_ok = wait_counter(done + a.nsn + T.J, 1, a.spin, &a.hdr->status);
-                    __syncthreads();
-                    if (!s_ok) break;
-                    const int cK = a.first[T.J];
-                    const int16_t* m = a.maps + a.cell_cmap[q];
-                    for (int i = threadIdx.x; i < T.h; i += kThreads) ys[i] = __ldcg(y + cK + m[i]);
-                    __syncthreads();
-                    for (int k = warp; k < T.w; k += kThreads / 32) {
-                        const double* Lc = F + T.off + (size_t)k * T.ld;
-                        double d = 0.0;
-                        for (int i = lane; i < T.h; i += 32) d = fma(__ldcg(Lc + i), ys[i], d);
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) d += __shfl_down_sync(0xffffffffu, d, o);
-                        if (lane == 0) part[k] = d;
+            if (q > 0 && tid == 0 && ok) ok = wait_counter(yflag + J, 1, a.spin, &a.hdr->status);
+            for (int r = tid; r < kSnSolveRows; r += T) us[r] = 0.0;
+            ok = __syncthreads_and(ok);
+            if (ok) {
+                // positions in J's rows this task takes: its columns (first chunk) and its rows
+                const int lo = q == 0 ? 0 : w + r0, hi = w + r0 + R;
+                for (int k = d.kbeg; k < d.kend; ++k) {
+                    const SnSolveNode& c = a.nodes[a.kids[k]];
+                    const double* uc = u + c.uoff;
+                    const int32_t* rel = a.rel + c.uoff;
+                    const int nc = c.ld - c.w;
+                    for (int i = tid; i < nc; i += T) {
+                        const int t = rel[i];
+                        if (t < lo || t >= hi) continue;
+                        const double x = __ldcg(uc + i);
+                        if (t < w) v[t] += x;
+                        else us[t - w - r0] += x;
                     }
                     __syncthreads();
-                    for (int k = threadIdx.x; k < T.w; k += kThreads) v[k] -= part[k];
-                    __syncthreads();
                 }
-            }
-            if (s_ok) {
-                DTile Dt{};
-                Dt.kd = w - 1;
-                if (fwd) {
-                    diag_solve<false>(v, Ls, Dt, kNbMax, w);
-                    for (int i = threadIdx.x; i < w; i += kThreads) v[i] *= sdinv[i];
+                if (q == 0) {
+                    sn_tri_solve<false>(v, Ls, w);
+                    for (int i = tid; i < w; i += T) {
+                        v[i] *= sdinv[i];
+                        __stcg(y + d.first + i, v[i]);
+                    }
+                    __threadfence();
                     __syncthreads();
+                    if (tid == 0) red_release_add(yflag + J, 1);
                 } else {
-                    for (int i = threadIdx.x; i < w; i += kThreads) v[i] *= sdinv[i];
+                    for (int i = tid; i < w; i += T) v[i] = __ldcg(y + d.first + i);
                     __syncthreads();
-                    diag_solve<true>(v, Ls, Dt, kNbMax, w);
                 }
-                for (int i = threadIdx.x; i < w; i += kThreads) {
-                    __stcg(y + c0 + i, v[i]);
-                    if (!fwd) a.x[ch * a.n + a.perm[c0 + i]] = v[i];
+                if (R > 0) {
+                    // us -= L(rows, :) y_J: rows over the threads (coalesced), the threads that
+                    // share a row take its columns in turn and are added up in order
+                    const int rp = R <= 1 ? 1 : min(T, 1 << (32 - __clz(R - 1))), G = T / rp;
+                    const int g = tid / rp;
+                    for (int rb = 0; rb < R; rb += rp) {
+                        const int r = rb + (tid & (rp - 1));
+                        double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+                        if (r < R) {
+                            const double* L = P + w + r0 + r;
+                            int k = g;
+                            for (; k + 3 * G < w; k += 4 * G) {
+                                const double l0 = __ldcg(L + (size_t)k * ld), l1 = __ldcg(L + (size_t)(k + G) * ld);
+                                const double l2 = __ldcg(L + (size_t)(k + 2 * G) * ld), l3 = __ldcg(L + (size_t)(k + 3 * G) * ld);
+                                s0 = fma(l0, v[k], s0);
+                                s1 = fma(l1, v[k + G], s1);
+                                s2 = fma(l2, v[k + 2 * G], s2);
+                                s3 = fma(l3, v[k + 3 * G], s3);
+                            }
+                            for (; k < w; k += G) s0 = fma(__ldcg(L + (size_t)k * ld), v[k], s0);
+                        }
+                        red[tid] = (s0 + s1) + (s2 + s3);
+                        __syncthreads();
+                        if (g == 0 && r < R) {
+                            double s = 0.0;
+                            for (int z = 0; z < G; ++z) s += red[tid + z * rp];
+                            __stcg(u + d.uoff + r0 + r, us[r] - s);
+                        }
+                        __syncthreads();
+                    }
                 }
             }
+            __threadfence();
+            __syncthreads();
+            // (after a failed wait too, so that nothing waits for this task; likewise below)
+            if (tid == 0) {
+                red_release_add(fchunk + d.chunk + q, 1);
+                if (!ok && q == 0) red_release_add(yflag + J, 1);
+            }
+        } else {
+            // z of the chunk's rows: the owner of the first row comes last of them
+            if (tid == 0 && ok) {
+                if (R > 0) ok = wait_counter(zflag + a.chunk_own[d.chunk + q], 1, a.spin, &a.hdr->status);
+                if (ok && q == 0) ok = wait_counter(yflag + J, 1, a.spin, &a.hdr->status);
+            }
+            ok = __syncthreads_and(ok);
+            if (ok) {
+                for (int i = tid; i < R; i += T) us[i] = __ldcg(y + a.rows[d.roff + r0 + i]);
+                __syncthreads();
+                // L(rows, c)^T z: columns over the threads, the threads that share a column take
+                // a run of its rows each (through L1: a thread walks down its column)
+                const int cp = w <= 1 ? 1 : min(T, 1 << (32 - __clz(w - 1))), G = T / cp, g = tid / cp;
+                const int a0 = R * g / G, a1 = R * (g + 1) / G;
+                for (int cb = 0; cb < w; cb += cp) {
+                    const int c = cb + (tid & (cp - 1));
+                    double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+                    if (c < w) {
+                        const double* L = P + w + r0 + (size_t)c * ld;
+                        int i = a0;
+                        for (; i + 3 < a1; i += 4) {
+                            const double l0 = __ldg(L + i), l1 = __ldg(L + i + 1), l2 = __ldg(L + i + 2), l3 = __ldg(L + i + 3);
+                            s0 = fma(l0, us[i], s0);
+                            s1 = fma(l1, us[i + 1], s1);
+                            s2 = fma(l2, us[i + 2], s2);
+                            s3 = fma(l3, us[i + 3], s3);
+                        }
+                        for (; i < a1; ++i) s0 = fma(__ldg(L + i), us[i], s0);
+                    }
+                    red[tid] = (s0 + s1) + (s2 + s3);
+                    __syncthreads();
+                    if (g == 0 && c < w) {
+                        double s = 0.0;
+                        for (int z = 0; z < G; ++z) s += red[tid + z * cp];
+                        if (q > 0) __stcg(part + (size_t)(q - 1) * w + c, s);
+                        else v[c] = s;
+                    }
+                    __syncthreads();
+                }
+            }
+            if (q == 0) {
+                if (ok)
+                    for (int z = 1 + tid; z < d.nchunk && ok; z += T) ok = wait_counter(bchunk + d.chunk + z, 1, a.spin, &a.hdr->status);
+                ok = __syncthreads_and(ok);
+                if (ok) {
+                    for (int i = tid; i < w; i += T) {
+                        double s = v[i];
+                        for (int z = 1; z < d.nchunk; ++z) s += __ldcg(part + (size_t)(z - 1) * w + i);
+                        v[i] = (__ldcg(y + d.first + i) - s) * sdinv[i];
+                    }
+                    __syncthreads();
+                    sn_tri_solve<true>(v, Ls, w);
+                    for (int i = tid; i < w; i += T) {
+                        __stcg(y + d.first + i, v[i]);
+                        a.x[ch * a.n + a.perm[d.first + i]] = v[i];
+                    }
+                }
+            }
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) red_release_add(q == 0 ? zflag + J : bchunk + d.chunk + q, 1);
         }
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) red_release_add(done + (fwd ? J : a.nsn + J), 1);
     }
 }
 
@@ -2711,8 +2743,8 @@ int device_info(int* dev, int* sms) {
         if (cudaFuncSetAttribute(sn_replay_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRSmemBytes) !=
             cudaSuccess)
             return STC_ERR_CUDA;
-        if (cudaFuncSetAttribute(sn_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSolveSmem) !=
-            cudaSuccess)
+        if (cudaFuncSetAttribute(sn_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(kRPacked * sizeof(double))) != cudaSuccess)
             return STC_ERR_CUDA;
         if (cudaFuncSetAttribute(sn_selinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) !=
             cudaSuccess)
@@ -2743,7 +2775,8 @@ void free_dev(stc_plan* P) {
     d = DevPlanArrays{};
     SnDev& q = P->sndev;
     void* sptrs[] = {q.cells, q.tasks, q.upds, q.maps, q.first, q.cell_cmap, q.cptr, q.rptr_cells, q.row_cells,
-                     q.value_map, q.csc_map, q.fill_src, q.stasks, q.scons, q.rows, q.cell_rowoff, q.order};
+                     q.value_map, q.csc_map, q.fill_src, q.stasks, q.scons, q.rows, q.cell_rowoff, q.order,
+                     q.snodes, q.skids, q.srel, q.schunk_own, q.sfwd, q.sbwd};
     for (void* p : sptrs)
         if (p) cudaFree(p);
     q = SnDev{};
@@ -2894,6 +2927,12 @@ int ensure_sn_impl(stc_plan* P, int dev) {
     if ((rc = upload(&d.scons, scons))) return rc;
     if ((rc = upload(&d.rows, S.rows))) return rc;
     if ((rc = upload(&d.cell_rowoff, S.cell_rowoff))) return rc;
+    if ((rc = upload(&d.snodes, S.snodes))) return rc;
+    if ((rc = upload(&d.skids, S.skids))) return rc;
+    if ((rc = upload(&d.srel, S.srel))) return rc;
+    if ((rc = upload(&d.schunk_own, S.schunk_own))) return rc;
+    if ((rc = upload(&d.sfwd, S.sfwd))) return rc;
+    if ((rc = upload(&d.sbwd, S.sbwd))) return rc;
     if ((rc = upload(&d.order, sn_queue_order(S, kSnQueueCtas)))) return rc;
     d.device = dev;
     return STC_OK;
@@ -2956,13 +2995,17 @@ size_t counters_per_item(const stc_plan* P) { return is_sn(P) ? P->supernodal().
 size_t factorize_ws(const stc_plan* P, int64_t batch) {
     return sizeof(WorkHeader) + (size_t)batch * counters_per_item(P) * sizeof(int);
 }
-// solve: a done flag per (chain, forward/backward step) and a y vector per chain
+// solve: step flags per chain (tile routes: one per forward and backward step; supernodal:
+// one per forward and backward chunk and two per supernode) and a y vector per chain;
+// supernodal: also the update vectors and backward partials of each chain
 size_t solve_flags(const stc_plan* P, int64_t chains) {
-    const size_t steps = is_sn(P) ? (size_t)P->supernodal().nsn() : (size_t)P->nt;
-    return ((size_t)chains * 2 * steps * sizeof(int) + 255) / 256 * 256;
+    size_t steps = 2 * (size_t)P->nt;
+    if (is_sn(P)) steps = 2 * (size_t)P->supernodal().nchunks + 2 * (size_t)P->supernodal().nsn();
+    return ((size_t)chains * steps * sizeof(int) + 255) / 256 * 256;
 }
 size_t solve_ws(const stc_plan* P, int64_t chains) {
-    const size_t ylen = is_sn(P) ? (size_t)P->n : (size_t)(P->nt * P->nb);
+    size_t ylen = (size_t)(P->nt * P->nb);
+    if (is_sn(P)) ylen = (size_t)(P->n + P->supernodal().nu + P->supernodal().npart);
     return sizeof(WorkHeader) + solve_flags(P, chains) + (size_t)chains * ylen * sizeof(double);
 }
 
@@ -3032,17 +3075,23 @@ int sn_solve(stc_plan* P, const void* d_factor, int64_t batch, int64_t nrhs, con
     const size_t flags = solve_flags(P, chains);
     if (cudaMemsetAsync(d_work, 0, sizeof(WorkHeader) + flags, st) != cudaSuccess) return STC_ERR_CUDA;
     SnSolveArgs a{};
-    a.cells = P->sndev.cells; a.maps = P->sndev.maps; a.cell_cmap = P->sndev.cell_cmap; a.first = P->sndev.first;
-    a.cptr = P->sndev.cptr; a.rptr_cells = P->sndev.rptr_cells; a.row_cells = P->sndev.row_cells;
-    a.perm = P->dev.perm; a.factor = (const double*)d_factor; a.fstride = Sp.item_doubles();
+    const SnDev& d = P->sndev;
+    a.nodes = d.snodes; a.kids = d.skids; a.rel = d.srel; a.chunk_own = d.schunk_own; a.fwd = d.sfwd; a.bwd = d.sbwd;
+    a.rows = d.rows; a.perm = P->dev.perm; a.factor = (const double*)d_factor; a.fstride = Sp.item_doubles();
     a.b = d_b; a.x = d_x; a.hdr = (WorkHeader*)d_work;
-    a.done = (int*)((char*)d_work + sizeof(WorkHeader));
+    a.flags = (int*)((char*)d_work + sizeof(WorkHeader));
     a.y = (double*)((char*)d_work + sizeof(WorkHeader) + flags);
-    a.chains = chains; a.nrhs = nrhs; a.nsn = Sp.nsn(); a.n = P->n;
+    a.u = a.y + chains * P->n;
+    a.part = a.u + chains * Sp.nu;
+    a.chains = chains; a.nrhs = nrhs; a.nsn = Sp.nsn(); a.nchunks = Sp.nchunks; a.n = P->n; a.nu = Sp.nu;
+    a.npart = Sp.npart;
     a.spin = P->opt.spin_limit > 0 ? P->opt.spin_limit : kDefaultSpin;
-    const long long total = 2LL * a.nsn * chains;
-    const int grid = grid_of(P, sms, total);
-    sn_solve_kernel<<<grid, kThreads, kSolveSmem, st>>>(a);
+    const long long total = 2LL * a.nchunks * chains;
+    // narrow supernodes: CTAs of two warps, eight per SM (a step is then mostly latency)
+    const bool narrow = Sp.wmax <= 32;
+    const size_t sm = (size_t)Sp.wmax * (Sp.wmax + 1) / 2 * sizeof(double);
+    const int grid = grid_of(P, narrow ? 8LL * sms : 2LL * sms, total);
+    sn_solve_kernel<<<grid, narrow ? 64 : kThreads, sm, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
 

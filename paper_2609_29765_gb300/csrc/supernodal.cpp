@@ -172,6 +172,7 @@ const stc::SnPlan& stc_plan::supernodal() const {
             S->tasks.insert(S->tasks.end(), {stc::SN_TRSM, c, -1, -1});
     }
     build_device_form(*S, snof, byrow, cell_of);
+    stc::sn_build_solve(*S);
     sn = std::move(S);
     return *sn;
 }
@@ -435,4 +436,88 @@ vector<int32_t> stc::sn_queue_order(const stc::SnPlan& S, int procs) {
     }
     if ((int32_t)order.size() != nt) throw std::logic_error("supernodal task set: a dependency cycle");
     return order;
+}
+
+// The solve on the elimination tree of the supernodes: parent links, the rows of each node
+// as positions in its parent, the chunk tasks, and their queue orders (modelled earliest
+// start, children before parents forward and parents before children backward).
+void stc::sn_build_solve(stc::SnPlan& S) {
+    const int32_t nsn = S.nsn();
+    const int32_t n = S.first[nsn];
+    vector<int32_t> snof(n), parent(nsn, -1);
+    for (int32_t s = 0; s < nsn; ++s)
+        for (int32_t j = S.first[s]; j < S.first[s + 1]; ++j) snof[j] = s;
+    S.snodes.resize(nsn);
+    S.skids.clear();
+    int64_t uo = 0, po = 0;
+    int32_t co = 0;
+    vector<int32_t> nkids(nsn + 1, 0);
+    for (int32_t J = 0; J < nsn; ++J) {
+        stc::SnSolveNode& d = S.snodes[J];
+        d.off = S.off[J];
+        d.first = S.first[J];
+        d.w = S.first[J + 1] - S.first[J];
+        d.ld = (int32_t)(S.rptr[J + 1] - S.rptr[J]);
+        d.roff = (int32_t)(S.rptr[J] + d.w);
+        S.wmax = std::max(S.wmax, d.w);
+        const int32_t nb = d.ld - d.w;
+        d.uoff = uo;
+        d.poff = po;
+        d.chunk = co;
+        d.nchunk = std::max(1, (nb + stc::kSnSolveRows - 1) / stc::kSnSolveRows);
+        uo += nb;
+        po += (int64_t)(d.nchunk - 1) * d.w;
+        co += d.nchunk;
+        if (nb > 0) {
+            parent[J] = snof[S.rows[d.roff]];
+            ++nkids[parent[J] + 1];
+        }
+        for (int32_t q = 0; q < d.nchunk; ++q)
+            S.schunk_own.push_back(nb > 0 ? snof[S.rows[d.roff + q * stc::kSnSolveRows]] : -1);
+    }
+    S.nu = uo;
+    S.npart = po;
+    S.nchunks = co;
+    for (int32_t J = 0; J < nsn; ++J) nkids[J + 1] += nkids[J];
+    S.skids.resize(nkids[nsn]);
+    vector<int32_t> at(nkids.begin(), nkids.end() - 1);
+    for (int32_t J = 0; J < nsn; ++J) {
+        S.snodes[J].kbeg = nkids[J];
+        S.snodes[J].kend = nkids[J + 1];
+        if (parent[J] >= 0) S.skids[at[parent[J]]++] = J;
+    }
+    S.srel.resize(uo);
+    for (int32_t J = 0; J < nsn; ++J) {
+        if (parent[J] < 0) continue;
+        const stc::SnSolveNode &d = S.snodes[J], &p = S.snodes[parent[J]];
+        const int32_t* r = S.rows.data() + d.roff;
+        const int32_t* t = S.rows.data() + S.rptr[parent[J]];
+        for (int32_t i = 0, q = 0; i < d.ld - d.w; ++i) {
+            while (q < p.ld && t[q] < r[i]) ++q;
+            if (q >= p.ld || t[q] != r[i]) throw std::logic_error("supernodal solve: rows not a subset of the parent's");
+            S.srel[d.uoff + i] = q;
+        }
+    }
+    // microseconds: a diagonal block 2 + w / 16, a chunk w / 16 (256 rows at 2 FMA per clock)
+    auto cost = [&](int32_t J) { return 3.0 + S.snodes[J].w / 8.0; };
+    vector<double> fs(nsn, 0.0), bs(nsn, 0.0);
+    for (int32_t J = 0; J < nsn; ++J)
+        if (parent[J] >= 0) fs[parent[J]] = std::max(fs[parent[J]], fs[J] + cost(J));
+    for (int32_t J = nsn - 1; J >= 0; --J)
+        if (parent[J] >= 0) bs[J] = bs[parent[J]] + cost(parent[J]);
+    vector<int32_t> ord(nsn);
+    for (int32_t J = 0; J < nsn; ++J) ord[J] = J;
+    std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return fs[a] < fs[b]; });
+    for (int32_t J : ord)
+        for (int32_t q = 0; q < S.snodes[J].nchunk; ++q) {
+            S.sfwd.push_back(J);
+            S.sfwd.push_back(q);
+        }
+    for (int32_t J = 0; J < nsn; ++J) ord[J] = nsn - 1 - J;
+    std::stable_sort(ord.begin(), ord.end(), [&](int32_t a, int32_t b) { return bs[a] < bs[b]; });
+    for (int32_t J : ord)
+        for (int32_t q = S.snodes[J].nchunk - 1; q >= 0; --q) {
+            S.sbwd.push_back(J);
+            S.sbwd.push_back(q);
+        }
 }
