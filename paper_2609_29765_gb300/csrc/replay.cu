@@ -34,12 +34,7 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kNbMax = 128;
 constexpr int kLdc = kNbMax + 1;   // shared-memory leading dimension of the tile buffer
-constexpr int kKc = 32;            // inner-dimension chunk staged per step
 constexpr int kPb = kPanelW;       // panel width of the blocked TRSM
-constexpr int kStage = kKc * (kNbMax + 9);          // doubles per staging buffer (odd ld)
-constexpr int kCbuf = kLdc * kNbMax + 16;           // tile buffer (+ overrun pad)
-constexpr int kSmemDoubles = kCbuf + 2 * kStage + kNbMax;
-constexpr size_t kSmemBytes = kSmemDoubles * sizeof(double) + 64;
 constexpr long long kDefaultSpin = 40000000LL;
 
 // Replay-kernel geometry, sized for two resident CTAs per SM (so one CTA's dependency
@@ -487,18 +482,16 @@ __device__ void store_diag_cols(const double* P, double* T, const DTile& d, int 
     }
 }
 
-// Full lower triangle (and zero upper) of a diagonal tile into C.
-__device__ void load_diag(double* C, const double* T, const DTile& d, int nb) {
-    for_rc(nb, nb, [&](int r, int c) { C[r + c * kLdc] = r >= c ? diag_at(T, d, nb, r, c) : 0.0; });
-}
-__device__ void store_diag(const double* C, double* T, const DTile& d, int nb) {
+// The leading w x w packed lower triangle P into a diagonal tile's storage, zero elsewhere
+// (dense: the upper part and the padding; banded: the padding, entries inside the band only).
+__device__ void write_sigma_diag(const double* P, int w, double* T, const DTile& d, int nb) {
     if (d.kind == TILE_DIAG_DENSE) {
-        for_rc(nb, nb, [&](int r, int c) { __stcg(T + r + (size_t)c * nb, r >= c ? C[r + c * kLdc] : 0.0); });
+        for_rc(nb, nb, [&](int r, int c) { __stcg(T + r + (size_t)c * nb, (r >= c && r < w) ? P[pk(w, r, c)] : 0.0); });
     } else {
-        const int w = d.kd + 1;
-        for_rc(w, nb, [&](int q, int r) {  // storage (q, r): L[r][r - kd + q]
+        const int bw = d.kd + 1;
+        for_rc(bw, nb, [&](int q, int r) {  // storage (q, r): L[r][r - kd + q]
             const int c = r - d.kd + q;
-            if (c >= 0) __stcg(T + q + (size_t)r * w, C[r + c * kLdc]);
+            if (c >= 0) __stcg(T + q + (size_t)r * bw, r < w ? P[pk(w, r, c)] : 0.0);
         });
     }
 }
@@ -1817,7 +1810,7 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                     const double* ga = F + A.off + (size_t)k0 * A.ld;
                     if (sp_worth(A.h * A.h / 2, K) &&
                         sp_stage_a(S0, A.h, [&](int r, int k) { return __ldcg(ga + r + (size_t)k * A.ld); }, K)) {
-                        sp_product<true>(S0, A.h, S0, A.h,
+                        sp_product<true>(S0, 0, A.h, S0, 0, A.h,
                                          [&](int r, int c, double v) { C[pk(w, s_rm[r], s_rm[c])] -= v; });
                     } else {
                         sn_stage(S0, kRStLd, F, A, 0, A.h, k0, K);
@@ -1864,7 +1857,7 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                     if (sp_worth(Ra * B.h, K) &&
                         sp_stage_ab(S0, Ra, [&](int r, int k) { return __ldcg(ga + r + (size_t)k * A.ld); }, S1, B.h,
                                     [&](int r, int k) { return __ldcg(gb + r + (size_t)k * B.ld); }, K)) {
-                        sp_product<false>(S0, Ra, S1, B.h,
+                        sp_product<false>(S0, 0, Ra, S1, 0, B.h,
                                           [&](int r, int c, double v) { C[s_rm[r] + s_cm[c] * kRLd] -= v; });
                     } else {
                         sn_stage(S0, kRStLd, F, A, u.ar0, Ra, k0, K);
@@ -1903,7 +1896,7 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                             if (sp_worth(R * Cn, K) &&
                                 sp_stage_ab(S0, R, [&](int r, int k) { return X[r + k * kRLd]; }, S1, Cn,
                                             [&](int c, int k) { return __ldcg(gb + c + (size_t)k * D.ld); }, K)) {
-                                sp_product<false>(S0, R, S1, Cn, [&](int r, int c, double v) { Y[r + c * kRLd] -= v; });
+                                sp_product<false>(S0, 0, R, S1, 0, Cn, [&](int r, int c, double v) { Y[r + c * kRLd] -= v; });
                             } else {
                                 const int Cp = ((Cn + 3) & ~3) + 4;
                                 for_rc(Cp, K, [&](int c, int k) {
@@ -2240,40 +2233,170 @@ __device__ __forceinline__ double sym_at(const double* T, const DTile& d, int nb
     return r >= c ? diag_at(T, d, nb, r, c) : diag_at(T, d, nb, c, r);
 }
 
-// S[r + k*ld] = get(r, k) for r < R, zero for R <= r < Rp, k < K; consecutive threads on
-// consecutive r (RFAST) or consecutive k -- whichever is contiguous in the source -- with
-// four loads in flight per thread.
-template <bool RFAST, class Get>
-__device__ void stage_gather(double* S, int ld, int R, int Rp, int K, Get get) {
-    const int n = Rp * K;
-    for (int b = threadIdx.x; b < n; b += 4 * kThreads) {
-        double v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int j = b + u * kThreads;
-            const int r = RFAST ? j % Rp : j / K, k = RFAST ? j / Rp : j % K;
-            v[u] = (j < n && r < R) ? get(r, k) : 0.0;
+// C(r, c) at C[r + c ldc] -= sum_k ga(r, k) gb(c, k), r < R, c < Cn, k < K <= 16 (the whole
+// CTA; a barrier before and after): by the split where it can take the chunk, else one DFMA
+// sum per entry straight from the operands.  S0, S1: digit buffers.
+template <class GetA, class GetB, class Epi>
+__device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int Cn, int K, GetA ga, GetB gb, Epi epi) {
+    if (!sp_stage_ab(S0, R, ga, S1, Cn, gb, K))
+        for (int e = threadIdx.x; e < R * Cn; e += kThreads) {
+            const int r = e % R, c = e / R;
+            double v = 0.0;
+            for (int k = 0; k < K; ++k) v = fma(ga(r, k), gb(c, k), v);
+            epi(r, c, v);
         }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            const int j = b + u * kThreads;
-            const int r = RFAST ? j % Rp : j / K, k = RFAST ? j / Rp : j % K;
-            if (j < n) S[r + k * ld] = v[u];
+    else
+        sp_product<false>(S0, 0, R, S1, 0, Cn, epi);
+    __syncthreads();
+}
+
+// Diagonal block of a selected inverse.  P holds -Z (packed lower triangle of width w) and
+// becomes Sigma:
+//   Sigma_rc = (-Z_rc - sum_{i>c} Sigma_ri L_ic) / L_cc              (r > c)
+//   Sigma_cc = 1/L_cc^2 + (-Z_cc - sum_{i>c} L_ic Sigma_ic) / L_cc
+// by panels of 16 columns from the right: the rows below a panel take the products with the
+// columns already done (chunk products of the symmetric part) and a triangular solve, the
+// panel's own 16 x 16 block the products with those rows and the element recurrence on one
+// warp.  One column at a time over the whole block (two barriers and a dot product of up to
+// w terms per column) was most of a diagonal task; a whole selected inverse
+// of 64 value sets at n = 4,020 went 35.5 -> 21.4 ms with this and the split products, of 16
+// bands (n = 50,000, half-bandwidth 20) 115 -> 101 ms.  Rows more than kd below the diagonal are outside the
+// band and left alone.  lget(i, c): L_ic, i >= c.  S0: digits; S1: digits, then the panel's
+// rows; sv: kNbMax doubles.
+constexpr int kSelP = 16;
+template <class LGet>
+__device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, double* sv, LGet lget) {
+    constexpr int LDX = kNbMax + 1 - kSelP;   // panel rows below: at most kNbMax - kSelP
+    static_assert(LDX * kSelP + kSelP * (kSelP + 1) <= kRStage, "panel rows and its diagonal block fit a staging buffer");
+    double* X = S1;                           // X(r, c), row b + r of the panel's columns
+    double* D = S1 + LDX * kSelP;             // L of the panel's diagonal block, (i, j) at i + 17 j
+    for (int p = ((w - 1) / kSelP) * kSelP; p >= 0; p -= kSelP) {
+        const int pw = min(kSelP, w - p), b = p + pw, m = max(0, min(w, b + kd) - b);
+        // L of the panel: the diagonal block and its reciprocals
+        for (int e = threadIdx.x; e < kSelP * kSelP; e += kThreads) {
+            const int i = e % kSelP, j = e / kSelP;
+            D[i + j * (kSelP + 1)] = (i < pw && j <= i) ? lget(p + i, p + j) : 0.0;
         }
+        for (int e = threadIdx.x; e < m * pw; e += kThreads) {
+            const int r = e % m, c = e / m;
+            X[r + c * LDX] = P[pk(w, b + r, p + c)];
+        }
+        __syncthreads();
+        if (threadIdx.x < pw) sv[threadIdx.x] = 1.0 / D[threadIdx.x * (kSelP + 2)];
+        __syncthreads();
+        if (m > 0) {
+            // X -= Sigma(below, below) L(below, panel); both operands' digits share S0 (m + 16 rows)
+            for (int i0 = 0; i0 < m; i0 += kSpK) {
+                const int K = min(kSpK, m - i0);
+                auto ga = [&](int r, int k) {
+                    const int x = b + r, y = b + i0 + k;
+                    return abs(x - y) <= kd ? P[pk(w, max(x, y), min(x, y))] : 0.0;
+                };
+                auto gb = [&](int c, int k) { return lget(b + i0 + k, p + c); };
+                auto gab = [&](int r, int k) { return r < m ? ga(r, k) : gb(r - m, k); };
+                if (sp_stage_a(S0, m + pw, gab, K)) {
+                    sp_product<false>(S0, 0, m, S0, m, pw, [&](int r, int c, double v) { X[r + c * LDX] -= v; });
+                } else {
+                    for (int e = threadIdx.x; e < m * pw; e += kThreads) {
+                        const int r = e % m, c = e / m;
+                        double v = X[r + c * LDX];
+                        for (int k = 0; k < K; ++k) v = fma(-ga(r, k), gb(c, k), v);
+                        X[r + c * LDX] = v;
+                    }
+                }
+                __syncthreads();
+            }
+            trsm_rows_dir<true>(X, LDX, m, pw, D, kSelP + 1, sv);
+            __syncthreads();
+        }
+        // the panel's own block: the products with the rows below, an entry per thread
+        double* LB = S0;  // L(below, panel)
+        for (int e = threadIdx.x; e < m * pw; e += kThreads) {
+            const int r = e % m, c = e / m;
+            LB[r + c * LDX] = lget(b + r, p + c);
+        }
+        __syncthreads();
+        {
+            const int r = threadIdx.x & (kSelP - 1), c = threadIdx.x / kSelP;
+            if (r >= c && r < pw) {
+                double s0 = P[pk(w, p + r, p + c)], s1 = 0.0;
+                int i = 0;
+                for (; i + 1 < m; i += 2) {
+                    s0 = fma(-X[i + r * LDX], LB[i + c * LDX], s0);
+                    s1 = fma(-X[i + 1 + r * LDX], LB[i + 1 + c * LDX], s1);
+                }
+                if (i < m) s0 = fma(-X[i + r * LDX], LB[i + c * LDX], s0);
+                P[pk(w, p + r, p + c)] = s0 + s1;
+            }
+            for (int e = threadIdx.x; e < m * pw; e += kThreads) {
+                const int rr = e % m, cc = e / m;
+                P[pk(w, b + rr, p + cc)] = X[rr + cc * LDX];
+            }
+        }
+        __syncthreads();
+        if (threadIdx.x < 32) {
+            // two lanes per row (odd and even inner rows)
+            const int r = threadIdx.x >> 1, hf = threadIdx.x & 1;
+            for (int c = pw - 1; c >= 0; --c) {
+                double sg = 0.0, own = 0.0;
+                if (r > c && r < pw) {
+                    for (int i = c + 1 + hf; i < pw; i += 2)
+                        sg = fma(-D[i + c * (kSelP + 1)], P[pk(w, p + max(i, r), p + min(i, r))], sg);
+                }
+                sg += __shfl_xor_sync(0xffffffffu, sg, 1);
+                if (r > c && r < pw && hf == 0) {
+                    sg = (P[pk(w, p + r, p + c)] + sg) * sv[c];
+                    P[pk(w, p + r, p + c)] = sg;
+                    own = D[r + c * (kSelP + 1)] * sg;
+                }
+#pragma unroll
+                for (int o = 16; o > 1; o >>= 1) own += __shfl_xor_sync(0xffffffffu, own, o);
+                if (threadIdx.x == 0) {
+                    const double inv = sv[c];
+                    P[pk(w, p + c, p + c)] = inv * inv + (P[pk(w, p + c, p + c)] - own) * inv;
+                }
+                __syncwarp();
+            }
+        }
+        __syncthreads();
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 1) selinv_kernel(SelinvArgs a) {
+// Rows [rs0, rs0 + R) of an off-diagonal block of a selected inverse, held in C (leading
+// dimension kRLd, w columns): C <- C L^{-1}, panels of 32 columns from the right.
+template <class LGet>
+__device__ __forceinline__ void selinv_back(double* C, int R, int w, double* S0, double* S1, double* sv, LGet lget) {
+    for (int p = ((w - 1) / kPb) * kPb; p >= 0; p -= kPb) {
+        const int pw = min(kPb, w - p);
+        for (int k0 = p + pw; k0 < w; k0 += kSpK) {
+            const double* X = C + k0 * kRLd;
+            double* Y = C + p * kRLd;
+            chunk_product(S0, S1, R, pw, min(kSpK, w - k0), [&](int r, int k) { return X[r + k * kRLd]; },
+                          [&](int c, int k) { return lget(k0 + k, p + c); },
+                          [&](int r, int c, double v) { Y[r + c * kRLd] -= v; });
+        }
+        for (int idx = threadIdx.x; idx < kPb * kPb; idx += kThreads) {
+            const int i = idx & (kPb - 1), j = idx / kPb;
+            S0[i + j * (kPb + 1)] = (i < pw && j < pw && i >= j) ? lget(p + i, p + j) : 0.0;
+        }
+        __syncthreads();
+        if (threadIdx.x < pw) sv[threadIdx.x] = 1.0 / S0[threadIdx.x * (kPb + 2)];
+        __syncthreads();
+        trsm_rows_dir<true>(C + p * kRLd, kRLd, R, pw, S0, kPb + 1, sv);
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
     extern __shared__ double smem[];
-    double* C = smem;
-    double* S0 = C + kCbuf;
-    double* S1 = S0 + kStage;
-    double* sv = S1 + kStage;
+    double* C = smem;                 // <= 64 rows of an off-diagonal tile, or a packed diagonal tile
+    double* S0 = C + kRCbuf;
+    double* S1 = S0 + kRStage;
+    double* sv = S1 + kRStage;
     __shared__ long long s_slot;
     __shared__ int s_ok;
     const long long total = (long long)a.ntasks * a.batch;
     const int nb = a.nb;
-    constexpr int LDS = kNbMax + 9;  // odd: column-wise staging stores hit distinct banks
     __shared__ int16_t s_idx[2][kNbMax];  // stored-column indices of a contribution's tiles
     for (;;) {
         if (threadIdx.x == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
@@ -2289,97 +2412,69 @@ __global__ void __launch_bounds__(kThreads, 1) selinv_kernel(SelinvArgs a) {
         int* cnt = a.counters + item * a.ntiles;
         const DTile O = a.tiles[t.tile];
         const DTile D = a.tiles[t.diag];
+        const double* DT = Lf + D.off;
         if (threadIdx.x == 0) s_ok = (*(volatile int*)&a.hdr->status == STC_OK);
         __syncthreads();
         if (t.kind == TASK_SOFF && s_ok) {
-            const int R = t.r1 - t.r0, sw = O.sw;
-            for_rc(R, sw, [&](int r, int c) { C[r + c * kLdc] = 0.0; });
-            __syncthreads();
-            for (int ci = t.cbeg; ci < t.cend; ++ci) {
-                const DSCon cn = a.cons[ci];
-                const DTile Lt = a.tiles[cn.ltile];
-                const DTile St = a.tiles[cn.stile];
-                if (threadIdx.x == 0) s_ok = wait_counter(cnt + cn.stile, 1, a.spin, &a.hdr->status);
+            const int sw = O.sw;
+            for (int rs0 = t.r0; rs0 < t.r1 && s_ok; rs0 += kRRows) {  // <= 64 rows at a time
+                const int R = min(kRRows, t.r1 - rs0);
+                for_rc(R, sw, [&](int r, int c) { C[r + c * kRLd] = 0.0; });
                 __syncthreads();
-                if (!s_ok) break;
-                const double* LT = Lf + Lt.off;
-                const double* ST = Sg + St.off;
-                const int16_t* si_S = a.sinv + (size_t)cn.stile * nb;
-                const int16_t* si_L = a.sinv + (size_t)cn.ltile * nb;
-                // stored-column indices used by every chunk: Sigma's for the inner rows i
-                // (MJ) or the output rows (JM), L's for the output's stored columns
-                for (int q = threadIdx.x; q < nb; q += kThreads) {
-                    s_idx[0][q] = si_S[q];
-                    s_idx[1][q] = q < sw ? si_L[logical_col(O, a.saind, q)] : (int16_t)-1;
-                }
-                __syncthreads();
-                for (int i0 = Lt.r0; i0 < Lt.r1; i0 += kKc) {
-                    const int K = min(kKc, Lt.r1 - i0);
-                    const int Rp = ((R + 3) & ~3) + 4, Cp = ((sw + 3) & ~3) + 4;
-                    if (cn.mode == SCON_MJ) {  // Sigma(m, j): output rows contiguous
-                        stage_gather<true>(S0, LDS, R, Rp, K, [&](int r, int kk) {
-                            const int sidx = s_idx[0][i0 + kk];
-                            return sidx >= 0 ? __ldcg(ST + t.r0 + r + (size_t)sidx * nb) : 0.0;
-                        });
-                    } else if (cn.mode == SCON_JM) {  // Sigma(j, m)^T: inner rows contiguous
-                        stage_gather<false>(S0, LDS, R, Rp, K, [&](int r, int kk) {
-                            const int sidx = s_idx[0][t.r0 + r];
-                            return sidx >= 0 ? __ldcg(ST + i0 + kk + (size_t)sidx * nb) : 0.0;
-                        });
-                    } else {
-                        stage_gather<true>(S0, LDS, R, Rp, K,
-                                           [&](int r, int kk) { return sym_at(ST, St, nb, t.r0 + r, i0 + kk); });
+                for (int ci = t.cbeg; ci < t.cend; ++ci) {
+                    const DSCon cn = a.cons[ci];
+                    const DTile Lt = a.tiles[cn.ltile];
+                    const DTile St = a.tiles[cn.stile];
+                    if (threadIdx.x == 0) s_ok = wait_counter(cnt + cn.stile, 1, a.spin, &a.hdr->status);
+                    __syncthreads();
+                    if (!s_ok) break;
+                    const double* LT = Lf + Lt.off;
+                    const double* ST = Sg + St.off;
+                    const int16_t* si_S = a.sinv + (size_t)cn.stile * nb;
+                    const int16_t* si_L = a.sinv + (size_t)cn.ltile * nb;
+                    // stored-column indices used by every chunk: Sigma's for the inner rows i
+                    // (MJ) or the output rows (JM), L's for the output's stored columns
+                    for (int q = threadIdx.x; q < nb; q += kThreads) {
+                        s_idx[0][q] = si_S[q];
+                        s_idx[1][q] = q < sw ? si_L[logical_col(O, a.saind, q)] : (int16_t)-1;
                     }
-                    // L(j, k) rows i0.. of the output's stored columns: rows contiguous
-                    stage_gather<false>(S1, LDS, sw, Cp, K, [&](int c, int kk) {
-                        const int sl = s_idx[1][c];
-                        return sl >= 0 ? __ldcg(LT + (i0 + kk) + (size_t)sl * nb) : 0.0;
+                    __syncthreads();
+                    for (int i0 = Lt.r0; i0 < Lt.r1; i0 += kSpK) {
+                        const int K = min(kSpK, Lt.r1 - i0);
+                        // Sigma(m, j): output rows contiguous; Sigma(j, m)^T: inner rows contiguous
+                        auto ga = [&](int r, int k) {
+                            if (cn.mode == SCON_MJ) {
+                                const int q = s_idx[0][i0 + k];
+                                return q >= 0 ? __ldcg(ST + rs0 + r + (size_t)q * nb) : 0.0;
+                            }
+                            if (cn.mode == SCON_JM) {
+                                const int q = s_idx[0][rs0 + r];
+                                return q >= 0 ? __ldcg(ST + i0 + k + (size_t)q * nb) : 0.0;
+                            }
+                            return sym_at(ST, St, nb, rs0 + r, i0 + k);
+                        };
+                        // L(j, k) rows i0.. of the output's stored columns (through L1: a
+                        // thread walks down its column)
+                        auto gb = [&](int c, int k) {
+                            const int q = s_idx[1][c];
+                            return q >= 0 ? __ldg(LT + (i0 + k) + (size_t)q * nb) : 0.0;
+                        };
+                        chunk_product(S0, S1, R, sw, K, ga, gb, [&](int r, int c, double v) { C[r + c * kRLd] -= v; });
+                    }
+                }
+                if (s_ok) {
+                    // X L_g = C on the stored columns
+                    selinv_back(C, R, sw, S0, S1, sv, [&](int i, int j) {
+                        return diag_at(DT, D, nb, logical_col(O, a.saind, i), logical_col(O, a.saind, j));
                     });
-                    __syncthreads();
-                    mma_sub<false>(C, kLdc, R, sw, S0, LDS, S1, LDS, K);  // C = -sum Sigma L
-                    __syncthreads();
+                    double* T = Sg + O.off;
+                    for_rc(R, sw, [&](int r, int c) { __stcg(T + rs0 + r + (size_t)c * nb, C[r + c * kRLd]); });
                 }
-            }
-            if (s_ok) {
-                // X L_g = C on the stored columns, panels from the right (backward)
-                const double* DT = Lf + D.off;
-                for (int p = ((sw - 1) / kPb) * kPb; p >= 0; p -= kPb) {
-                    const int pw = min(kPb, sw - p);
-                    for (int k0 = p + pw; k0 < sw; k0 += kKc) {
-                        const int K = min(kKc, sw - k0);
-                        const int Cp = ((pw + 3) & ~3) + 4;
-                        for_rc(Cp, K, [&](int c, int kk) {
-                            double v = 0.0;
-                            if (c < pw)
-                                v = diag_at(DT, D, nb, logical_col(O, a.saind, k0 + kk), logical_col(O, a.saind, p + c));
-                            S1[c + kk * LDS] = v;
-                        });
-                        __syncthreads();
-                        mma_sub<false>(C + p * kLdc, kLdc, R, pw, C + k0 * kLdc, kLdc, S1, LDS, K);
-                        __syncthreads();
-                    }
-                    const bool band = D.kind == TILE_DIAG_BAND;
-                    for (int idx = threadIdx.x; idx < kPb * kPb; idx += kThreads) {
-                        const int i = band ? idx / kPb : idx & (kPb - 1);
-                        const int j = band ? idx & (kPb - 1) : idx / kPb;
-                        double v = 0.0;
-                        if (i < pw && j < pw && i >= j)
-                            v = diag_at(DT, D, nb, logical_col(O, a.saind, p + i), logical_col(O, a.saind, p + j));
-                        S0[i + j * (kPb + 1)] = v;
-                    }
-                    __syncthreads();
-                    if (threadIdx.x < pw) sv[threadIdx.x] = 1.0 / S0[threadIdx.x * (kPb + 2)];
-                    __syncthreads();
-                    trsm_rows_dir<true>(C + p * kLdc, kLdc, R, pw, S0, kPb + 1, sv);
-                    __syncthreads();
-                }
-                double* T = Sg + O.off;
-                for_rc(R, sw, [&](int r, int c) { __stcg(T + t.r0 + r + (size_t)c * nb, C[r + c * kLdc]); });
+                __syncthreads();
             }
         } else if (t.kind == TASK_SDIAG && s_ok) {
             const int w = O.sw;
-            const int kd = min(O.kd, nb - 1);
-            for_rc(nb, nb, [&](int r, int c) { C[r + c * kLdc] = 0.0; });
+            for (int e = threadIdx.x; e < w * (w + 1) / 2; e += kThreads) C[e] = 0.0;
             __syncthreads();
             for (int ci = t.cbeg; ci < t.cend; ++ci) {
                 const DSCon cn = a.cons[ci];
@@ -2391,59 +2486,40 @@ __global__ void __launch_bounds__(kThreads, 1) selinv_kernel(SelinvArgs a) {
                 const double* ST = Sg + Tt.off;
                 const bool contig = Tt.c0 >= 0;
                 const int M = contig ? Tt.sw : w;   // rows/cols of the Z block
+                const int z0 = contig ? Tt.c0 : 0;
                 const int16_t* si = a.sinv + (size_t)cn.ltile * nb;
                 for (int q = threadIdx.x; q < nb; q += kThreads) s_idx[0][q] = contig ? (int16_t)q : si[q];
                 __syncthreads();
-                for (int i0 = Tt.r0; i0 < Tt.r1; i0 += kKc) {
-                    const int K = min(kKc, Tt.r1 - i0);
-                    const int Mp = ((M + 3) & ~3) + 4;
-                    // rows i0.. of the stored columns: contiguous along the inner index
-                    stage_gather<false>(S0, LDS, M, Mp, K, [&](int r, int kk) {
-                        const int sidx = s_idx[0][r];
-                        return sidx >= 0 ? __ldcg(ST + (i0 + kk) + (size_t)sidx * nb) : 0.0;
-                    });
-                    stage_gather<false>(S1, LDS, M, Mp, K, [&](int r, int kk) {
-                        const int sidx = s_idx[0][r];
-                        return sidx >= 0 ? __ldcg(LT + (i0 + kk) + (size_t)sidx * nb) : 0.0;
-                    });
-                    __syncthreads();
-                    double* Cz = contig ? C + Tt.c0 * (1 + kLdc) : C;
-                    mma_sub<true>(Cz, kLdc, M, M, S0, LDS, S1, LDS, K);  // C = -Z (lower)
+                for (int i0 = Tt.r0; i0 < Tt.r1; i0 += kSpK) {
+                    const int K = min(kSpK, Tt.r1 - i0);
+                    auto ga = [&](int r, int k) {
+                        const int q = s_idx[0][r];
+                        return q >= 0 ? __ldcg(ST + (i0 + k) + (size_t)q * nb) : 0.0;
+                    };
+                    auto gb = [&](int r, int k) {
+                        const int q = s_idx[0][r];
+                        return q >= 0 ? __ldg(LT + (i0 + k) + (size_t)q * nb) : 0.0;
+                    };
+                    auto epi = [&](int r, int c, double v) { C[pk(w, z0 + r, z0 + c)] -= v; };
+                    if (sp_stage_ab(S0, M, ga, S1, M, gb, K)) {
+                        sp_product<true>(S0, 0, M, S1, 0, M, epi);
+                    } else {
+                        for (int e = threadIdx.x; e < M * M; e += kThreads) {
+                            const int r = e % M, c = e / M;
+                            if (r < c) continue;
+                            double v = 0.0;
+                            for (int k = 0; k < K; ++k) v = fma(ga(r, k), gb(c, k), v);
+                            epi(r, c, v);
+                        }
+                    }
                     __syncthreads();
                 }
             }
             if (s_ok) {
-                // packed lower triangle of L_kk in the staging area: (r, c) at c*nb - c(c-1)/2 + r - c
-                double* Lp = S0;
-                const double* DT = Lf + D.off;
-                read_diag_rows(DT, D, nb, 0, nb,
-                               [&](int r, int c, double v) { Lp[c * nb - c * (c - 1) / 2 + (r - c)] = v; });
-                __syncthreads();
-                for (int c = w - 1; c >= 0; --c) {
-                    const double* Lc = Lp + c * nb - c * (c - 1) / 2 - c;  // Lc[i] = L[i][c]
-                    const double inv = 1.0 / Lc[c];
-                    const int iend = min(w, c + kd + 1);
-                    for (int r = c + 1 + threadIdx.x; r < iend; r += kThreads) {
-                        double s0 = C[r + c * kLdc], s1 = 0.0;
-                        int i = c + 1;
-                        for (; i + 1 < iend; i += 2) {
-                            s0 = fma(-Lc[i], i >= r ? C[i + r * kLdc] : C[r + i * kLdc], s0);
-                            s1 = fma(-Lc[i + 1], i + 1 >= r ? C[i + 1 + r * kLdc] : C[r + (i + 1) * kLdc], s1);
-                        }
-                        if (i < iend) s0 = fma(-Lc[i], i >= r ? C[i + r * kLdc] : C[r + i * kLdc], s0);
-                        C[r + c * kLdc] = (s0 + s1) * inv;
-                    }
-                    __syncthreads();
-                    if (threadIdx.x < 32) {
-                        double sacc = 0.0;
-                        for (int i = c + 1 + threadIdx.x; i < iend; i += 32) sacc = fma(Lc[i], C[i + c * kLdc], sacc);
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) sacc += __shfl_down_sync(0xffffffffu, sacc, o);
-                        if (threadIdx.x == 0) C[c + c * kLdc] = inv * inv + (C[c + c * kLdc] - sacc) * inv;
-                    }
-                    __syncthreads();
-                }
-                store_diag(C, Sg + O.off, O, nb);
+                selinv_diag(C, w, min(O.kd, nb - 1), S0, S1, sv,
+                            [&](int i, int c) { return diag_at(DT, D, nb, i, c); });
+                // padding rows and columns of a ragged tile: zero
+                write_sigma_diag(C, w, Sg + O.off, O, nb);
             }
         }
         __threadfence();
@@ -2481,16 +2557,15 @@ struct SnSelinvArgs {
     long long spin;
 };
 
-__global__ void __launch_bounds__(kThreads, 1) sn_selinv_kernel(SnSelinvArgs a) {
+__global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) {
     extern __shared__ double smem[];
-    double* C = smem;
-    double* S0 = C + kCbuf;
-    double* S1 = S0 + kStage;
-    double* sv = S1 + kStage;
+    double* C = smem;                 // <= 64 rows of a cell, or a packed diagonal block
+    double* S0 = C + kRCbuf;
+    double* S1 = S0 + kRStage;
+    double* sv = S1 + kRStage;
     __shared__ long long s_slot;
     __shared__ int s_ok;
     __shared__ int ia[kNbMax], ja[kNbMax], srow[kNbMax];
-    constexpr int LDS = kNbMax + 9;
     const long long total = (long long)a.ntasks * a.batch;
     for (;;) {
         if (threadIdx.x == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
@@ -2508,12 +2583,13 @@ __global__ void __launch_bounds__(kThreads, 1) sn_selinv_kernel(SnSelinvArgs a) 
         const SnDevCell D = a.cells[t.diag];
         const int w = D.w;
         const double* DL = Lf + D.off;  // L_JJ(r, c) = DL[r + c * D.ld], r >= c
+        auto lget = [&](int i, int c) { return __ldg(DL + i + (size_t)c * D.ld); };
         if (threadIdx.x == 0) s_ok = (*(volatile int*)&a.hdr->status == STC_OK);
         __syncthreads();
         if (t.kind == SN_S_OFF && s_ok) {
             const int R = t.rs1 - t.rs0;
             const int K = O.J;
-            for_rc(R, w, [&](int r, int c) { C[r + c * kLdc] = 0.0; });
+            for_rc(R, w, [&](int r, int c) { C[r + c * kRLd] = 0.0; });
             __syncthreads();
             for (int ci = t.cbeg; ci < t.cend; ++ci) {
                 const SnSCon q = a.cons[ci];
@@ -2543,54 +2619,26 @@ __global__ void __launch_bounds__(kThreads, 1) sn_selinv_kernel(SnSelinvArgs a) 
                 __syncthreads();
                 const double* ST = Sg + Sc.off;
                 const double* LT = Lf + Lc.off;
-                for (int j0 = 0; j0 < h; j0 += kKc) {
-                    const int Kc = min(kKc, h - j0);
-                    const int Rp = ((R + 3) & ~3) + 4, Cp = ((w + 3) & ~3) + 4;
-                    stage_gather<true>(S0, LDS, R, Rp, Kc, [&](int r, int k) {
+                for (int j0 = 0; j0 < h; j0 += kSpK) {
+                    auto ga = [&](int r, int k) {
                         const int x = ia[r], y = ja[j0 + k];
-                        if (q.mode == SN_SC_SAME)
-                            return __ldcg(ST + max(x, y) + (size_t)min(x, y) * Sc.ld);
+                        if (q.mode == SN_SC_SAME) return __ldcg(ST + max(x, y) + (size_t)min(x, y) * Sc.ld);
                         if (q.mode == SN_SC_LOWER) return __ldcg(ST + x + (size_t)y * Sc.ld);
                         return __ldcg(ST + y + (size_t)x * Sc.ld);
-                    });
-                    // L(K',J) rows j0.. (contiguous along the inner index)
-                    stage_gather<false>(S1, LDS, w, Cp, Kc,
-                                        [&](int c, int k) { return __ldcg(LT + (j0 + k) + (size_t)c * Lc.ld); });
-                    __syncthreads();
-                    mma_sub<false>(C, kLdc, R, w, S0, LDS, S1, LDS, Kc);  // C = -sum G L
-                    __syncthreads();
+                    };
+                    // L(K',J) rows j0.. (through L1: a thread walks down its column)
+                    auto gb = [&](int c, int k) { return __ldg(LT + (j0 + k) + (size_t)c * Lc.ld); };
+                    chunk_product(S0, S1, R, w, min(kSpK, h - j0), ga, gb,
+                                  [&](int r, int c, double v) { C[r + c * kRLd] -= v; });  // C = -sum G L
                 }
             }
             if (s_ok) {
-                // X L_JJ = C, panels from the right (backward)
-                for (int p = ((w - 1) / kPb) * kPb; p >= 0; p -= kPb) {
-                    const int pw = min(kPb, w - p);
-                    for (int k0 = p + pw; k0 < w; k0 += kKc) {
-                        const int Kc = min(kKc, w - k0);
-                        const int Cp = ((pw + 3) & ~3) + 4;
-                        for_rc(Cp, Kc, [&](int c, int kk) {
-                            S1[c + kk * LDS] = c < pw ? __ldcg(DL + (k0 + kk) + (size_t)(p + c) * D.ld) : 0.0;
-                        });
-                        __syncthreads();
-                        mma_sub<false>(C + p * kLdc, kLdc, R, pw, C + k0 * kLdc, kLdc, S1, LDS, Kc);
-                        __syncthreads();
-                    }
-                    for (int idx = threadIdx.x; idx < kPb * kPb; idx += kThreads) {
-                        const int i = idx & (kPb - 1), j = idx / kPb;
-                        S0[i + j * (kPb + 1)] =
-                            (i < pw && j < pw && i >= j) ? __ldcg(DL + (p + i) + (size_t)(p + j) * D.ld) : 0.0;
-                    }
-                    __syncthreads();
-                    if (threadIdx.x < pw) sv[threadIdx.x] = 1.0 / S0[threadIdx.x * (kPb + 2)];
-                    __syncthreads();
-                    trsm_rows_dir<true>(C + p * kLdc, kLdc, R, pw, S0, kPb + 1, sv);
-                    __syncthreads();
-                }
+                selinv_back(C, R, w, S0, S1, sv, lget);
                 double* T = Sg + O.off + t.rs0;
-                for_rc(R, w, [&](int r, int c) { __stcg(T + r + (size_t)c * O.ld, C[r + c * kLdc]); });
+                for_rc(R, w, [&](int r, int c) { __stcg(T + r + (size_t)c * O.ld, C[r + c * kRLd]); });
             }
         } else if (t.kind == SN_S_DIAG && s_ok) {
-            for_rc(w, w, [&](int r, int c) { C[r + c * kLdc] = 0.0; });
+            for (int e = threadIdx.x; e < w * (w + 1) / 2; e += kThreads) C[e] = 0.0;
             __syncthreads();
             for (int ci = t.cbeg; ci < t.cend; ++ci) {
                 const SnSCon q = a.cons[ci];
@@ -2600,51 +2648,30 @@ __global__ void __launch_bounds__(kThreads, 1) sn_selinv_kernel(SnSelinvArgs a) 
                 if (!s_ok) break;
                 const double* ST = Sg + Lc.off;
                 const double* LT = Lf + Lc.off;
-                for (int i0 = 0; i0 < Lc.h; i0 += kKc) {
-                    const int Kc = min(kKc, Lc.h - i0);
-                    const int Mp = ((w + 3) & ~3) + 4;
-                    stage_gather<false>(S0, LDS, w, Mp, Kc,
-                                        [&](int r, int k) { return __ldcg(ST + (i0 + k) + (size_t)r * Lc.ld); });
-                    stage_gather<false>(S1, LDS, w, Mp, Kc,
-                                        [&](int r, int k) { return __ldcg(LT + (i0 + k) + (size_t)r * Lc.ld); });
-                    __syncthreads();
-                    mma_sub<true>(C, kLdc, w, w, S0, LDS, S1, LDS, Kc);  // C = -Z (lower)
+                for (int i0 = 0; i0 < Lc.h; i0 += kSpK) {
+                    const int Kc = min(kSpK, Lc.h - i0);
+                    auto ga = [&](int r, int k) { return __ldcg(ST + (i0 + k) + (size_t)r * Lc.ld); };
+                    auto gb = [&](int r, int k) { return __ldg(LT + (i0 + k) + (size_t)r * Lc.ld); };
+                    auto epi = [&](int r, int c, double v) { C[pk(w, r, c)] -= v; };  // C = -Z (lower)
+                    if (sp_stage_ab(S0, w, ga, S1, w, gb, Kc)) {
+                        sp_product<true>(S0, 0, w, S1, 0, w, epi);
+                    } else {
+                        for (int e = threadIdx.x; e < w * w; e += kThreads) {
+                            const int r = e % w, c = e / w;
+                            if (r < c) continue;
+                            double v = 0.0;
+                            for (int k = 0; k < Kc; ++k) v = fma(ga(r, k), gb(c, k), v);
+                            epi(r, c, v);
+                        }
+                    }
                     __syncthreads();
                 }
             }
             if (s_ok) {
-                // packed lower triangle of L_JJ: (r, c) at c*w - c(c-1)/2 + r - c
-                double* Lp = S0;
-                for_rc(w, w, [&](int r, int c) {
-                    if (r >= c) Lp[c * w - c * (c - 1) / 2 + (r - c)] = __ldcg(DL + r + (size_t)c * D.ld);
-                });
-                __syncthreads();
-                for (int c = w - 1; c >= 0; --c) {
-                    const double* Lcol = Lp + c * w - c * (c - 1) / 2 - c;  // Lcol[i] = L[i][c]
-                    const double inv = 1.0 / Lcol[c];
-                    for (int r = c + 1 + threadIdx.x; r < w; r += kThreads) {
-                        double s0 = C[r + c * kLdc], s1 = 0.0;
-                        int i = c + 1;
-                        for (; i + 1 < w; i += 2) {
-                            s0 = fma(-Lcol[i], i >= r ? C[i + r * kLdc] : C[r + i * kLdc], s0);
-                            s1 = fma(-Lcol[i + 1], i + 1 >= r ? C[i + 1 + r * kLdc] : C[r + (i + 1) * kLdc], s1);
-                        }
-                        if (i < w) s0 = fma(-Lcol[i], i >= r ? C[i + r * kLdc] : C[r + i * kLdc], s0);
-                        C[r + c * kLdc] = (s0 + s1) * inv;
-                    }
-                    __syncthreads();
-                    if (threadIdx.x < 32) {
-                        double sacc = 0.0;
-                        for (int i = c + 1 + threadIdx.x; i < w; i += 32) sacc = fma(Lcol[i], C[i + c * kLdc], sacc);
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) sacc += __shfl_down_sync(0xffffffffu, sacc, o);
-                        if (threadIdx.x == 0) C[c + c * kLdc] = inv * inv + (C[c + c * kLdc] - sacc) * inv;
-                    }
-                    __syncthreads();
-                }
+                selinv_diag(C, w, w - 1, S0, S1, sv, lget);
                 double* T = Sg + D.off;
                 for_rc(w, w, [&](int r, int c) {
-                    if (r >= c) __stcg(T + r + (size_t)c * D.ld, C[r + c * kLdc]);
+                    if (r >= c) __stcg(T + r + (size_t)c * D.ld, C[pk(w, r, c)]);
                 });
             }
         }
@@ -2736,7 +2763,7 @@ int device_info(int* dev, int* sms) {
         if (cudaFuncSetAttribute(replay_kernel_t<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)kRSmemBytes) != cudaSuccess)
             return STC_ERR_CUDA;
-        if (cudaFuncSetAttribute(selinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) != cudaSuccess)
+        if (cudaFuncSetAttribute(selinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRSmemBytes) != cudaSuccess)
             return STC_ERR_CUDA;
         if (cudaFuncSetAttribute(solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSolveSmem) != cudaSuccess)
             return STC_ERR_CUDA;
@@ -2746,7 +2773,7 @@ int device_info(int* dev, int* sms) {
         if (cudaFuncSetAttribute(sn_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(kRPacked * sizeof(double))) != cudaSuccess)
             return STC_ERR_CUDA;
-        if (cudaFuncSetAttribute(sn_selinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemBytes) !=
+        if (cudaFuncSetAttribute(sn_selinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRSmemBytes) !=
             cudaSuccess)
             return STC_ERR_CUDA;
         d.attr_set = true;
@@ -3112,8 +3139,8 @@ int sn_selinv(stc_plan* P, const void* d_factor, int64_t batch, void* d_sigma, v
     a.ntasks = (int)Sp.stasks.size(); a.batch = batch;
     a.spin = P->opt.spin_limit > 0 ? P->opt.spin_limit : kDefaultSpin;
     const long long total = (long long)a.ntasks * batch;
-    const int grid = grid_of(P, sms, total);
-    sn_selinv_kernel<<<grid, kThreads, kSmemBytes, st>>>(a);
+    const int grid = grid_of(P, default_ctas(sms, batch), total);
+    sn_selinv_kernel<<<grid, kThreads, kRSmemBytes, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
 
@@ -3497,8 +3524,8 @@ extern "C" int stc_selinv(const stc_plan* Pc, const void* d_factor, int64_t batc
     a.ntasks = (int)P->stasks.size(); a.batch = batch; a.nb = (int)P->nb;
     a.spin = P->opt.spin_limit > 0 ? P->opt.spin_limit : kDefaultSpin;
     const long long total = (long long)a.ntasks * batch;
-    const int grid = grid_of(P, sms, total);
-    selinv_kernel<<<grid, kThreads, kSmemBytes, st>>>(a);
+    const int grid = grid_of(P, default_ctas(sms, batch), total);
+    selinv_kernel<<<grid, kThreads, kRSmemBytes, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
 

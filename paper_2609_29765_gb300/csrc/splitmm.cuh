@@ -45,9 +45,9 @@ __device__ __forceinline__ int* sp_exp(double* S) { return reinterpret_cast<int*
 // and two rows of four pairs (the fragment loads) both touch every bank once.
 __device__ __forceinline__ int sp_slot(int r, int kp) { return r * 8 + (kp ^ (((r & 1) << 2) | ((r >> 1) & 3))); }
 
-// One row of a chunk, v[0..15] (zero from K on), to digits and exponent.  Returns false when the row must
-// not take this path (see above).
-__device__ __forceinline__ bool sp_split_row(const double (&v)[kSpK], int K, double* S, int r) {
+// Biased exponent of the largest entry of a chunk row v[0..15]; ok: the row can take this
+// path (see above).
+__device__ __forceinline__ int sp_row_exp(const double (&v)[kSpK], bool& ok) {
     unsigned m = 0u, any = 0u;
 #pragma unroll
     for (int k = 0; k < kSpK; ++k) {
@@ -56,7 +56,12 @@ __device__ __forceinline__ bool sp_split_row(const double (&v)[kSpK], int K, dou
         any |= h | (unsigned)__double2loint(v[k]);
     }
     const int e = (int)(m >> 20);
-    const bool ok = any == 0u || (e >= 1023 - 400 && e <= 1023 + 400);
+    ok = any == 0u || (e >= 1023 - 400 && e <= 1023 + 400);
+    return e;
+}
+
+// The digits of row r, v[0..15] (zero from K on), e its exponent.
+__device__ __forceinline__ void sp_split_row(const double (&v)[kSpK], int e, int K, double* S, int r) {
     sp_exp(S)[r] = e;
     uint4* D = sp_digits(S);
 #pragma unroll
@@ -83,7 +88,6 @@ __device__ __forceinline__ bool sp_split_row(const double (&v)[kSpK], int K, dou
         D[sp_slot(r, kp)] = make_uint4(__byte_perm(hi[0], hi[1], 0x7632), __byte_perm(hi[0], hi[1], 0x5410),
                                        __byte_perm(lo[0], lo[1], 0x7632), __byte_perm(lo[0], lo[1], 0x5410));
     }
-    return ok;
 }
 
 // Whether a chunk's product is worth the split: 2 x 2 DFMA micro-tiles take 256 clocks per
@@ -94,34 +98,38 @@ __device__ __forceinline__ bool sp_split_row(const double (&v)[kSpK], int K, dou
 constexpr int kSpWorth = 8;
 __device__ __forceinline__ bool sp_worth(int entries, int K) { return K * ((entries + 511) >> 9) >= kSpWorth; }
 
-// The chunk's row r as get(r, k), k < K; zero for r >= R or k >= K.
-template <class Get>
-__device__ __forceinline__ bool sp_stage_row(double* S, int r, int R, int K, Get get) {
+// Operands A (R x K, entries ga(r, k)) and B (Cn x K, gb(c, k)) of a chunk into the digit
+// buffers SA and SB, a thread per row (R + Cn <= blockDim.x); returns on every thread
+// whether all rows can take the tensor path, after a barrier.  IN_PLACE: ga or gb may read
+// SA or SB; nothing is written unless the result is true.
+template <bool IN_PLACE, class GetA, class GetB>
+__device__ __forceinline__ bool sp_stage_t(double* SA, int R, GetA ga, double* SB, int Cn, GetB gb, int K) {
+    const int i = threadIdx.x;
     double v[kSpK];
 #pragma unroll
-    for (int k = 0; k < kSpK; ++k) v[k] = (r < R && k < K) ? get(r, k) : 0.0;
-    return sp_split_row(v, K, S, r);
+    for (int k = 0; k < kSpK; ++k) v[k] = 0.0;
+    if (i < R) {
+#pragma unroll
+        for (int k = 0; k < kSpK; ++k)
+            if (k < K) v[k] = ga(i, k);
+    } else if (i < R + Cn) {
+#pragma unroll
+        for (int k = 0; k < kSpK; ++k)
+            if (k < K) v[k] = gb(i - R, k);
+    }
+    bool ok = true;
+    const int e = sp_row_exp(v, ok);
+    if (IN_PLACE && !__syncthreads_and(ok)) return false;
+    if (i < R + Cn) sp_split_row(v, e, K, i < R ? SA : SB, i < R ? i : i - R);
+    return __syncthreads_and(ok);
 }
-
-// Operands A (R x K) and B (Cn x K) of a chunk into the digit buffers SA and SB, a thread
-// per row; every thread returns whether all rows can take the tensor path (a barrier).
-// R, Cn <= kSpRows, K <= kSpK.
 template <class GetA, class GetB>
 __device__ __forceinline__ bool sp_stage_ab(double* SA, int R, GetA ga, double* SB, int Cn, GetB gb, int K) {
-    const int Ra = (R + 15) & ~15, Rb = (Cn + 7) & ~7;
-    bool ok = true;
-    for (int i = threadIdx.x; i < Ra + Rb; i += blockDim.x) {
-        if (i < Ra) ok &= sp_stage_row(SA, i, R, K, ga);
-        else ok &= sp_stage_row(SB, i - Ra, Cn, K, gb);
-    }
-    return __syncthreads_and(ok);
+    return sp_stage_t<false>(SA, R, ga, SB, Cn, gb, K);
 }
 template <class GetA>
 __device__ __forceinline__ bool sp_stage_a(double* SA, int R, GetA ga, int K) {
-    const int Ra = (R + 15) & ~15;
-    bool ok = true;
-    for (int i = threadIdx.x; i < Ra; i += blockDim.x) ok &= sp_stage_row(SA, i, R, K, ga);
-    return __syncthreads_and(ok);
+    return sp_stage_t<false>(SA, R, ga, SA, 0, ga, K);
 }
 
 // Digits of one 16-byte pair as eight f16x2 registers (the two columns of digit d), exact:
@@ -157,12 +165,12 @@ __device__ __forceinline__ double sp_double(long long T, int E) {
     return __longlong_as_double((long long)(bits | ((unsigned long long)T & 0x8000000000000000ull)));
 }
 
-// sum over the chunk of A(r, k) B(c, k) for every r < R, c < Cn (LOWER: at least every
+// sum over the chunk of A(a0 + r, k) B(b0 + c, k) for every r < R, c < Cn (LOWER: at least every
 // r >= c), one call epi(r, c, value) per entry; 16 x 8 units of the product spread over the
 // CTA's warps in contiguous runs, so that a warp expands a strip of A once.  epi must not
 // synchronise.
 template <bool LOWER, class Epi>
-__device__ __forceinline__ void sp_product(double* SA, int R, double* SB, int Cn, Epi epi) {
+__device__ __forceinline__ void sp_product(double* SA, int a0, int R, double* SB, int b0, int Cn, Epi epi) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const uint4 *A = sp_digits(SA), *B = sp_digits(SB);
@@ -187,16 +195,18 @@ __device__ __forceinline__ void sp_product(double* SA, int R, double* SB, int Cn
     while (u < uend) {
         unsigned fa[4][8];
         const int r0 = s * 16 + g;
-        sp_expand(A[sp_slot(r0, t)], fa[0]);
-        sp_expand(A[sp_slot(r0 + 8, t)], fa[1]);
-        sp_expand(A[sp_slot(r0, t + 4)], fa[2]);
-        sp_expand(A[sp_slot(r0 + 8, t + 4)], fa[3]);
-        const int e0 = ea[r0], e1 = ea[r0 + 8];
+        const int ra = a0 + min(r0, R - 1), rb = a0 + min(r0 + 8, R - 1);  // rows past the end: not used
+        sp_expand(A[sp_slot(ra, t)], fa[0]);
+        sp_expand(A[sp_slot(rb, t)], fa[1]);
+        sp_expand(A[sp_slot(ra, t + 4)], fa[2]);
+        sp_expand(A[sp_slot(rb, t + 4)], fa[3]);
+        const int e0 = ea[ra], e1 = ea[rb];
         const int cend = LOWER ? min(2 * s + 2, NC) : NC;
         for (; c < cend && u < uend; ++c, ++u) {
             unsigned fb[2][8];
-            sp_expand(B[sp_slot(c * 8 + g, t)], fb[0]);
-            sp_expand(B[sp_slot(c * 8 + g, t + 4)], fb[1]);
+            const int cb = b0 + min(c * 8 + g, Cn - 1);
+            sp_expand(B[sp_slot(cb, t)], fb[0]);
+            sp_expand(B[sp_slot(cb, t + 4)], fb[1]);
             float acc[8][4];
 #pragma unroll
             for (int i = 0; i < 8; ++i)
@@ -206,7 +216,7 @@ __device__ __forceinline__ void sp_product(double* SA, int R, double* SB, int Cn
                     else sp_mma(acc[i + j], acc[i + j], fa[0][i], fa[1][i], fa[2][i], fa[3][i], fb[0][j], fb[1][j]);
                 }
             const int c0 = c * 8 + 2 * t;
-            const int f0 = eb[c0], f1 = eb[c0 + 1];
+            const int f0 = eb[b0 + min(c0, Cn - 1)], f1 = eb[b0 + min(c0 + 1, Cn - 1)];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int r = r0 + (q >> 1) * 8, cc = c0 + (q & 1);
