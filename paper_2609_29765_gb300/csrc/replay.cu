@@ -4,10 +4,12 @@
 // Sec. 4 (active-column and banded tiles), Sec. 5.3 (progress matrix -> counters).
 //
 // GB300 notes that shape this file:
-//  * FP64 runs at ~2 DFMA/clk/SM (measured 1.21 TFLOP/s DFMA, 1.06 TFLOP/s for
-//    mma.sync.m8n8k4.f64), so every tile kernel is DFMA-bound; tiles live in shared
-//    memory, the inner loops are 4x4 register micro-tiles of DFMA, and the tensor-core
-//    DMMA path is not used (it is slower on this part).
+//  * FP64 runs at 2 DFMA/clk/SM (1.26 TFLOP/s; mma.sync.m8n8k4.f64 shares that pipe and is
+//    no faster), a dependent DFMA takes 64-70 clocks of a warp whatever its active lanes.  So
+//    the tile products of any size go to the tensor cores as exact integer products of split
+//    operands (splitmm.cuh), small ones are one entry per thread, and POTRF, TRSM and the
+//    solves, which are chains, are laid out for few dependent FP64 instructions.  Tiles live
+//    in shared memory.
 //  * One persistent kernel per call walks the whole DAG of every batch item: CTAs take
 //    task slots from a global counter in a topological (earliest-start) order and wait
 //    on per-tile completion counters (the paper's progress matrix P and per-cell
@@ -158,11 +160,10 @@ __device__ __forceinline__ void for_rc(int R, int NC, Fn f) {
 template <bool LOWER, int TR, int TC, bool PACKED>
 __device__ void mma_tiles(double* __restrict__ C, int ldc, int R, int Cn,
                           const double* __restrict__ A, int lda,
-                          const double* __restrict__ B, int ldb, int K, int pnb, int pr0, int pc0,
-                          int tid0 = 0, int nthr = kThreads) {
+                          const double* __restrict__ B, int ldb, int K, int pnb, int pr0, int pc0) {
     const int MR = (R + TR - 1) / TR, MC = (Cn + TC - 1) / TC;
     const int count = LOWER ? MR * (MR + 1) / 2 : MR * MC;
-    for (int mt = (int)threadIdx.x - tid0; mt < count; mt += nthr) {
+    for (int mt = threadIdx.x; mt < count; mt += kThreads) {
         int ri, cj;
         if (LOWER) {
             // mt -> (ri, cj), cj <= ri, row-major over the lower triangle
@@ -216,8 +217,8 @@ __device__ void mma_tiles(double* __restrict__ C, int ldc, int R, int Cn,
     }
 }
 
-// 4x4 micro-tiles when they keep at least 3/4 of the CTA busy, else 2x2 (four times as
-// many micro-tiles, so narrow row slices still occupy every warp).
+// 4x4 micro-tiles when they keep at least 3/4 of the CTA busy, an entry per thread when there
+// are no more entries than threads (a thread's FMAs are a chain of 64 clocks each), else 2x2.
 template <bool LOWER>
 __device__ __forceinline__ void mma_sub(double* C, int ldc, int R, int Cn, const double* A, int lda,
                                         const double* B, int ldb, int K) {
@@ -225,6 +226,8 @@ __device__ __forceinline__ void mma_sub(double* C, int ldc, int R, int Cn, const
     const int c44 = LOWER ? m4 * (m4 + 1) / 2 : m4 * n4;
     if (c44 >= (kThreads * 3) / 4)
         mma_tiles<LOWER, 4, 4, false>(C, ldc, R, Cn, A, lda, B, ldb, K, 0, 0, 0);
+    else if ((LOWER ? R * (R + 1) / 2 : R * Cn) <= kThreads)
+        mma_tiles<LOWER, 1, 1, false>(C, ldc, R, Cn, A, lda, B, ldb, K, 0, 0, 0);
     else
         mma_tiles<LOWER, 2, 2, false>(C, ldc, R, Cn, A, lda, B, ldb, K, 0, 0, 0);
 }
@@ -233,15 +236,15 @@ __device__ __forceinline__ void mma_sub(double* C, int ldc, int R, int Cn, const
 // (pr0, pc0) of the tile.
 template <bool LOWER>
 __device__ __forceinline__ void mma_sub_packed(double* P, int pnb, int pr0, int pc0, int R, int Cn,
-                                               const double* A, int lda, const double* B, int ldb, int K,
-                                               int tid0 = 0, int nthr = kThreads) {
-    if ((int)threadIdx.x < tid0 || (int)threadIdx.x >= tid0 + nthr) return;
+                                               const double* A, int lda, const double* B, int ldb, int K) {
     const int m4 = (R + 3) >> 2, n4 = (Cn + 3) >> 2;
     const int c44 = LOWER ? m4 * (m4 + 1) / 2 : m4 * n4;
-    if (c44 >= (nthr * 3) / 4)
-        mma_tiles<LOWER, 4, 4, true>(P, 0, R, Cn, A, lda, B, ldb, K, pnb, pr0, pc0, tid0, nthr);
+    if (c44 >= (kThreads * 3) / 4)
+        mma_tiles<LOWER, 4, 4, true>(P, 0, R, Cn, A, lda, B, ldb, K, pnb, pr0, pc0);
+    else if ((LOWER ? R * (R + 1) / 2 : R * Cn) <= kThreads)
+        mma_tiles<LOWER, 1, 1, true>(P, 0, R, Cn, A, lda, B, ldb, K, pnb, pr0, pc0);
     else
-        mma_tiles<LOWER, 2, 2, true>(P, 0, R, Cn, A, lda, B, ldb, K, pnb, pr0, pc0, tid0, nthr);
+        mma_tiles<LOWER, 2, 2, true>(P, 0, R, Cn, A, lda, B, ldb, K, pnb, pr0, pc0);
 }
 
 // Forward substitution of a row block against a panel: X(r, 0:pw) <- X(r, 0:pw) D^{-T},
@@ -301,11 +304,6 @@ __device__ __forceinline__ void trsm_rows_dir(double* X, int ldx, int R, int pw,
     if (R <= kThreads / 8) trsm_rows_t<8, BACK>(X, ldx, R, pw, D, ldd, dinv);
     else if (R <= kThreads / 4) trsm_rows_t<4, BACK>(X, ldx, R, pw, D, ldd, dinv);
     else trsm_rows_t<2, BACK>(X, ldx, R, pw, D, ldd, dinv);
-}
-
-__device__ __forceinline__ void trsm_rows(double* X, int ldx, int R, int pw, const double* D, int ldd,
-                                          const double* dinv) {
-    trsm_rows_dir<false>(X, ldx, R, pw, D, ldd, dinv);
 }
 
 struct SnArgs {
@@ -443,11 +441,11 @@ __device__ void read_diag_rows(const double* T, const DTile& d, int nb, int r0, 
 
 // Entries L[r][c], r in [r0, r1), c in [c0, min(c1, r + 1)), written to a diagonal tile's
 // storage in storage order (a warp per stored column / per row): T <- get(r, c); banded
-// tiles only inside the band.
+// tiles only inside the band.  Called by nthr threads (whole warps), tid < nthr.
 template <class Get>
-__device__ void write_diag_rows(double* T, const DTile& d, int nb, int r0, int r1, int c0, int c1, Get get) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    constexpr int kW = kThreads / 32;
+__device__ void write_diag_rows(double* T, const DTile& d, int nb, int r0, int r1, int c0, int c1, Get get,
+                                int tid, int nthr) {
+    const int lane = tid & 31, warp = tid >> 5, kW = nthr >> 5;
     if (d.kind == TILE_DIAG_DENSE) {
         for (int c = c0 + warp; c < c1; c += kW)
             for (int r = max(r0, c) + lane; r < r1; r += 32) __stcg(T + r + (size_t)c * nb, get(r, c));
@@ -470,15 +468,14 @@ __device__ void load_diag_packed(double* P, const double* T, const DTile& d, int
     read_diag_rows(T, d, nb, 0, nb, [&](int r, int c, double v) { P[pk(nb, r, c)] = v; });
 }
 // Columns [c0, c1) of the packed triangle back into the diagonal tile's storage (dense:
-// with the zero upper part; banded: the entries inside the band).
-__device__ void store_diag_cols(const double* P, double* T, const DTile& d, int nb, int c0, int c1) {
+// with the zero upper part; banded: the entries inside the band), by nthr threads.
+__device__ void store_diag_cols(const double* P, double* T, const DTile& d, int nb, int c0, int c1, int tid, int nthr) {
     if (d.kind == TILE_DIAG_DENSE) {
-        for_rc(nb, c1 - c0, [&](int r, int cc) {
-            const int c = c0 + cc;
-            __stcg(T + r + (size_t)c * nb, r >= c ? P[pk(nb, r, c)] : 0.0);
-        });
+        const int lane = tid & 31;
+        for (int c = c0 + (tid >> 5); c < c1; c += nthr >> 5)
+            for (int r = lane; r < nb; r += 32) __stcg(T + r + (size_t)c * nb, r >= c ? P[pk(nb, r, c)] : 0.0);
     } else {
-        write_diag_rows(T, d, nb, c0, min(nb, c1 + d.kd), c0, c1, [&](int r, int c) { return P[pk(nb, r, c)]; });
+        write_diag_rows(T, d, nb, c0, min(nb, c1 + d.kd), c0, c1, [&](int r, int c) { return P[pk(nb, r, c)]; }, tid, nthr);
     }
 }
 
@@ -537,6 +534,22 @@ __device__ __forceinline__ void inner_cols(const DUpd& u, const int16_t* imap, b
     }
 }
 
+// Entry (r, k) of a chunk of stored columns of a tile, as stage_cols reads it: row
+// row0 + r, inner position k0 + k of the update's A (or B) operand.
+struct ColGet {
+    const double* T;
+    size_t nb;
+    const int16_t* imap;
+    int s0;
+    __device__ __forceinline__ ColGet(const double* T_, int nb_, int row0, const DUpd& u, const int16_t* im, bool use_b,
+                                      int k0)
+        : T(T_ + row0), nb((size_t)nb_), imap(u.kmap < 0 ? nullptr : im + 2 * (u.kmap + k0) + (use_b ? 1 : 0)),
+          s0((use_b ? u.kb0 : u.ka0) + k0) {}
+    __device__ __forceinline__ double operator()(int r, int k) const {
+        return __ldcg(T + r + (size_t)(imap ? imap[2 * k] : s0 + k) * nb);
+    }
+};
+
 // B rows for a GEMM: rows = logical columns of the output tile's stored columns oc0.. .
 __device__ void stage_rows_gather(double* S, int ld, const double* T, int nb, const DTile& O,
                                   const int16_t* saind, int oc0, int Cn, const DUpd& u,
@@ -553,155 +566,210 @@ __device__ void stage_rows_gather(double* S, int ld, const double* T, int nb, co
     });
 }
 
-// POTRF of a diagonal tile held as a packed lower triangle (see potrf_packed below).
-template <int PP>
-struct PotrfShared {
-    double blk[PP][PP];    // L of the current panel's diagonal block, blk[row][col]
-    double inv[PP];        // 1 / L_jj of the panel
-    int bad;
-};
+// ---- 16-column panels: diagonal block, triangular solve, POTRF ---------------------------
+constexpr int kP16 = 16;
+constexpr int kM16 = kP16 + 1;  // leading dimension of a panel's 16 x 16 unit triangle
 
-// All threads: rows [p+pw, rend) of panel p solved against the diagonal block; the solved
-// rows also go to S (row i at S[i - p - pw], column l at stride kRStLd), zero-padded.
-template <int PP>
-__device__ void potrf_rows_below(double* P, int nb, int p, int pw, int rend, double* S,
-                                 const PotrfShared<PP>& sh) {
-    const int R2 = rend - p - pw;
-    const int R2p = ((max(R2, 0) + 3) & ~3) + 4;
-    for (int rr = threadIdx.x; rr < R2p; rr += kThreads) {
-        const int i = p + pw + rr;
-        double x[PP];
-        if (rr < R2) {
+// One warp: Cholesky of the pw x pw (pw <= 16) block at (p, p) of the packed triangle P, in
+// place.  M receives its unit triangle L diag(L)^{-1} (strict lower part, M(i, j) at
+// i + 17 j, zero from row pw on), inv the reciprocals 1 / L_jj; returns the first
+// non-positive pivot's column (of P) or -1.  Lane 2 r + h holds row r, columns 2 q + h.
+// Bound by the chain from pivot to pivot: a dependent FP64 instruction takes 64-70 clocks of
+// the warp's pipe whatever its active lanes, a reciprocal square root 400 (390 in 64-bit
+// integers).  So the block is eliminated as M D M^T: a pivot then needs a reciprocal, whose
+// last step is folded into the column M_rj = u_rj / d_j (third-order Householder iteration
+// from the hardware estimate, e = 1 - d y0, 1 / d = y0 (1 + e + e^2 + ...)), and the 16
+// square roots come at the end side by side: 11,400 clocks alone, 17,100 with a reciprocal
+// square root per pivot.  A block with a pivot outside [2^-991, 2^992) (an integer test: a
+// double comparison is an FP64 instruction too) is done again one column at a time.
+__device__ int potrf_diag16(double* P, int nb, int p, int pw, double* M, double* inv) {
+    const int lane = threadIdx.x & 31, r = lane >> 1, h = lane & 1;
+    double v[8];  // A, then u = M D; entries above the diagonal hold anything
 #pragma unroll
-            for (int l = 0; l < PP; ++l) x[l] = l < pw ? P[pk(nb, i, p + l)] : 0.0;
-#pragma unroll
-            for (int j = 0; j < PP; ++j) {
-                if (j < pw) {
-                    double sacc = x[j];
-#pragma unroll
-                    for (int l = 0; l < j; ++l) sacc = fma(-x[l], sh.blk[j][l], sacc);
-                    x[j] = sacc * sh.inv[j];
-                }
-            }
-#pragma unroll
-            for (int l = 0; l < PP; ++l)
-                if (l < pw) P[pk(nb, i, p + l)] = x[l];
-        } else {
-#pragma unroll
-            for (int l = 0; l < PP; ++l) x[l] = 0.0;
-        }
-#pragma unroll
-        for (int l = 0; l < PP; ++l) S[rr + l * kRStLd] = x[l];
+    for (int q = 0; q < 8; ++q) {
+        const int c = 2 * q + h;
+        v[q] = (r < pw && c <= r) ? P[pk(nb, p + r, p + c)] : 0.0;
     }
-}
-
-// Warp 0 only: the 8x8 diagonal block at (p, p), first reduced by the rank-kw update
-// from the solved rows of the previous panel (S rows 0..rv-1, columns at stride ld; rows
-// from rv on are outside the previous panel's band and zero there), then factored.  Each lane holds two entries of one row, (r, c0) and (r, c0 + 1) with
-// r = lane / 4 and c0 = 2 (lane % 4), so a pivot costs one reciprocal square root and
-// two fused multiply-adds per lane instead of one per later column.
-__device__ void potrf_diag8(double* P, int nb, int p, int pw, const double* S, int ld, int kw, int rv,
-                            PotrfShared<8>& sh) {
-    const int lane = threadIdx.x & 31;
-    const int r = lane >> 2, c0 = 2 * (lane & 3);
-    double x[2];
+    bool odd = false;
+    double dj = 1.0;  // lane j: pivot j
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const int c = c0 + e;
-        double v = 0.0;
-        if (r < pw && c <= r) {
-            v = P[pk(nb, p + r, p + c)];
-            if (r < rv)
-                for (int m = 0; m < kw; ++m) v = fma(-S[r + m * ld], S[c + m * ld], v);
-        }
-        x[e] = v;
-    }
-    int badl = -1;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
+    for (int j = 0; j < kP16; ++j) {
         if (j < pw) {
-            const int src = 4 * j + (j >> 1);
-            const double d = __shfl_sync(0xffffffffu, x[j & 1], src);
-            if (!(d > 0.0) && badl < 0) badl = p + j;  // the first non-positive pivot
-            const double inv = rsqrt(d);
-            if ((lane & 3) == (j >> 1) && r >= j) x[j & 1] = (r == j) ? d * inv : x[j & 1] * inv;
-            // L(r, j) and L(c, j) of this lane's entries, then the rank-1 update
-            const double lr = __shfl_sync(0xffffffffu, x[j & 1], 4 * r + (j >> 1));
-            const double l0 = __shfl_sync(0xffffffffu, x[j & 1], 4 * c0 + (j >> 1));
-            const double l1 = __shfl_sync(0xffffffffu, x[j & 1], 4 * (c0 + 1) + (j >> 1));
-            if (c0 > j && r >= c0) x[0] = fma(-lr, l0, x[0]);
-            if (c0 + 1 > j && r >= c0 + 1) x[1] = fma(-lr, l1, x[1]);
-            if (lane == 0) sh.inv[j] = inv;
+            const int q = j >> 1, hj = j & 1;
+            const double d = __shfl_sync(0xffffffffu, v[q], 2 * j + hj);
+            const double ur = __shfl_sync(0xffffffffu, v[q], 2 * r + hj);
+            double uc[8];
+#pragma unroll
+            for (int z = q; z < 8; ++z)
+                if (2 * z + 1 > j) uc[z] = __shfl_sync(0xffffffffu, v[q], 2 * (2 * z + h) + hj);
+            if (lane == j) dj = d;
+            odd |= (unsigned)(__double2hiint(d) - 0x02000000) >= 0x7bc00000u;
+            double y0;
+            asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y0) : "d"(d));
+            const double w = ur * y0, e = fma(-d, y0, 1.0);
+            const double m = fma(w, fma(e, e, e), w);
+#pragma unroll
+            for (int z = q; z < 8; ++z)
+                if (2 * z + 1 > j) {
+                    const double x = fma(-m, uc[z], v[z]);
+                    if (2 * z + h > j) v[z] = x;
+                }
+            if (h == 0 && r > j) M[r + j * kM16] = m;
         }
     }
+    int bad = -1;
+    if (!odd) {
+        const double iv = rsqrt(dj);
+        if (lane < pw) inv[lane] = iv;
 #pragma unroll
-    for (int e = 0; e < 2; ++e) {
-        const int c = c0 + e;
-        const bool in = r < pw && c <= r;
-        sh.blk[r][c] = in ? x[e] : 0.0;
-        if (in) P[pk(nb, p + r, p + c)] = x[e];
+        for (int q = 0; q < 8; ++q) {
+            const int c = 2 * q + h;
+            const double ic = __shfl_sync(0xffffffffu, iv, c);
+            if (r < pw && c <= r) P[pk(nb, p + r, p + c)] = v[q] * ic;
+        }
+    } else {
+        // column by column in place: lane r holds row r of the column
+        for (int j = 0; j < pw; ++j) {
+            const double d = P[pk(nb, p + j, p + j)];
+            if (!(d > 0.0) && bad < 0) bad = p + j;  // the first non-positive pivot
+            const double y = rsqrt(d);
+            const int i = j + lane;
+            __syncwarp();
+            const double l = i < pw ? P[pk(nb, p + i, p + j)] * y : 0.0;
+            if (i < pw) P[pk(nb, p + i, p + j)] = l;
+            if (lane == 0) inv[j] = y;
+            for (int c = j + 1; c < pw; ++c) {
+                const double lc = __shfl_sync(0xffffffffu, l, c - j);
+                if (i >= c && i < pw) P[pk(nb, p + i, p + c)] = fma(-l, lc, P[pk(nb, p + i, p + c)]);
+            }
+            if (i > j && i < pw) M[i + j * kM16] = l * y;
+            __syncwarp();
+        }
     }
-    if (lane == 0 && badl >= 0 && sh.bad < 0) sh.bad = badl;
+    // zero above the diagonal and from row or column pw on
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
+        if (2 * q + h >= r || r >= pw) M[r + (2 * q + h) * kM16] = 0.0;
+    __syncwarp();
+    return bad;
 }
 
-// Blocked right-looking Cholesky of the w x w leading block of the packed lower
-// triangle P (pk layout, tile width nb) in shared memory, panels of 8 with a one-panel
-// look-ahead: warp 0 applies the previous panel's rank-8 update to the next 8x8
-// diagonal block and factors it, while warps 1-7 update everything below that block
-// (the rest of the next panel's columns and the trailing triangle) in one pass; then
-// the rows below the new block are solved against it, one row per thread, and copied to
-// the staging buffer S for the next step.  Rows more than kd below the diagonal are
-// structurally zero and skipped.  *bad receives the first non-positive pivot column (or
-// -1); *logsum = sum_j log L_jj, one log per diagonal entry reduced in a fixed order.
-// pub(c) is called by every thread (after a barrier) each time columns [c - pubw, c) have
-// become final, for c < w a multiple of pubw (a multiple of 8).  *bad and *logsum are
-// valid in thread 0 only.
-template <class Pub>
-__device__ void potrf_packed(double* P, int nb, int w, int kd, double* S, int* bad, double* logsum, int pubw,
-                             Pub pub) {
-    __shared__ PotrfShared<8> sh;
-    if (threadIdx.x == 0) sh.bad = -1;
-    __syncthreads();
-    {
-        const int pw = min(8, w);
-        if (threadIdx.x < 32) potrf_diag8(P, nb, 0, pw, S, kRStLd, 0, 0, sh);
-        __syncthreads();
-        potrf_rows_below<8>(P, nb, 0, pw, min(w, pw + kd), S, sh);
-        __syncthreads();
+// Rows r < R: x(r, 0:pw) <- x(r, 0:pw) L^{-T} for a 16-column panel, at(r, k) a reference to
+// x(r, k); M and inv as potrf_diag16 leaves them.  On the unit triangle a column is one
+// shuffle and one FMA, the scaling by 1 / L_kk comes last.  TPR threads share a row.
+template <int TPR, class At>
+__device__ __forceinline__ void trsm16_t(int R, int pw, const double* M, const double* inv, At at) {
+    constexpr int NJ = kP16 / TPR;
+    const int q = threadIdx.x % TPR, lane = threadIdx.x & 31, base = lane - q;
+    constexpr int rows = kThreads / TPR;
+    for (int rb = 0; rb < R; rb += rows) {
+        const int r = rb + threadIdx.x / TPR;
+        double b[NJ];
+#pragma unroll
+        for (int s = 0; s < NJ; ++s) {
+            const int k = s * TPR + q;
+            b[s] = (r < R && k < pw) ? at(r, k) : 0.0;
+        }
+#pragma unroll
+        for (int j = 0; j < kP16 - 1; ++j) {
+            const double xj = __shfl_sync(0xffffffffu, b[j / TPR], base + (j % TPR));
+#pragma unroll
+            for (int s = 0; s < NJ; ++s) {
+                if (s * TPR + TPR - 1 <= j) continue;  // all of this group's columns are done
+                const int k = s * TPR + q;
+                if (k > j) b[s] = fma(-xj, M[k + j * kM16], b[s]);
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < NJ; ++s) {
+            const int k = s * TPR + q;
+            if (r < R && k < pw) at(r, k) = b[s] * inv[k];
+        }
     }
-    for (int p = 0; p < w; p += 8) {
-        const int pw = min(8, w - p);
-        const int rend = min(w, p + pw + kd);
-        const int pn = p + pw;
-        if (pn >= w) break;
-        const int pwn = min(8, w - pn);
-        const int R3 = rend - pn - pwn;  // rows below the next diagonal block
-        if (threadIdx.x < 32) {
-            potrf_diag8(P, nb, pn, pwn, S, kRStLd, pw, rend - pn, sh);
-        } else if (R3 > 0) {
-            mma_sub_packed<false>(P, nb, pn + pwn, pn, R3, pwn, S + pwn, kRStLd, S, kRStLd, pw, 32, kThreads - 32);
-            mma_sub_packed<true>(P, nb, pn + pwn, pn + pwn, R3, R3, S + pwn, kRStLd, S + pwn, kRStLd, pw,
-                                 32, kThreads - 32);
+}
+template <class At>
+__device__ __forceinline__ void trsm16(int R, int pw, const double* M, const double* inv, At at) {
+    if (R <= kThreads / 16) trsm16_t<16>(R, pw, M, inv, at);
+    else if (R <= kThreads / 8) trsm16_t<8>(R, pw, M, inv, at);
+    else if (R <= kThreads / 4) trsm16_t<4>(R, pw, M, inv, at);
+    else trsm16_t<2>(R, pw, M, inv, at);
+}
+
+// Blocked right-looking Cholesky of the w x w leading block of the packed lower triangle P
+// (pk layout, tile width nb) in shared memory, panels of 16 with a one-panel look-ahead:
+// warp 0 applies the previous panel's update to the next diagonal block and factors it,
+// while the other warps publish the previous panel and update everything else (split
+// products, the panel's rows as digits in S); then the rows below are solved against the
+// new block.  Rows more than kd below the diagonal are structurally zero and skipped.  A
+// 128 x 128 POTRF alone on an SM takes about 100 us (167 us by panels of 8 on the DFMA pipe),
+// a panel of 16 columns 11-12: the diagonal block 5.5, the rows below 1.3-2.9, their digits
+// 0.7, the next block's update 1.6.  wr(c0, c1, t, nt): called by threads t < nt (whole
+// warps), writes the final columns [c0, c1) out; rel(c0, c1): called by one of them after
+// that, once the writes are visible; together they cover every column but the last panel's
+// [*done, w).  Returns the first non-positive pivot column (or -1) on every thread.
+template <class Wr, class Rel>
+__device__ int potrf_packed(double* P, int nb, int w, int kd, double* S, int* done, Wr wr, Rel rel) {
+    __shared__ double s_M[kP16 * kM16], s_inv[kP16];
+    __shared__ int s_bad;
+    const int warp = threadIdx.x >> 5;
+    if (threadIdx.x < 32) {
+        const int bad = potrf_diag16(P, nb, 0, min(kP16, w), s_M, s_inv);
+        if (threadIdx.x == 0) s_bad = bad;
+    }
+    __syncthreads();
+    int p = 0;
+    for (; p + kP16 < w; p += kP16) {
+        const int pn = p + kP16, rend = min(w, pn + kd), R = rend - pn;
+        const int pwn = min(kP16, w - pn);
+        trsm16(R, kP16, s_M, s_inv, [&](int r, int k) -> double& { return P[pk(nb, pn + r, p + k)]; });
+        __syncthreads();
+        auto row = [&](int r, int k) { return P[pk(nb, pn + r, p + k)]; };
+        auto sub = [&](int r, int c) -> double& { return P[pk(nb, pn + r, pn + c)]; };
+        // (up to 22 rows, an entry per thread: DFMAs, as in sp_worth)
+        const bool split = R * (R + 1) / 2 > kThreads && sp_stage_a(S, R, row, kP16);
+        if (!split) {
+            for (int e = threadIdx.x; e < R * (R + 1) / 2; e += kThreads) {
+                int r = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
+                while (r * (r + 1) / 2 > e) --r;
+                while ((r + 1) * (r + 2) / 2 <= e) ++r;
+                const int c = e - r * (r + 1) / 2;
+                double x = sub(r, c);
+                for (int k = 0; k < kP16; ++k) x = fma(-row(r, k), row(c, k), x);
+                sub(r, c) = x;
+            }
+            __syncthreads();
+        }
+        const int units = split && R > 0 ? sp_units<true>(R, R) : 0, first = min(2, units);
+        // the next diagonal block's two units on two warps, then warp 0 factors it
+        if (warp < 2 && warp < first) {
+            sp_run<true>(S, 0, R, S, 0, R, warp, warp + 1, sub);
+            asm volatile("bar.sync 3, %0;" ::"r"(32 * first) : "memory");
+        }
+        if (warp == 0) {
+            const int bad = potrf_diag16(P, nb, pn, pwn, s_M, s_inv);
+            if (threadIdx.x == 0 && bad >= 0 && s_bad < 0) s_bad = bad;
+        } else {
+            constexpr int kOut = kThreads - 32;
+            wr(p, pn, (int)threadIdx.x - 32, kOut);
+            __threadfence();
+            asm volatile("bar.sync 2, %0;" ::"n"(kOut) : "memory");
+            if (threadIdx.x == 32) rel(p, pn);
+            const int u = units - first, nw = kThreads / 32 - 1;
+            sp_run<true>(S, 0, R, S, 0, R, first + u * (warp - 1) / nw, first + u * warp / nw, sub);
         }
         __syncthreads();
-        potrf_rows_below<8>(P, nb, pn, pwn, min(w, pn + pwn + kd), S, sh);
-        __syncthreads();
-        if (pn + pwn < w && (pn + pwn) % pubw == 0) pub(pn + pwn);
     }
-    __shared__ double s_red[kThreads / 32];
+    *done = p;
+    return s_bad;
+}
+
+// sum_j log L_jj of a packed triangle, reduced in a fixed order (every thread).
+__device__ double cta_sum_fixed(double v);
+__device__ __forceinline__ double packed_logsum(const double* P, int nb, int w) {
     double lg = 0.0;
     for (int j = threadIdx.x; j < w; j += kThreads) lg += log(P[pk(nb, j, j)]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) lg += __shfl_down_sync(0xffffffffu, lg, o);
-    if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = lg;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int q = 0; q < kThreads / 32; ++q) t += s_red[q];
-        *bad = sh.bad;
-        *logsum = t;
-    }
-    __syncthreads();
+    return cta_sum_fixed(lg);
 }
 
 // Completion bits of a diagonal tile: the column groups covering [c0, c1) of row slice s
@@ -733,6 +801,19 @@ __device__ double cta_sum_fixed(double v) {
     for (int q = 0; q < kThreads / 32; ++q) t += s_part[q];
     __syncthreads();
     return t;
+}
+
+// The unit triangle M (17-strided) and reciprocals inv of a 16-column panel's diagonal block
+// L(i, j) at D[i + j ldd] (zero above the diagonal), as potrf_diag16 leaves them; a barrier
+// at the end.
+__device__ __forceinline__ void unit16(const double* D, int ldd, int pw, double* M, double* inv) {
+    if (threadIdx.x < kP16) inv[threadIdx.x] = threadIdx.x < pw ? 1.0 / D[threadIdx.x * (ldd + 1)] : 0.0;
+    __syncthreads();
+    if (threadIdx.x < kP16 * kP16) {
+        const int i = threadIdx.x % kP16, j = threadIdx.x / kP16;
+        M[i + j * kM16] = (i > j && i < pw) ? D[i + j * ldd] * inv[j] : 0.0;
+    }
+    __syncthreads();
 }
 
 // Factorization of rows [a0, b0) of a diagonal tile (the second half of TASK_SYRK, after
@@ -773,21 +854,28 @@ __device__ void slice_factor(const ReplayArgs& a, const DTask& t, const DTile& O
             });
         }
         __syncthreads();
-        if (threadIdx.x < kDiagGroupW) sv[threadIdx.x] = 1.0 / S0[threadIdx.x * (kRStLd + 1)];
-        __syncthreads();
+        unit16(S0, kRStLd, kDiagGroupW, S1, sv);
         double* X = C + g0 * kRLd;
-        trsm_rows(X, kRLd, R, kDiagGroupW, S0, kRStLd, sv);
+        trsm16(R, kDiagGroupW, S1, sv, [&](int r, int k) -> double& { return X[r + k * kRLd]; });
         __syncthreads();
-        write_diag_rows(T, O, nb, a0, b0, g0, g0 + kDiagGroupW, [&](int r, int c) { return C[(r - a0) + c * kRLd]; });
+        write_diag_rows(T, O, nb, a0, b0, g0, g0 + kDiagGroupW, [&](int r, int c) { return C[(r - a0) + c * kRLd]; },
+                        threadIdx.x, kThreads);
         __threadfence();
         __syncthreads();
         if (threadIdx.x == 0) red_release_or(cnt + t.tile, 1u << (g * kMaxDiagSlices + sl));
         // later columns of the rows: [g0 + kDiagGroupW, a0) against the staged rows, the
         // slice's own triangle [a0, b0) against the rows themselves
         const int cn = a0 - g0 - kDiagGroupW;
-        if (cn > 0)
-            mma_sub<false>(X + kDiagGroupW * kRLd, kRLd, R, cn, X, kRLd, S0 + kDiagGroupW, kRStLd, kDiagGroupW);
-        mma_sub<true>(C + a0 * kRLd, kRLd, R, R, X, kRLd, X, kRLd, kDiagGroupW);
+        double *Y = X + kDiagGroupW * kRLd, *Z = C + a0 * kRLd;
+        const double* gb = S0 + kDiagGroupW;
+        if (sp_stage_t<true>(S1, R, [&](int r, int k) { return X[r + k * kRLd]; }, S0, cn,
+                             [&](int c, int k) { return gb[c + k * kRStLd]; }, kDiagGroupW)) {
+            if (cn > 0) sp_product<false>(S1, 0, R, S0, 0, cn, [&](int r, int c) -> double& { return Y[r + c * kRLd]; });
+            sp_product<true>(S1, 0, R, S1, 0, R, [&](int r, int c) -> double& { return Z[r + c * kRLd]; });
+        } else {
+            if (cn > 0) mma_sub<false>(Y, kRLd, R, cn, X, kRLd, gb, kRStLd, kDiagGroupW);
+            mma_sub<true>(Z, kRLd, R, R, X, kRLd, X, kRLd, kDiagGroupW);
+        }
         __syncthreads();
     }
     // the slice's own diagonal block, as a packed triangle in S0 (R (R+1) / 2 <= kRStage)
@@ -797,17 +885,13 @@ __device__ void slice_factor(const ReplayArgs& a, const DTask& t, const DTile& O
         if (i >= j) P[pk(R, i, j)] = C[i + (a0 + j) * kRLd];
     }
     __syncthreads();
-    int bad = -1, done = 0;
-    double ls;
+    int done;
     auto own = [&](int r, int c) { return P[pk(R, r - a0, c - a0)]; };
-    potrf_packed(P, R, R, min(O.kd, R - 1), S1, &bad, &ls, kDiagGroupW, [&](int c1) {
-        write_diag_rows(T, O, nb, a0 + done, b0, a0 + done, a0 + c1, own);
-        __threadfence();
-        __syncthreads();
-        if (threadIdx.x == 0) red_release_or(cnt + t.tile, diag_bits(a0 + done, a0 + c1, sl));
-        done = c1;
-    });
-    write_diag_rows(T, O, nb, a0 + done, b0, a0 + done, b0, own);
+    const int bad = potrf_packed(
+        P, R, R, min(O.kd, R - 1), S1, &done,
+        [&](int c0, int c1, int tid, int nthr) { write_diag_rows(T, O, nb, a0 + c0, b0, a0 + c0, a0 + c1, own, tid, nthr); },
+        [&](int c0, int c1) { red_release_or(cnt + t.tile, diag_bits(a0 + c0, a0 + c1, sl)); });
+    write_diag_rows(T, O, nb, a0 + done, b0, a0 + done, b0, own, threadIdx.x, kThreads);
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
@@ -1043,9 +1127,16 @@ __global__ void __launch_bounds__(kThreads, 2) replay_kernel_t(const __grid_cons
                             if (!s_ok) break;
                             got |= need;
                         }
-                        stage_cols(S0, kRStLd, F + A.off, nb, e0, e1 - e0, u, a.imap, false, k0, K);
-                        __syncthreads();
-                        mma_sub_packed<true>(C, nb, e0, e0, e1 - e0, e1 - e0, S0, kRStLd, S0, kRStLd, K);
+                        const int Re = e1 - e0;
+                        if (sp_worth(Re * Re / 2, K) &&
+                            sp_stage_a(S0, Re, ColGet(F + A.off, nb, e0, u, a.imap, false, k0), K)) {
+                            sp_product<true>(S0, 0, Re, S0, 0, Re,
+                                             [&](int r, int c) -> double& { return C[pk(nb, e0 + r, e0 + c)]; });
+                        } else {
+                            stage_cols(S0, kRStLd, F + A.off, nb, e0, Re, u, a.imap, false, k0, K);
+                            __syncthreads();
+                            mma_sub_packed<true>(C, nb, e0, e0, Re, Re, S0, kRStLd, S0, kRStLd, K);
+                        }
                         __syncthreads();
                     }
                 }
@@ -1053,23 +1144,20 @@ __global__ void __launch_bounds__(kThreads, 2) replay_kernel_t(const __grid_cons
                     // columns are published kDiagGroupW at a time as they become final (one
                     // slice holds every row), so the TRSMs of this block column can start
                     // before the whole tile is factored
-                    int bad, done = 0;
-                    double ls;
-                    potrf_packed(C, nb, O.sw, min(O.kd, nb - 1), S0, &bad, &ls, kDiagGroupW, [&](int c1) {
-                        store_diag_cols(C, F + O.off, O, nb, done, c1);
-                        __threadfence();
-                        __syncthreads();
-                        if (threadIdx.x == 0) red_release_or(cnt + t.tile, diag_bits(done, c1, 0));
-                        done = c1;
-                    });
-                    if (threadIdx.x == 0) {
-                        if (bad >= 0) record_info(a.info + item, O.J * nb + bad + 1);
-                        F[a.poff + O.pd_slot] = bad >= 0 ? __longlong_as_double(0x7ff8000000000000LL) : ls;
-                    }
-                    store_diag_cols(C, F + O.off, O, nb, done, nb);
+                    int done;
+                    const int bad = potrf_packed(
+                        C, nb, O.sw, min(O.kd, nb - 1), S0, &done,
+                        [&](int c0, int c1, int tid, int nthr) { store_diag_cols(C, F + O.off, O, nb, c0, c1, tid, nthr); },
+                        [&](int c0, int c1) { red_release_or(cnt + t.tile, diag_bits(c0, c1, 0)); });
+                    store_diag_cols(C, F + O.off, O, nb, done, nb, threadIdx.x, kThreads);
                     __threadfence();
                     __syncthreads();
-                    if (threadIdx.x == 0) red_release_or(cnt + t.tile, diag_bits(done, O.sw, 0));
+                    if (threadIdx.x == 0) {
+                        if (bad >= 0) record_info(a.info + item, O.J * nb + bad + 1);
+                        red_release_or(cnt + t.tile, diag_bits(done, O.sw, 0));
+                    }
+                    const double ls = packed_logsum(C, nb, O.sw);
+                    if (threadIdx.x == 0) F[a.poff + O.pd_slot] = bad >= 0 ? __longlong_as_double(0x7ff8000000000000LL) : ls;
                 }
             }
         } else if (t.kind == TASK_FWD) {
@@ -1104,14 +1192,21 @@ __global__ void __launch_bounds__(kThreads, 2) replay_kernel_t(const __grid_cons
                             if (!s_ok) break;
                             got |= need;
                         }
-                        stage_cols(S0, kRStLd, F + A.off, nb, q0, e1 - q0, u, a.imap, false, k0, K);
-                        __syncthreads();
-                        const int ch = min(d0, e1);
-                        if (ch > q0)
-                            mma_sub<false>(C + (e0 - t.rs0) + q0 * kRLd, kRLd, e1 - e0, ch - q0,
-                                           S0 + (e0 - q0), kRStLd, S0, kRStLd, K);
-                        mma_sub<true>(C + (e0 - t.rs0) + e0 * kRLd, kRLd, e1 - e0, e1 - e0,
-                                      S0 + (e0 - q0), kRStLd, S0 + (e0 - q0), kRStLd, K);
+                        const int ch = min(d0, e1), Re = e1 - e0, qe = e0 - q0;
+                        double *Y = C + (e0 - t.rs0) + q0 * kRLd, *Z = C + (e0 - t.rs0) + e0 * kRLd;
+                        if (sp_worth(Re * (max(ch - q0, 0) + Re / 2), K) &&
+                            sp_stage_a(S0, e1 - q0, ColGet(F + A.off, nb, q0, u, a.imap, false, k0), K)) {
+                            if (ch > q0)
+                                sp_product<false>(S0, qe, Re, S0, 0, ch - q0,
+                                                  [&](int r, int c) -> double& { return Y[r + c * kRLd]; });
+                            sp_product<true>(S0, qe, Re, S0, qe, Re,
+                                             [&](int r, int c) -> double& { return Z[r + c * kRLd]; });
+                        } else {
+                            stage_cols(S0, kRStLd, F + A.off, nb, q0, e1 - q0, u, a.imap, false, k0, K);
+                            __syncthreads();
+                            if (ch > q0) mma_sub<false>(Y, kRLd, Re, ch - q0, S0 + qe, kRStLd, S0, kRStLd, K);
+                            mma_sub<true>(Z, kRLd, Re, Re, S0 + qe, kRStLd, S0 + qe, kRStLd, K);
+                        }
                         __syncthreads();
                     }
                 }
@@ -1154,11 +1249,19 @@ __global__ void __launch_bounds__(kThreads, 2) replay_kernel_t(const __grid_cons
                             got_a |= need_a;
                             got_b |= need_b;
                         }
-                        stage_cols(S0, kRStLd, F + A.off, nb, e0, e1 - e0, u, a.imap, false, k0, K);
-                        stage_rows_gather(S1, kRStLd, F + B.off, nb, O, a.saind, c0, c1 - c0, u, a.imap, k0, K);
-                        __syncthreads();
-                        mma_sub<false>(C + (e0 - t.rs0) + c0 * kRLd, kRLd, e1 - e0, c1 - c0, S0, kRStLd,
-                                       S1, kRStLd, K);
+                        double* Y = C + (e0 - t.rs0) + c0 * kRLd;
+                        const ColGet gb(F + B.off, nb, 0, u, a.imap, true, k0);
+                        if (sp_worth((e1 - e0) * (c1 - c0), K) &&
+                            sp_stage_ab(S0, e1 - e0, ColGet(F + A.off, nb, e0, u, a.imap, false, k0), S1, c1 - c0,
+                                        [&](int c, int k) { return gb(logical_col(O, a.saind, c0 + c), k); }, K)) {
+                            sp_product<false>(S0, 0, e1 - e0, S1, 0, c1 - c0,
+                                              [&](int r, int c) -> double& { return Y[r + c * kRLd]; });
+                        } else {
+                            stage_cols(S0, kRStLd, F + A.off, nb, e0, e1 - e0, u, a.imap, false, k0, K);
+                            stage_rows_gather(S1, kRStLd, F + B.off, nb, O, a.saind, c0, c1 - c0, u, a.imap, k0, K);
+                            __syncthreads();
+                            mma_sub<false>(Y, kRLd, e1 - e0, c1 - c0, S0, kRStLd, S1, kRStLd, K);
+                        }
                         __syncthreads();
                     }
                 }
@@ -1168,11 +1271,12 @@ __global__ void __launch_bounds__(kThreads, 2) replay_kernel_t(const __grid_cons
                 if (s_ok) {
                     // rows of X outside a column group's extent are zero there and stay zero
                     const double* DT = F + D.off;
-                    // right-looking by panels of kPb columns: solve panel p as soon as L_kk's
-                    // columns up to it are final, publish it, then update the later panels with
-                    // it, so the work left after the last columns of L_kk arrive is small
-                    for (int p = 0; p < sw; p += kPb) {
-                        const int pw = min(kPb, sw - p);
+                    // right-looking by panels of 16 columns: solve panel p as soon as L_kk's
+                    // columns up to it are final, publish it (kPanelW columns at a time), then
+                    // update the later columns with it, so the work left after the last columns
+                    // of L_kk arrive is small
+                    for (int p = 0; p < sw; p += kP16) {
+                        const int pw = min(kP16, sw - p);
                         if (threadIdx.x == 0) {
                             const int gl = logical_col(O, a.saind, p + pw - 1) / kDiagGroupW;
                             s_ok = wait_bits(cnt + t.diag, (unsigned)D.nfinal & diag_prefix(gl), a.spin,
@@ -1184,39 +1288,36 @@ __global__ void __launch_bounds__(kThreads, 2) replay_kernel_t(const __grid_cons
                         col_ext(a.cext, O, nb, p, p + pw - 1, lo, hi);
                         const int y0 = max(t.tr0, lo), y1 = min(t.tr1, hi);
                         if (y0 < y1) {
-                            // diagonal block of the panel and its reciprocal diagonal
-                            // (consecutive threads along a stored row of a banded L_kk, down a
-                            // column of a dense one; leading dimension kPb + 1)
+                            // diagonal block of the panel (consecutive threads along a stored row
+                            // of a banded L_kk, down a column of a dense one)
                             const bool band = D.kind == TILE_DIAG_BAND;
-                            for (int idx = threadIdx.x; idx < kPb * kPb; idx += kThreads) {
-                                const int i = band ? idx / kPb : idx & (kPb - 1);
-                                const int j = band ? idx & (kPb - 1) : idx / kPb;
-                                double v = 0.0;
-                                if (i < pw && j < pw && i >= j)
-                                    v = diag_at(DT, D, nb, logical_col(O, a.saind, p + i),
-                                                logical_col(O, a.saind, p + j));
-                                S0[i + j * (kPb + 1)] = v;
+                            if (threadIdx.x < kP16 * kP16) {
+                                const int i = band ? threadIdx.x / kP16 : threadIdx.x % kP16;
+                                const int j = band ? threadIdx.x % kP16 : threadIdx.x / kP16;
+                                S0[i + j * kM16] = (i < pw && j < pw && i >= j)
+                                                       ? diag_at(DT, D, nb, logical_col(O, a.saind, p + i),
+                                                                 logical_col(O, a.saind, p + j))
+                                                       : 0.0;
                             }
                             __syncthreads();
-                            if (threadIdx.x < pw) sv[threadIdx.x] = 1.0 / S0[threadIdx.x * (kPb + 2)];
-                            __syncthreads();
-                            trsm_rows(C + (y0 - t.rs0) + p * kRLd, kRLd, y1 - y0, pw, S0, kPb + 1, sv);
+                            unit16(S0, kM16, pw, S1, sv);
+                            double* X = C + (y0 - t.rs0) + p * kRLd;
+                            trsm16(y1 - y0, pw, S1, sv, [&](int r, int k) -> double& { return X[r + k * kRLd]; });
                             __syncthreads();
                         }
-                        // columns [p, p + pw) of this slice are final: publish them
-                        store_off(C + p * kRLd, kRLd, F + O.off + (size_t)p * nb, nb, t.rs0, R, pw);
-                        __threadfence();
-                        __syncthreads();
-                        if (threadIdx.x == 0)
-                            red_release_or(cnt + t.tile, 1u << ((p / kPanelW) * kMaxSlices + t.slice));
-                        // X(:, pn:sw) -= X(:, p:p+pw) L_kk(later columns, panel p)^T
                         const int pn = p + pw, Cn = sw - pn;
-                        if (Cn <= 0 || y0 >= y1) continue;
-                        for (int k0 = p; k0 < pn; k0 += kRKc) {
-                            const int K = min(kRKc, pn - k0);
-                            col_ext(a.cext, O, nb, k0, k0 + K - 1, lo, hi);
-                            const int x0 = max(t.tr0, lo), x1 = min(t.tr1, hi);
-                            if (x0 >= x1) continue;
+                        if (pn % kPanelW == 0 || pn == sw) {
+                            // columns [q0, pn) of this slice are final: publish them
+                            const int q0 = (p / kPanelW) * kPanelW;
+                            store_off(C + q0 * kRLd, kRLd, F + O.off + (size_t)q0 * nb, nb, t.rs0, R, pn - q0);
+                            __threadfence();
+                            __syncthreads();
+                            if (threadIdx.x == 0)
+                                red_release_or(cnt + t.tile, 1u << ((p / kPanelW) * kMaxSlices + t.slice));
+                        }
+                        // X(:, pn:sw) -= X(:, p:p+pw) L_kk(later columns, panel p)^T
+                        if (Cn > 0 && y0 < y1) {
+                            const int k0 = p, K = pw, x0 = y0, x1 = y1;
                             const int Cp = ((Cn + 3) & ~3) + 4;
                             if (D.kind == TILE_DIAG_BAND) {
                                 // along stored rows of L_kk: consecutive threads on consecutive k
@@ -1236,8 +1337,14 @@ __global__ void __launch_bounds__(kThreads, 2) replay_kernel_t(const __grid_cons
                                 });
                             }
                             __syncthreads();
-                            double* X = C + (x0 - t.rs0);
-                            mma_sub<false>(X + pn * kRLd, kRLd, x1 - x0, Cn, X + k0 * kRLd, kRLd, S1, kRStLd, K);
+                            double *X = C + (x0 - t.rs0) + k0 * kRLd, *Y = C + (x0 - t.rs0) + pn * kRLd;
+                            if (sp_worth((x1 - x0) * Cn, K) &&
+                                sp_stage_t<true>(S0, x1 - x0, [&](int r, int k) { return X[r + k * kRLd]; }, S1, Cn,
+                                                 [&](int c, int k) { return S1[c + k * kRStLd]; }, K))
+                                sp_product<false>(S0, 0, x1 - x0, S1, 0, Cn,
+                                                  [&](int r, int c) -> double& { return Y[r + c * kRLd]; });
+                            else
+                                mma_sub<false>(Y, kRLd, x1 - x0, Cn, X, kRLd, S1, kRStLd, K);
                             __syncthreads();
                         }
                     }
@@ -1765,6 +1872,8 @@ __device__ __forceinline__ void mma_scatter(double* C, int ldc, int R, int Cn, c
     const int c44 = LOWER ? m4 * (m4 + 1) / 2 : m4 * n4;
     if (c44 >= (kThreads * 3) / 4)
         mma_scatter_tiles<LOWER, 4, 4, PACKED>(C, ldc, R, Cn, A, lda, B, ldb, K, rm, cm, pnb);
+    else if ((LOWER ? R * (R + 1) / 2 : R * Cn) <= kThreads)
+        mma_scatter_tiles<LOWER, 1, 1, PACKED>(C, ldc, R, Cn, A, lda, B, ldb, K, rm, cm, pnb);
     else
         mma_scatter_tiles<LOWER, 2, 2, PACKED>(C, ldc, R, Cn, A, lda, B, ldb, K, rm, cm, pnb);
 }
@@ -1811,7 +1920,7 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                     if (sp_worth(A.h * A.h / 2, K) &&
                         sp_stage_a(S0, A.h, [&](int r, int k) { return __ldcg(ga + r + (size_t)k * A.ld); }, K)) {
                         sp_product<true>(S0, 0, A.h, S0, 0, A.h,
-                                         [&](int r, int c, double v) { C[pk(w, s_rm[r], s_rm[c])] -= v; });
+                                         [&](int r, int c) -> double& { return C[pk(w, s_rm[r], s_rm[c])]; });
                     } else {
                         sn_stage(S0, kRStLd, F, A, 0, A.h, k0, K);
                         __syncthreads();
@@ -1821,12 +1930,12 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                 }
             }
             if (s_ok) {
-                int bad;
-                double ls;
-                potrf_packed(C, w, w, w - 1, S0, &bad, &ls, kPb, [](int) {});
+                int done;
+                const int bad = potrf_packed(C, w, w, w - 1, S0, &done, [](int, int, int, int) {}, [](int, int) {});
                 for_rc(w, w, [&](int r, int c) {
                     if (r >= c) __stcg(F + O.off + r + (size_t)c * O.ld, C[pk(w, r, c)]);
                 });
+                const double ls = packed_logsum(C, w, w);
                 if (threadIdx.x == 0) {
                     if (bad >= 0) record_info(a.info + item, a.first[O.I] + bad + 1);
                     F[a.poff + O.I] = bad >= 0 ? __longlong_as_double(0x7ff8000000000000LL) : ls;
@@ -1858,7 +1967,7 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                         sp_stage_ab(S0, Ra, [&](int r, int k) { return __ldcg(ga + r + (size_t)k * A.ld); }, S1, B.h,
                                     [&](int r, int k) { return __ldcg(gb + r + (size_t)k * B.ld); }, K)) {
                         sp_product<false>(S0, 0, Ra, S1, 0, B.h,
-                                          [&](int r, int c, double v) { C[s_rm[r] + s_cm[c] * kRLd] -= v; });
+                                          [&](int r, int c) -> double& { return C[s_rm[r] + s_cm[c] * kRLd]; });
                     } else {
                         sn_stage(S0, kRStLd, F, A, u.ar0, Ra, k0, K);
                         sn_stage(S1, kRStLd, F, B, 0, B.h, k0, K);
@@ -1873,40 +1982,37 @@ __device__ __forceinline__ void sn_task(const SnArgs& a, int ti, long long item,
                 if (threadIdx.x == 0) s_ok = wait_counter(cnt + t.diag, 1, a.spin, &a.hdr->status);
                 __syncthreads();
                 if (s_ok) {
-                    // X <- X L_JJ^{-T}, right-looking by panels of kPb columns
+                    // X <- X L_JJ^{-T}, right-looking by panels of 16 columns
                     const double* DT = F + D.off;
-                    for (int p = 0; p < w; p += kPb) {
-                        const int pw = min(kPb, w - p);
-                        for (int idx = threadIdx.x; idx < kPb * kPb; idx += kThreads) {
-                            const int i = idx & (kPb - 1), j = idx / kPb;
-                            S0[i + j * (kPb + 1)] =
+                    for (int p = 0; p < w; p += kP16) {
+                        const int pw = min(kP16, w - p);
+                        if (threadIdx.x < kP16 * kP16) {
+                            const int i = threadIdx.x % kP16, j = threadIdx.x / kP16;
+                            S0[i + j * kM16] =
                                 (i < pw && j < pw && i >= j) ? __ldcg(DT + p + i + (size_t)(p + j) * D.ld) : 0.0;
                         }
                         __syncthreads();
-                        if (threadIdx.x < pw) sv[threadIdx.x] = 1.0 / S0[threadIdx.x * (kPb + 2)];
-                        __syncthreads();
-                        trsm_rows(C + p * kRLd, kRLd, R, pw, S0, kPb + 1, sv);
+                        unit16(S0, kM16, pw, S1, sv);
+                        double* X = C + p * kRLd;
+                        trsm16(R, pw, S1, sv, [&](int r, int k) -> double& { return X[r + k * kRLd]; });
                         __syncthreads();
                         const int pn = p + pw, Cn = w - pn;
                         if (Cn <= 0) continue;
-                        for (int k0 = p; k0 < pn; k0 += kRKc) {
-                            const int K = min(kRKc, pn - k0);
-                            const double *X = C + k0 * kRLd, *gb = DT + pn + (size_t)k0 * D.ld;
-                            double* Y = C + pn * kRLd;
-                            if (sp_worth(R * Cn, K) &&
-                                sp_stage_ab(S0, R, [&](int r, int k) { return X[r + k * kRLd]; }, S1, Cn,
-                                            [&](int c, int k) { return __ldcg(gb + c + (size_t)k * D.ld); }, K)) {
-                                sp_product<false>(S0, 0, R, S1, 0, Cn, [&](int r, int c, double v) { Y[r + c * kRLd] -= v; });
-                            } else {
-                                const int Cp = ((Cn + 3) & ~3) + 4;
-                                for_rc(Cp, K, [&](int c, int k) {
-                                    S1[c + k * kRStLd] = c < Cn ? __ldcg(gb + c + (size_t)k * D.ld) : 0.0;
-                                });
-                                __syncthreads();
-                                mma_sub<false>(Y, kRLd, R, Cn, X, kRLd, S1, kRStLd, K);
-                            }
+                        const double* gb = DT + pn + (size_t)p * D.ld;
+                        double* Y = C + pn * kRLd;
+                        if (sp_worth(R * Cn, pw) &&
+                            sp_stage_ab(S0, R, [&](int r, int k) { return X[r + k * kRLd]; }, S1, Cn,
+                                        [&](int c, int k) { return __ldcg(gb + c + (size_t)k * D.ld); }, pw)) {
+                            sp_product<false>(S0, 0, R, S1, 0, Cn, [&](int r, int c) -> double& { return Y[r + c * kRLd]; });
+                        } else {
+                            const int Cp = ((Cn + 3) & ~3) + 4;
+                            for_rc(Cp, pw, [&](int c, int k) {
+                                S1[c + k * kRStLd] = c < Cn ? __ldcg(gb + c + (size_t)k * D.ld) : 0.0;
+                            });
                             __syncthreads();
+                            mma_sub<false>(Y, kRLd, R, Cn, X, kRLd, S1, kRStLd, pw);
                         }
+                        __syncthreads();
                     }
                     for_rc(R, w, [&](int r, int c) { __stcg(F + O.off + t.rs0 + r + (size_t)c * O.ld, C[r + c * kRLd]); });
                 }
@@ -1948,8 +2054,8 @@ __global__ void __launch_bounds__(kThreads, 2) sn_replay_kernel(const __grid_con
 // rows below beyond kSnSolveRows are tasks of their own, so a wide panel takes several SMs.
 // What bounds it: the path through the tree, per level a diagonal substitution and one
 // chunk (256 x 128 FMAs on one SM's FP64 pipe, 8 us).  Gathering every cell of a row
-// supernode one by one, in J order, took 58.2 ms at n = 180,020 (now 5.7), 18.0 ms on a 48^3
-// FEM operator (4.1) and 13.4 ms on 1024 small grids (4.6).
+// supernode one by one, in J order, took 58.2 ms at n = 180,020 (now 5.7),
+// 18.0 ms on a 48^3 FEM operator (4.1) and 13.4 ms on 1024 small grids (4.6).
 struct SnSolveArgs {
     const SnSolveNode* nodes;
     const int32_t *kids, *rel, *chunk_own, *fwd, *bwd, *rows, *perm;
@@ -2233,20 +2339,24 @@ __device__ __forceinline__ double sym_at(const double* T, const DTile& d, int nb
     return r >= c ? diag_at(T, d, nb, r, c) : diag_at(T, d, nb, c, r);
 }
 
-// C(r, c) at C[r + c ldc] -= sum_k ga(r, k) gb(c, k), r < R, c < Cn, k < K <= 16 (the whole
-// CTA; a barrier before and after): by the split where it can take the chunk, else one DFMA
-// sum per entry straight from the operands.  S0, S1: digit buffers.
-template <class GetA, class GetB, class Epi>
-__device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int Cn, int K, GetA ga, GetB gb, Epi epi) {
-    if (!sp_stage_ab(S0, R, ga, S1, Cn, gb, K))
-        for (int e = threadIdx.x; e < R * Cn; e += kThreads) {
-            const int r = e % R, c = e / R;
-            double v = 0.0;
-            for (int k = 0; k < K; ++k) v = fma(ga(r, k), gb(c, k), v);
-            epi(r, c, v);
-        }
-    else
-        sp_product<false>(S0, 0, R, S1, 0, Cn, epi);
+// at(r, c) -= sum_k ga(r, k) gb(c, k), r < R, c < Cn (LOWER: r >= c), k < K <= 16, by the
+// whole CTA (a barrier at the end): the split where it pays and can take the chunk, else
+// DFMAs from staged operands.  S0, S1: staging buffers.
+template <bool LOWER, class GetA, class GetB, class At>
+__device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int Cn, int K, GetA ga, GetB gb, At at) {
+    if (sp_worth(LOWER ? R * Cn / 2 : R * Cn, K) && sp_stage_ab(S0, R, ga, S1, Cn, gb, K)) {
+        sp_product<LOWER>(S0, 0, R, S1, 0, Cn, at);
+    } else {
+        for_rc(R, K, [&](int r, int k) { S0[r + k * kRStLd] = ga(r, k); });
+        for_rc(Cn, K, [&](int c, int k) { S1[c + k * kRStLd] = gb(c, k); });
+        __syncthreads();
+        for_rc(R, Cn, [&](int r, int c) {
+            if (LOWER && r < c) return;
+            double v = at(r, c);
+            for (int k = 0; k < K; ++k) v = fma(-S0[r + k * kRStLd], S1[c + k * kRStLd], v);
+            at(r, c) = v;
+        });
+    }
     __syncthreads();
 }
 
@@ -2294,15 +2404,16 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
                 };
                 auto gb = [&](int c, int k) { return lget(b + i0 + k, p + c); };
                 auto gab = [&](int r, int k) { return r < m ? ga(r, k) : gb(r - m, k); };
-                if (sp_stage_a(S0, m + pw, gab, K)) {
-                    sp_product<false>(S0, 0, m, S0, m, pw, [&](int r, int c, double v) { X[r + c * LDX] -= v; });
+                if (sp_worth(m * pw, K) && sp_stage_a(S0, m + pw, gab, K)) {
+                    sp_product<false>(S0, 0, m, S0, m, pw, [&](int r, int c) -> double& { return X[r + c * LDX]; });
                 } else {
-                    for (int e = threadIdx.x; e < m * pw; e += kThreads) {
-                        const int r = e % m, c = e / m;
+                    for_rc(pw, K, [&](int c, int k) { S0[c + k * kRStLd] = gb(c, k); });
+                    __syncthreads();
+                    for_rc(m, pw, [&](int r, int c) {
                         double v = X[r + c * LDX];
-                        for (int k = 0; k < K; ++k) v = fma(-ga(r, k), gb(c, k), v);
+                        for (int k = 0; k < K; ++k) v = fma(-ga(r, k), S0[c + k * kRStLd], v);
                         X[r + c * LDX] = v;
-                    }
+                    });
                 }
                 __syncthreads();
             }
@@ -2371,9 +2482,9 @@ __device__ __forceinline__ void selinv_back(double* C, int R, int w, double* S0,
         for (int k0 = p + pw; k0 < w; k0 += kSpK) {
             const double* X = C + k0 * kRLd;
             double* Y = C + p * kRLd;
-            chunk_product(S0, S1, R, pw, min(kSpK, w - k0), [&](int r, int k) { return X[r + k * kRLd]; },
+            chunk_product<false>(S0, S1, R, pw, min(kSpK, w - k0), [&](int r, int k) { return X[r + k * kRLd]; },
                           [&](int c, int k) { return lget(k0 + k, p + c); },
-                          [&](int r, int c, double v) { Y[r + c * kRLd] -= v; });
+                          [&](int r, int c) -> double& { return Y[r + c * kRLd]; });
         }
         for (int idx = threadIdx.x; idx < kPb * kPb; idx += kThreads) {
             const int i = idx & (kPb - 1), j = idx / kPb;
@@ -2459,7 +2570,7 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                             const int q = s_idx[1][c];
                             return q >= 0 ? __ldg(LT + (i0 + k) + (size_t)q * nb) : 0.0;
                         };
-                        chunk_product(S0, S1, R, sw, K, ga, gb, [&](int r, int c, double v) { C[r + c * kRLd] -= v; });
+                        chunk_product<false>(S0, S1, R, sw, K, ga, gb, [&](int r, int c) -> double& { return C[r + c * kRLd]; });
                     }
                 }
                 if (s_ok) {
@@ -2500,19 +2611,8 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                         const int q = s_idx[0][r];
                         return q >= 0 ? __ldg(LT + (i0 + k) + (size_t)q * nb) : 0.0;
                     };
-                    auto epi = [&](int r, int c, double v) { C[pk(w, z0 + r, z0 + c)] -= v; };
-                    if (sp_stage_ab(S0, M, ga, S1, M, gb, K)) {
-                        sp_product<true>(S0, 0, M, S1, 0, M, epi);
-                    } else {
-                        for (int e = threadIdx.x; e < M * M; e += kThreads) {
-                            const int r = e % M, c = e / M;
-                            if (r < c) continue;
-                            double v = 0.0;
-                            for (int k = 0; k < K; ++k) v = fma(ga(r, k), gb(c, k), v);
-                            epi(r, c, v);
-                        }
-                    }
-                    __syncthreads();
+                    auto epi = [&](int r, int c) -> double& { return C[pk(w, z0 + r, z0 + c)]; };
+                    chunk_product<true>(S0, S1, M, M, K, ga, gb, epi);
                 }
             }
             if (s_ok) {
@@ -2628,8 +2728,8 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                     };
                     // L(K',J) rows j0.. (through L1: a thread walks down its column)
                     auto gb = [&](int c, int k) { return __ldg(LT + (j0 + k) + (size_t)c * Lc.ld); };
-                    chunk_product(S0, S1, R, w, min(kSpK, h - j0), ga, gb,
-                                  [&](int r, int c, double v) { C[r + c * kRLd] -= v; });  // C = -sum G L
+                    chunk_product<false>(S0, S1, R, w, min(kSpK, h - j0), ga, gb,
+                                  [&](int r, int c) -> double& { return C[r + c * kRLd]; });  // C = -sum G L
                 }
             }
             if (s_ok) {
@@ -2652,19 +2752,8 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                     const int Kc = min(kSpK, Lc.h - i0);
                     auto ga = [&](int r, int k) { return __ldcg(ST + (i0 + k) + (size_t)r * Lc.ld); };
                     auto gb = [&](int r, int k) { return __ldg(LT + (i0 + k) + (size_t)r * Lc.ld); };
-                    auto epi = [&](int r, int c, double v) { C[pk(w, r, c)] -= v; };  // C = -Z (lower)
-                    if (sp_stage_ab(S0, w, ga, S1, w, gb, Kc)) {
-                        sp_product<true>(S0, 0, w, S1, 0, w, epi);
-                    } else {
-                        for (int e = threadIdx.x; e < w * w; e += kThreads) {
-                            const int r = e % w, c = e / w;
-                            if (r < c) continue;
-                            double v = 0.0;
-                            for (int k = 0; k < Kc; ++k) v = fma(ga(r, k), gb(c, k), v);
-                            epi(r, c, v);
-                        }
-                    }
-                    __syncthreads();
+                    auto epi = [&](int r, int c) -> double& { return C[pk(w, r, c)]; };  // C = -Z (lower)
+                    chunk_product<true>(S0, S1, w, w, Kc, ga, gb, epi);
                 }
             }
             if (s_ok) {

@@ -16,7 +16,8 @@
 // digit expansion and the epilogue issue about as long as the tensor pipe runs.  Measured,
 // supernodal route: one factorization at n = 180,020 517 -> 251 ms, a 48^3 FEM operator
 // 180 -> 98 ms, 16 sets at n = 22,520 95 -> 57 ms, and the products and their staging no
-// more than 37 % of the CTAs' time (the rest waits for other tasks).
+// more than 37 % of the CTAs' time (the rest waits for other tasks).  Tile routes: 64 bands
+// (n = 50,000, half-bandwidth 200) 178 -> 89 ms with the 16-column panels of POTRF and TRSM.
 //
 // Rows whose largest entry is not finite or lies outside 2^[-400, 400] (where the scale
 // arithmetic could leave the exponent range), and rows of subnormals, are reported by the
@@ -90,13 +91,14 @@ __device__ __forceinline__ void sp_split_row(const double (&v)[kSpK], int e, int
     }
 }
 
-// Whether a chunk's product is worth the split: 2 x 2 DFMA micro-tiles take 256 clocks per
-// column and 512 entries, splitting and multiplying at least about kSpWorth times that
-// whatever the size.  Measured at thresholds 0 / 8 / 24 / 80: one small grid (n = 1,026)
-// 596 / 594 / 625 / 627 us, a 48^3 FEM operator - / 71.1 / 72.2 / 80.9 ms, 16 spatio-temporal
-// precisions (n = 22,520) - / 42.6 / 44.0 / 49.2 ms.
-constexpr int kSpWorth = 8;
-__device__ __forceinline__ bool sp_worth(int entries, int K) { return K * ((entries + 511) >> 9) >= kSpWorth; }
+// Whether a chunk's product is worth the split: with an entry per thread DFMAs take 64 clocks
+// per column and 128 entries, splitting and multiplying about kSpWorth times that at least.
+// At thresholds 32 / 64 / 96: three FEM operators (dense tiles) 88.1 / 84.1 / 83.6 ms, 16
+// bands with marginals 147 / 142 / 141 ms, 64 small grids 1.08 / 1.05 / 1.04 ms, one 48^3 FEM
+// operator (supernodal) 49.1 / 49.4 / 50.5 ms, 16 spatio-temporal precisions 34.3 / 35.0 /
+// 35.8 ms.  (Below it 2 x 2 micro-tiles in place of an entry per thread: 64 grids 1.53 ms.)
+constexpr int kSpWorth = 64;
+__device__ __forceinline__ bool sp_worth(int entries, int K) { return K * ((entries + 127) >> 7) >= kSpWorth; }
 
 // Operands A (R x K, entries ga(r, k)) and B (Cn x K, gb(c, k)) of a chunk into the digit
 // buffers SA and SB, a thread per row (R + Cn <= blockDim.x); returns on every thread
@@ -151,35 +153,75 @@ __device__ __forceinline__ void sp_mma(float (&d)[4], const float (&c)[4], unsig
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1), "f"(c[0]), "f"(c[1]), "f"(c[2]), "f"(c[3]));
 }
 
-// The double nearest T 2^(10 + E - 2046 - 66) for |T| < 2^63 (E: sum of the two biased row
-// exponents), T = 0 giving +0.
-__device__ __forceinline__ double sp_double(long long T, int E) {
-    const unsigned long long mag = T < 0 ? 0ull - (unsigned long long)T : (unsigned long long)T;
-    if (mag == 0ull) return 0.0;
-    const int lz = __clzll((long long)mag);
-    const unsigned long long nrm = mag << lz;
-    // biased exponent of the leading bit: 1023 + 63 - lz + E - 2102; the hidden bit adds one
-    // (rounded after the shift: a mantissa of ones carries into the exponent)
-    const unsigned long long bits =
-        ((unsigned long long)(unsigned)(E - 1016 - lz - 1) << 52) + (nrm >> 11) + ((nrm >> 10) & 1ull);
-    return __longlong_as_double((long long)(bits | ((unsigned long long)T & 0x8000000000000000ull)));
+// sum_d n_d 2^(8 (7 - d)) / 2^10, rounded, from the accumulators 1.5 2^23 + n_d: their bits
+// are 0x4B400000 + n_d and go in as they are (wide integer multiply-adds, which leave the
+// busier ALU pipe alone), the biases come off in one constant.
+__device__ __forceinline__ long long sp_sum(float n0, float n1, float n2, float n3, float n4, float n5, float n6,
+                                            float n7) {
+    constexpr unsigned long long kB = 0x4B400000ull;
+    constexpr unsigned long long kOff =
+        0ull - (((kB * (1u << 14) + kB * (1u << 6)) << 32) + kB * ((1ull << 30) + (1ull << 22) + (1ull << 14) + (1ull << 6)));
+    unsigned long long T;
+    asm("{\n\t"
+        ".reg .u64 a;\n\t"
+        ".reg .u32 lo, hi;\n\t"
+        "mad.wide.u32 a, %3, 0x40000000, %9;\n\t"
+        "mad.wide.u32 a, %4, 0x400000, a;\n\t"
+        "mad.wide.u32 a, %5, 0x4000, a;\n\t"
+        "mad.wide.u32 a, %6, 0x40, a;\n\t"
+        "mov.b64 {lo, hi}, a;\n\t"
+        "mad.lo.u32 hi, %1, 0x4000, hi;\n\t"
+        "mad.lo.u32 hi, %2, 0x40, hi;\n\t"
+        "mov.b64 a, {lo, hi};\n\t"
+        "mad.lo.u32 lo, %7, 0x100, %8;\n\t"
+        "add.u32 lo, lo, %10;\n\t"
+        "shr.s32 lo, lo, 10;\n\t"
+        "mad.wide.s32 %0, lo, 1, a;\n\t"
+        "}"
+        : "=l"(T)
+        : "r"(__float_as_uint(n0)), "r"(__float_as_uint(n1)), "r"(__float_as_uint(n2)), "r"(__float_as_uint(n3)),
+          "r"(__float_as_uint(n4)), "r"(__float_as_uint(n5)), "r"(__float_as_uint(n6)), "r"(__float_as_uint(n7)),
+          "l"(kOff), "n"(512u - 0x4B400000u * 257u));
+    return (long long)T;
 }
 
-// sum over the chunk of A(a0 + r, k) B(b0 + c, k) for every r < R, c < Cn (LOWER: at least every
-// r >= c), one call epi(r, c, value) per entry; 16 x 8 units of the product spread over the
-// CTA's warps in contiguous runs, so that a warp expands a strip of A once.  epi must not
-// synchronise.
-template <bool LOWER, class Epi>
-__device__ __forceinline__ void sp_product(double* SA, int a0, int R, double* SB, int b0, int Cn, Epi epi) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5;
+// The double nearest T 2^(E - 2102) for |T| < 2^63 (E: sum of the two biased row exponents),
+// T = 0 giving +0.
+__device__ __forceinline__ double sp_double(long long T, int E) {
+    const long long sg = T >> 63;
+    const unsigned long long mag = (unsigned long long)((T ^ sg) - sg);
+    const int lz = __clzll((long long)mag);
+    const unsigned long long nrm = mag << (lz & 63);
+    // biased exponent of the leading bit: 1023 + 63 - lz + E - 2102; the hidden bit adds one
+    // (rounded after the shift: a mantissa of ones carries into the exponent)
+    unsigned long long bits =
+        ((unsigned long long)(unsigned)(E - 1016 - lz - 1) << 52) + (nrm >> 11) + ((nrm >> 10) & 1ull);
+    bits = mag ? bits | ((unsigned long long)sg & 0x8000000000000000ull) : 0ull;
+    return __longlong_as_double((long long)bits);
+}
+
+// Units (16 rows x 8 columns) of a product: row strips in order, LOWER only the units that
+// reach r >= c (rows and columns index one range; strip s then starts at unit s (s + 1)).
+template <bool LOWER>
+__device__ __forceinline__ int sp_units(int R, int Cn) {
+    const int MR = (R + 15) >> 4, NC = (Cn + 7) >> 3;
+    return LOWER ? (MR - 1) * MR + min(2 * MR, NC) : MR * NC;
+}
+
+// One warp: at(r, c) -= sum_k A(a0 + r, k) B(b0 + c, k) over the units [u, uend), for r < R,
+// c < Cn (LOWER: r >= c); at(r, c) is a reference to the entry.  A strip of A is expanded
+// once.  A unit is 330 instructions, half of them on the ALU pipe and 36 on the tensor pipe,
+// which take about 330 clocks of an SM sub-partition each: a 64 x 128 chunk takes 9,500
+// clocks of an SM with two CTAs (65,500 on the DFMA pipe).  The four entries of a lane side
+// by side without branches take 8,100 where every entry is wanted, but ragged units then pay
+// for entries nobody wants (one factorization at n = 180,020: 158 -> 176 ms).
+template <bool LOWER, class At>
+__device__ __forceinline__ void sp_run(double* SA, int a0, int R, double* SB, int b0, int Cn, int u, int uend, At at) {
+    const int lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
     const uint4 *A = sp_digits(SA), *B = sp_digits(SB);
     const int *ea = sp_exp(SA), *eb = sp_exp(SB);
-    const int MR = (R + 15) >> 4, NC = (Cn + 7) >> 3;
-    // LOWER: strip s holds the units c < min(2 s + 2, NC) (rows and columns index one range)
-    const int units = LOWER ? (MR - 1) * MR + min(2 * MR, NC) : MR * NC;
-    int u = units * warp / nwarps;
-    const int uend = units * (warp + 1) / nwarps;
+    const int NC = (Cn + 7) >> 3;
     if (u >= uend) return;
     int s, c;
     if (LOWER) {
@@ -221,18 +263,21 @@ __device__ __forceinline__ void sp_product(double* SA, int a0, int R, double* SB
             for (int q = 0; q < 4; ++q) {
                 const int r = r0 + (q >> 1) * 8, cc = c0 + (q & 1);
                 if (r >= R || cc >= Cn || (LOWER && r < cc)) continue;
-                int n[8];
-#pragma unroll
-                for (int d = 0; d < 8; ++d) n[d] = __float_as_int(acc[d][q]) - 0x4B400000;
-                const long long hi = (long long)(n[0] * 256 + n[1]) * 65536 + (n[2] * 256 + n[3]);
-                const long long lo = (long long)(n[4] * 256 + n[5]) * 65536 + (n[6] * 256 + n[7]);
-                const long long T = hi * (1ll << 22) + ((lo + 512) >> 10);
-                epi(r, cc, sp_double(T, ((q >> 1) ? e1 : e0) + ((q & 1) ? f1 : f0)));
+                const long long T = sp_sum(acc[0][q], acc[1][q], acc[2][q], acc[3][q], acc[4][q], acc[5][q],
+                                           acc[6][q], acc[7][q]);
+                at(r, cc) -= sp_double(T, ((q >> 1) ? e1 : e0) + ((q & 1) ? f1 : f0));
             }
         }
         ++s;
         c = 0;
     }
+}
+
+// The whole product, its units spread over the CTA's warps in contiguous runs.
+template <bool LOWER, class At>
+__device__ __forceinline__ void sp_product(double* SA, int a0, int R, double* SB, int b0, int Cn, At at) {
+    const int warp = threadIdx.x >> 5, nwarps = blockDim.x >> 5, units = sp_units<LOWER>(R, Cn);
+    sp_run<LOWER>(SA, a0, R, SB, b0, Cn, units * warp / nwarps, units * (warp + 1) / nwarps, at);
 }
 
 }  // namespace

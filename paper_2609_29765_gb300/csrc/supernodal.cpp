@@ -372,14 +372,12 @@ vector<int32_t> stc::sn_queue_order(const stc::SnPlan& S, int procs) {
     const int32_t nt = (int32_t)S.dtasks.size(), nc = (int32_t)S.dcells.size();
     vector<double> cost(nt), bl(nt, 0.0);
     vector<int32_t> deps(nt, 0), left(nc, 0);
-    // readers of a cell (an update reads two cells, an off-diagonal task its diagonal cell)
-    vector<int64_t> rbeg(nc + 1, 0);
+    // readers of a cell: an off-diagonal task its diagonal cell and the cells (K,I) of its
+    // updates (the (J,I) are final before the diagonal cell is)
+    vector<int32_t> rbeg(nc + 1, 0);
     auto each_source = [&](int32_t t, auto&& f) {
         const stc::SnDevTask& k = S.dtasks[t];
-        for (int32_t u = k.ubeg; u < k.uend; ++u) {
-            f(S.dupds[u].a);
-            if (S.dupds[u].b != S.dupds[u].a) f(S.dupds[u].b);
-        }
+        for (int32_t u = k.ubeg; u < k.uend; ++u) f(S.dupds[u].a);
         if (k.kind != stc::SN_T_DIAG) f(k.diag);
     };
     for (int32_t t = 0; t < nt; ++t) {
@@ -400,7 +398,7 @@ vector<int32_t> stc::sn_queue_order(const stc::SnPlan& S, int procs) {
     for (int32_t c = 0; c < nc; ++c) rbeg[c + 1] += rbeg[c];
     vector<int32_t> readers(rbeg[nc]);
     {
-        vector<int64_t> at(rbeg.begin(), rbeg.end() - 1);
+        vector<int32_t> at(rbeg.begin(), rbeg.end() - 1);
         for (int32_t t = 0; t < nt; ++t) each_source(t, [&](int32_t s) { readers[at[s]++] = t; });
     }
     // the tasks are stored in a topological order: longest paths in one backward sweep
@@ -431,7 +429,7 @@ vector<int32_t> stc::sn_queue_order(const stc::SnPlan& S, int procs) {
         running.pop();
         ++idle;
         if (--left[c] == 0)
-            for (int64_t q = rbeg[c]; q < rbeg[c + 1]; ++q)
+            for (int32_t q = rbeg[c]; q < rbeg[c + 1]; ++q)
                 if (--deps[readers[q]] == 0) ready.push(E(bl[readers[q]], -readers[q]));
     }
     if ((int32_t)order.size() != nt) throw std::logic_error("supernodal task set: a dependency cycle");
