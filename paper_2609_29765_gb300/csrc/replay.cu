@@ -3082,14 +3082,20 @@ int own_buffer(stc_plan* P, bool sigma, size_t bytes, void** out) {
     return STC_OK;
 }
 
-// Two CTAs per SM hide one CTA's waits behind the other's arithmetic when many items
-// are in flight; with few items every task is on the critical path and gets an SM alone.
+// Two CTAs per SM hide one CTA's staging, waits and barriers behind the other's products.
+// The tile routes take them when there is work in flight for both (items times the modelled
+// parallelism of one item's task DAG); where the chain decides, a CTA alone on its SM runs it
+// faster (one band, n = 50,000: 52.7 ms against 54.3).  The supernodal kernels and the
+// selected inverses always do: one factorization at n = 180,020 138 -> 107 ms, a 48^3 FEM
+// operator 45 -> 33 ms, one small grid unchanged.
 long long batch_total(const ReplayLaunch& L) {
     long long b = 0;
     for (int j = 0; j < L.njobs; ++j) b += L.job[j].batch;
     return b;
 }
-long long default_ctas(int sms, long long batch) { return batch >= 16 ? 2LL * sms : (long long)sms; }
+long long default_ctas(int sms, long long batch, double par) {
+    return batch >= 16 || double(batch) * par >= 64.0 ? 2LL * sms : (long long)sms;
+}
 // Grid of a persistent kernel: the plan's replay_ctas option when set (1 = serial replay
 // in queue order, the race check's reference schedule), else `dflt`; never more CTAs
 // than slots.
@@ -3179,7 +3185,7 @@ int sn_factorize_scattered(stc_plan* P, int64_t batch, void* d_factor, void* d_w
     fill_sn(a, P, d_factor, (int*)((char*)d_work + sizeof(WorkHeader)), d_info, batch, (WorkHeader*)d_work);
     a.order = batch < kSnOrderBatch ? P->sndev.order : nullptr;
     const long long total = (long long)a.ntasks * batch;
-    const int grid = grid_of(P, default_ctas(sms, batch), total);
+    const int grid = grid_of(P, 2LL * sms, total);
     sn_replay_kernel<<<grid, kThreads, kRSmemBytes, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
@@ -3231,7 +3237,7 @@ int sn_selinv(stc_plan* P, const void* d_factor, int64_t batch, void* d_sigma, v
     a.ntasks = (int)Sp.stasks.size(); a.batch = batch;
     a.spin = P->opt.spin_limit > 0 ? P->opt.spin_limit : kDefaultSpin;
     const long long total = (long long)a.ntasks * batch;
-    const int grid = grid_of(P, default_ctas(sms, batch), total);
+    const int grid = grid_of(P, 2LL * sms, total);
     sn_selinv_kernel<<<grid, kThreads, kRSmemBytes, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
@@ -3350,7 +3356,7 @@ extern "C" int stc_factorize_scattered(const stc_plan* Pc, int64_t batch, void* 
     Lc.queue = nullptr;
     Lc.hdr = (WorkHeader*)d_work;
     Lc.total = (long long)ts->tasks.size() * batch;
-    const int grid = grid_of(P, default_ctas(sms, batch_total(Lc)), Lc.total);
+    const int grid = grid_of(P, default_ctas(sms, batch_total(Lc), ts->par), Lc.total);
     replay_kernel_t<false><<<grid, kThreads, kRSmemBytes, st>>>(Lc);
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
@@ -3499,7 +3505,7 @@ extern "C" int stc_factorize_forward(const stc_plan* Pc, const double* d_values,
     Lc.queue = nullptr;
     Lc.hdr = hdr;
     Lc.total = (long long)ts->tasks.size() * batch;
-    replay_kernel_t<false><<<grid_of(P, default_ctas(sms, batch_total(Lc)), Lc.total), kThreads, kRSmemBytes, st>>>(Lc);
+    replay_kernel_t<false><<<grid_of(P, default_ctas(sms, batch_total(Lc), ts->par), Lc.total), kThreads, kRSmemBytes, st>>>(Lc);
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
 
@@ -3616,7 +3622,7 @@ extern "C" int stc_selinv(const stc_plan* Pc, const void* d_factor, int64_t batc
     a.ntasks = (int)P->stasks.size(); a.batch = batch; a.nb = (int)P->nb;
     a.spin = P->opt.spin_limit > 0 ? P->opt.spin_limit : kDefaultSpin;
     const long long total = (long long)a.ntasks * batch;
-    const int grid = grid_of(P, default_ctas(sms, batch), total);
+    const int grid = grid_of(P, 2LL * sms, total);
     selinv_kernel<<<grid, kThreads, kRSmemBytes, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
@@ -3787,7 +3793,9 @@ extern "C" int stc_factorize_group(stc_group* g, const double* const* d_values, 
     Lc.queue = g->d_queue;
     Lc.hdr = (WorkHeader*)d_work;
     Lc.total = g->total;
-    const int grid = grid_of(g->plans[0], default_ctas(sms, batch_total(Lc)), Lc.total);
+    double par = 1.0;
+    for (int p = 0; p < np; ++p) par = std::max(par, g->ts[p] ? g->ts[p]->par : 2.0 * sms);
+    const int grid = grid_of(g->plans[0], default_ctas(sms, batch_total(Lc), par), Lc.total);
     if (g->has_sn)
         replay_kernel_t<true><<<grid, kThreads, kRSmemBytes, st>>>(Lc);
     else
@@ -3837,7 +3845,7 @@ extern "C" int stc_factorize_noalloc(const stc_plan* Pc, const double* d_values,
     Lc.queue = nullptr;
     Lc.hdr = (WorkHeader*)scratch;
     Lc.total = (long long)ts->tasks.size() * batch;
-    const int grid = grid_of(P, default_ctas(sms, batch_total(Lc)), Lc.total);
+    const int grid = grid_of(P, default_ctas(sms, batch_total(Lc), ts->par), Lc.total);
     replay_kernel_t<false><<<grid, kThreads, kRSmemBytes, st>>>(Lc);
     if (cudaGetLastError() != cudaSuccess) return STC_ERR_CUDA;
     if (d_status && cudaMemcpyAsync(d_status, &Lc.hdr->status, sizeof(int32_t), cudaMemcpyDeviceToDevice, st) !=
