@@ -247,14 +247,13 @@ __device__ __forceinline__ void mma_sub_packed(double* P, int pnb, int pr0, int 
         mma_tiles<LOWER, 2, 2, true>(P, 0, R, Cn, A, lda, B, ldb, K, pnb, pr0, pc0);
 }
 
-// Forward substitution of a row block against a panel: X(r, 0:pw) <- X(r, 0:pw) D^{-T},
+// Backward substitution of a row block against a panel: X(r, 0:pw) <- X(r, 0:pw) D^{-1},
 // D lower pw x pw in shared memory (D(i,j) = D[i + j*ldd]), reciprocal diagonal dinv[].
 // TPR threads share a row: each keeps the columns j = q (mod TPR) in registers, the
 // owner of column j finishes x_j and broadcasts it by shuffle, and every thread then
-// removes x_j's contribution from its later columns (right-looking).
-template <int TPR, bool BACK>
-__device__ void trsm_rows_t(double* X, int ldx, int R, int pw, const double* D, int ldd,
-                            const double* dinv) {
+// removes x_j's contribution from its earlier columns.
+template <int TPR>
+__device__ void trsm_back_t(double* X, int ldx, int R, int pw, const double* D, int ldd, const double* dinv) {
     constexpr int NJ = kPb / TPR;
     const int q = threadIdx.x % TPR;
     const int lane = threadIdx.x & 31;
@@ -269,20 +268,17 @@ __device__ void trsm_rows_t(double* X, int ldx, int R, int pw, const double* D, 
             b[s] = (live && k < pw) ? X[rr + k * ldx] : 0.0;
         }
 #pragma unroll
-        for (int jj = 0; jj < kPb; ++jj) {
-            const int j = BACK ? kPb - 1 - jj : jj;
+        for (int j = kPb - 1; j >= 0; --j) {
             if (j < pw) {
                 const double xj = __shfl_sync(0xffffffffu, b[j / TPR] * dinv[j], base + (j % TPR));
                 if (q == j % TPR) b[j / TPR] = xj;
 #pragma unroll
                 for (int s = 0; s < NJ; ++s) {
-                    // s and j are compile-time here: register groups whose columns all lie on
-                    // the finished side of j issue no instruction (a masked DFMA still takes a
-                    // slot of the FP64 pipe)
-                    if (BACK ? s * TPR >= j : s * TPR + TPR - 1 <= j) continue;
+                    // register groups whose columns all lie on the finished side of j issue no
+                    // instruction (a masked DFMA still takes a slot of the FP64 pipe)
+                    if (s * TPR >= j) continue;
                     const int k = s * TPR + q;
-                    if (!BACK && k > j && k < pw) b[s] = fma(-xj, D[k + j * ldd], b[s]);
-                    if (BACK && k < j) b[s] = fma(-xj, D[j + k * ldd], b[s]);
+                    if (k < j) b[s] = fma(-xj, D[j + k * ldd], b[s]);
                 }
             }
         }
@@ -296,14 +292,12 @@ __device__ void trsm_rows_t(double* X, int ldx, int R, int pw, const double* D, 
     }
 }
 
-// Forward (X D^{-T}) or backward (X D^{-1}) substitution of a row block against a
-// lower pw x pw panel block D, choosing 2, 4 or 8 threads per row from the row count.
-template <bool BACK>
-__device__ __forceinline__ void trsm_rows_dir(double* X, int ldx, int R, int pw, const double* D, int ldd,
-                                              const double* dinv) {
-    if (R <= kThreads / 8) trsm_rows_t<8, BACK>(X, ldx, R, pw, D, ldd, dinv);
-    else if (R <= kThreads / 4) trsm_rows_t<4, BACK>(X, ldx, R, pw, D, ldd, dinv);
-    else trsm_rows_t<2, BACK>(X, ldx, R, pw, D, ldd, dinv);
+// 2, 4 or 8 threads per row from the row count.
+__device__ __forceinline__ void trsm_back(double* X, int ldx, int R, int pw, const double* D, int ldd,
+                                          const double* dinv) {
+    if (R <= kThreads / 8) trsm_back_t<8>(X, ldx, R, pw, D, ldd, dinv);
+    else if (R <= kThreads / 4) trsm_back_t<4>(X, ldx, R, pw, D, ldd, dinv);
+    else trsm_back_t<2>(X, ldx, R, pw, D, ldd, dinv);
 }
 
 struct SnArgs {
@@ -2363,18 +2357,53 @@ __device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int
     __syncthreads();
 }
 
+// The inverses W = L_pp^{-1} of the 16 x 16 diagonal blocks of a w x w triangle (w <=
+// kSelWMax) behind the packed triangle in C, panel q at C + w (w + 1) / 2 + 272 q, entry
+// (i, l) at i + 17 l: they need L only and are made before the first wait.  A column per lane
+// of a half-warp.
+constexpr int kSelWMax = 112;
+static_assert(kSelWMax * (kSelWMax + 1) / 2 + (kSelWMax / 16) * 272 <= kRCbuf, "the inverses fit behind the triangle");
+template <class LGet>
+__device__ void selinv_inverses(double* C, int w, LGet lget) {
+    double* Wb = C + w * (w + 1) / 2;
+    const int np = (w + 15) / 16;
+    for (int e = threadIdx.x; e < np * 256; e += kThreads) {
+        const int q = e >> 8, i = e & 15, l = (e >> 4) & 15, p = 16 * q, pw = min(16, w - p);
+        Wb[q * 272 + i + 17 * l] = (i < pw && l <= i) ? lget(p + i, p + l) : (i == l ? 1.0 : 0.0);
+    }
+    __syncthreads();
+    const int l = threadIdx.x & 15, q = threadIdx.x >> 4;  // np <= 7 < 16 half-warps
+    if (q < ((np + 1) & ~1)) {
+        const double* M = Wb + min(q, np - 1) * 272;
+        double x[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+            double t = i == l ? 1.0 : 0.0;
+#pragma unroll
+            for (int k = 0; k < i; ++k) t = fma(-M[i + 17 * k], x[k], t);
+            x[i] = t / M[i + 17 * i];
+        }
+        __syncwarp();
+        if (q < np)
+#pragma unroll
+            for (int i = 0; i < 16; ++i) Wb[q * 272 + i + 17 * l] = i >= l ? x[i] : 0.0;
+    }
+    __syncthreads();
+}
+
 // Diagonal block of a selected inverse.  P holds -Z (packed lower triangle of width w) and
 // becomes Sigma:
 //   Sigma_rc = (-Z_rc - sum_{i>c} Sigma_ri L_ic) / L_cc              (r > c)
 //   Sigma_cc = 1/L_cc^2 + (-Z_cc - sum_{i>c} L_ic Sigma_ic) / L_cc
 // by panels of 16 columns from the right: the rows below a panel take the products with the
 // columns already done (chunk products of the symmetric part) and a triangular solve, the
-// panel's own 16 x 16 block the products with those rows and the element recurrence on one
-// warp.  One column at a time over the whole block (two barriers and a dot product of up to
-// w terms per column) was most of a diagonal task; a whole selected inverse
-// of 64 value sets at n = 4,020 went 35.5 -> 21.4 ms with this and the split products, of 16
-// bands (n = 50,000, half-bandwidth 20) 115 -> 101 ms.  Rows more than kd below the diagonal are outside the
-// band and left alone.  lget(i, c): L_ic, i >= c.  S0: digits; S1: digits, then the panel's
+// panel's own 16 x 16 block the products with those rows.  With Z' the panel's part of Z then
+// and W = L_pp^{-1}, that block is Sigma_pp = W^T Y W, Y = I - L_pp^T Z', whose lower triangle
+// needs only that of Z': three products of an entry per thread, W made before the task's
+// first wait (w <= kSelWMax, where it fits beside the block).  Wider blocks take the element
+// recurrence on one warp, 18 FP64 instructions (1,150 clocks) a column: 16 bands of n = 50,000
+// with it 93.5 ms, without 65.6 (one column at a time over the whole block: 115).  Rows more
+// than kd below the diagonal are outside the band and left alone.  lget(i, c): L_ic, i >= c.  S0: digits; S1: digits, then the panel's
 // rows; sv: kNbMax doubles.
 constexpr int kSelP = 16;
 template <class LGet>
@@ -2420,7 +2449,7 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
                 }
                 __syncthreads();
             }
-            trsm_rows_dir<true>(X, LDX, m, pw, D, kSelP + 1, sv);
+            trsm_back(X, LDX, m, pw, D, kSelP + 1, sv);
             __syncthreads();
         }
         // the panel's own block: the products with the rows below, an entry per thread
@@ -2448,7 +2477,32 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
             }
         }
         __syncthreads();
-        if (threadIdx.x < 32) {
+        if (w <= kSelWMax) {
+            // Sigma_pp = W^T Y W, Y = I - L_pp^T Z' (P holds -Z'): three products of an entry
+            // per thread, Y and Y W in the rows' buffer
+            const double* W = P + w * (w + 1) / 2 + (p / kSelP) * 272;
+            double *Y = X, *T = X + 272;
+            const int r = threadIdx.x & 15, c = threadIdx.x >> 4;
+            const bool in = r < pw && c < pw;
+            if (in && r >= c) {
+                double y = r == c ? 1.0 : 0.0;
+                for (int i = r; i < pw; ++i) y = fma(D[i + r * (kSelP + 1)], P[pk(w, p + i, p + c)], y);
+                Y[r + 17 * c] = y;
+                Y[c + 17 * r] = y;
+            }
+            __syncthreads();
+            if (in) {
+                double t = 0.0;
+                for (int i = c; i < pw; ++i) t = fma(Y[r + 17 * i], W[i + 17 * c], t);
+                T[r + 17 * c] = t;
+            }
+            __syncthreads();
+            if (in && r >= c) {
+                double g = 0.0;
+                for (int i = r; i < pw; ++i) g = fma(W[i + 17 * r], T[i + 17 * c], g);
+                P[pk(w, p + r, p + c)] = g;
+            }
+        } else if (threadIdx.x < 32) {
             // two lanes per row (odd and even inner rows)
             const int r = threadIdx.x >> 1, hf = threadIdx.x & 1;
             for (int c = pw - 1; c >= 0; --c) {
@@ -2496,7 +2550,7 @@ __device__ __forceinline__ void selinv_back(double* C, int R, int w, double* S0,
         __syncthreads();
         if (threadIdx.x < pw) sv[threadIdx.x] = 1.0 / S0[threadIdx.x * (kPb + 2)];
         __syncthreads();
-        trsm_rows_dir<true>(C + p * kRLd, kRLd, R, pw, S0, kPb + 1, sv);
+        trsm_back(C + p * kRLd, kRLd, R, pw, S0, kPb + 1, sv);
         __syncthreads();
     }
 }
@@ -2589,6 +2643,7 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
         } else if (t.kind == TASK_SDIAG && s_ok) {
             const int w = O.sw;
             for (int e = threadIdx.x; e < w * (w + 1) / 2; e += kThreads) C[e] = 0.0;
+            if (w <= kSelWMax) selinv_inverses(C, w, [&](int i, int c) { return diag_at(DT, D, nb, i, c); });
             __syncthreads();
             for (int ci = t.cbeg; ci < t.cend; ++ci) {
                 const DSCon cn = a.cons[ci];
@@ -2742,6 +2797,7 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
             }
         } else if (t.kind == SN_S_DIAG && s_ok) {
             for (int e = threadIdx.x; e < w * (w + 1) / 2; e += kThreads) C[e] = 0.0;
+            if (w <= kSelWMax) selinv_inverses(C, w, lget);
             __syncthreads();
             for (int ci = t.cbeg; ci < t.cend; ++ci) {
                 const SnSCon q = a.cons[ci];

@@ -17,7 +17,6 @@
 // supernodal route: one factorization at n = 180,020 517 -> 251 ms, a 48^3 FEM operator
 // 180 -> 98 ms, 16 sets at n = 22,520 95 -> 57 ms, and the products and their staging no
 // more than 37 % of the CTAs' time (the rest waits for other tasks).  Tile routes: 64 bands
-// (n = 50,000, half-bandwidth 200) 178 -> 89 ms with the 16-column panels of POTRF and TRSM.  Tile routes: 64 bands
 // (n = 50,000, half-bandwidth 200) 178 -> 89 ms with the 16-column panels of POTRF and TRSM.
 //
 // Rows whose largest entry is not finite or lies outside 2^[-400, 400] (where the scale
