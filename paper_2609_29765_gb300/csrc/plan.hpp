@@ -289,9 +289,6 @@ struct SnPlan {
     std::vector<int16_t> maps;
     std::vector<int64_t> value_map;  // per A entry: arena offset (permuted lower entry)
     std::vector<int64_t> csc_map;    // per structural L entry: arena offset
-    std::vector<int32_t> cell_cmap;  // per cell: offset in maps of its rows as columns of
-                                     // its row supernode (-1 for diagonal cells)
-    std::vector<int32_t> rptr_cells, row_cells;  // per row supernode J: cells (J, I), I < J
     double fma_exec = 0.0;           // FMAs of the device form (updates, POTRF, TRSM)
     std::vector<SnSTask> stasks;     // selected inverse, reverse supernode order
     std::vector<SnSCon> scons;
@@ -326,10 +323,6 @@ struct SnDev {
     SnDevUpd* upds = nullptr;
     int16_t* maps = nullptr;
     int32_t* first = nullptr;       // nsn + 1
-    int32_t* cell_cmap = nullptr;
-    int32_t* cptr = nullptr;        // nsn + 1: cells of column supernode I (diagonal first)
-    int32_t* rptr_cells = nullptr;  // nsn + 1
-    int32_t* row_cells = nullptr;
     int64_t* value_map = nullptr;
     int64_t* csc_map = nullptr;
     int32_t* fill_src = nullptr;    // per arena double: the A entry stored there or -1

@@ -2949,8 +2949,7 @@ void free_dev(stc_plan* P) {
         if (p) cudaFree(p);
     d = DevPlanArrays{};
     SnDev& q = P->sndev;
-    void* sptrs[] = {q.cells, q.tasks, q.upds, q.maps, q.first, q.cell_cmap, q.cptr, q.rptr_cells, q.row_cells,
-                     q.value_map, q.csc_map, q.fill_src, q.stasks, q.scons, q.rows, q.cell_rowoff, q.order,
+    void* sptrs[] = {q.cells, q.tasks, q.upds, q.maps, q.first, q.value_map, q.csc_map, q.fill_src, q.stasks, q.scons, q.rows, q.cell_rowoff, q.order,
                      q.snodes, q.skids, q.srel, q.schunk_own, q.sfwd, q.sbwd};
     for (void* p : sptrs)
         if (p) cudaFree(p);
@@ -3075,20 +3074,13 @@ int ensure_sn_impl(stc_plan* P, int dev) {
     if (d.device == dev) return STC_OK;
     if (d.device >= 0) return STC_ERR_UNSUPPORTED;  // one device per plan's supernodal copy
     int rc;
-    std::vector<int32_t> cptr(S.cptr.begin(), S.cptr.end());
     std::vector<int16_t> maps = S.maps;
     if (maps.empty()) maps.push_back(0);
-    std::vector<int32_t> rc_list = S.row_cells;
-    if (rc_list.empty()) rc_list.push_back(0);
     if ((rc = upload(&d.cells, S.dcells))) return rc;
     if ((rc = upload(&d.tasks, S.dtasks))) return rc;
     if ((rc = upload(&d.upds, S.dupds))) return rc;
     if ((rc = upload(&d.maps, maps))) return rc;
     if ((rc = upload(&d.first, S.first))) return rc;
-    if ((rc = upload(&d.cell_cmap, S.cell_cmap))) return rc;
-    if ((rc = upload(&d.cptr, cptr))) return rc;
-    if ((rc = upload(&d.rptr_cells, S.rptr_cells))) return rc;
-    if ((rc = upload(&d.row_cells, rc_list))) return rc;
     if ((rc = upload(&d.value_map, S.value_map))) return rc;
     if ((rc = upload(&d.csc_map, S.csc_map))) return rc;
     {

@@ -271,15 +271,7 @@ void stc_plan::build_device_form(stc::SnPlan& S, const vector<int32_t>& snof,
             }
         }
     }
-    // per-cell column maps (every off-diagonal cell (J, I) is a source of J's diagonal
-    // task, so each has one), the cells owned by each row supernode, and the FMAs the
-    // device form executes: updates (lower half on a diagonal target), POTRF, TRSM
-    S.cell_cmap = cmap_of;
-    S.rptr_cells.assign(nsn + 1, 0);
-    for (int32_t J = 0; J < nsn; ++J) {
-        S.rptr_cells[J + 1] = S.rptr_cells[J] + (int32_t)byrow[J].size();
-        S.row_cells.insert(S.row_cells.end(), byrow[J].begin(), byrow[J].end());
-    }
+    // the FMAs the device form executes: updates (lower half on a diagonal target), POTRF, TRSM
     double fma = 0.0;
     for (const stc::SnDevTask& t : S.dtasks) {
         const double w = S.dcells[t.cell].w;
