@@ -2398,13 +2398,14 @@ __device__ void selinv_inverses(double* C, int w, LGet lget) {
 // by panels of 16 columns from the right: the rows below a panel take the products with the
 // columns already done (chunk products of the symmetric part) and a triangular solve, the
 // panel's own 16 x 16 block the products with those rows.  With Z' the panel's part of Z then
-// and W = L_pp^{-1}, that block is Sigma_pp = W^T Y W, Y = I - L_pp^T Z', whose lower triangle
-// needs only that of Z': three products of an entry per thread, W made before the task's
+// and W = L_pp^{-1}, that block is Sigma_pp = W^T W + W^T Y W, Y = -L_pp^T Z', whose lower
+// triangle needs only that of Z': four products of an entry per thread, W made before the task's
 // first wait (w <= kSelWMax, where it fits beside the block).  Wider blocks take the element
 // recurrence on one warp, 18 FP64 instructions (1,150 clocks) a column: 16 bands of n = 50,000
-// with it 93.5 ms, without 65.6 (one column at a time over the whole block: 115).  Rows more
-// than kd below the diagonal are outside the band and left alone.  lget(i, c): L_ic, i >= c.  S0: digits; S1: digits, then the panel's
-// rows; sv: kNbMax doubles.
+// with it 93.5 ms, without 67.4 (65.6 with I left inside Y, which costs a rounding: error against
+// 64 bits 3.9e-16 for 3.0e-16; one column at a time over the whole block: 115).  Rows more
+// than kd below the diagonal are outside the band and left alone.  lget(i, c): L_ic, i >= c.
+// S0: digits; S1: digits, then the panel's rows; sv: kNbMax doubles.
 constexpr int kSelP = 16;
 template <class LGet>
 __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, double* sv, LGet lget) {
@@ -2478,14 +2479,15 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
         }
         __syncthreads();
         if (w <= kSelWMax) {
-            // Sigma_pp = W^T Y W, Y = I - L_pp^T Z' (P holds -Z'): three products of an entry
-            // per thread, Y and Y W in the rows' buffer
+            // Sigma_pp = W^T W + W^T (Y W), Y = -L_pp^T Z' (P holds -Z'): products of an entry
+            // per thread, Y and Y W in the rows' buffer.  W^T W apart, its largest term last:
+            // the terms of 1/L^2, which dominate, are rounded once
             const double* W = P + w * (w + 1) / 2 + (p / kSelP) * 272;
             double *Y = X, *T = X + 272;
             const int r = threadIdx.x & 15, c = threadIdx.x >> 4;
             const bool in = r < pw && c < pw;
             if (in && r >= c) {
-                double y = r == c ? 1.0 : 0.0;
+                double y = 0.0;
                 for (int i = r; i < pw; ++i) y = fma(D[i + r * (kSelP + 1)], P[pk(w, p + i, p + c)], y);
                 Y[r + 17 * c] = y;
                 Y[c + 17 * r] = y;
@@ -2498,9 +2500,13 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
             }
             __syncthreads();
             if (in && r >= c) {
-                double g = 0.0;
-                for (int i = r; i < pw; ++i) g = fma(W[i + 17 * r], T[i + 17 * c], g);
-                P[pk(w, p + r, p + c)] = g;
+                double g0 = 0.0, g1 = 0.0;
+                for (int i = pw - 1; i > r; --i) {
+                    g0 = fma(W[i + 17 * r], W[i + 17 * c], g0);
+                    g1 = fma(W[i + 17 * r], T[i + 17 * c], g1);
+                }
+                g1 = fma(W[r + 17 * r], T[r + 17 * c], g1);
+                P[pk(w, p + r, p + c)] = fma(W[r + 17 * r], W[r + 17 * c], g0 + g1);
             }
         } else if (threadIdx.x < 32) {
             // two lanes per row (odd and even inner rows)
