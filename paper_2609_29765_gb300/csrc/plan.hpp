@@ -243,13 +243,13 @@ struct SnSTask {
     int32_t diag;      // diagonal cell of J
     int32_t cbeg, cend;
     int32_t rs0, rs1;  // rows of the target cell written
-    int32_t pad;
+    int32_t rdiag;     // diagonal cell of the target's row supernode
 };
 struct SnSCon {
     int32_t lcell;     // L cell (K',J)
     int32_t scell;     // Sigma cell read
     int32_t mode;      // SN_SC_*
-    int32_t pad;
+    int32_t diag;      // diagonal cell of K'
 };
 constexpr int kSnSolveRows = 256;
 struct SnSolveNode {   // one supernode as the solve sees it

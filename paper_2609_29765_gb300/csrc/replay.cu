@@ -2320,6 +2320,7 @@ struct SelinvArgs {
     const int16_t* sinv;     // [ntiles][nb]
     const DSTask* tasks;
     const DSCon* cons;
+    const int32_t* diag_tile;  // per block: tile of (k,k)
     const double* factor;
     double* sigma;
     long long fstride;
@@ -2336,12 +2337,26 @@ __device__ __forceinline__ double sym_at(const double* T, const DTile& d, int nb
     return r >= c ? diag_at(T, d, nb, r, c) : diag_at(T, d, nb, c, r);
 }
 
+// Balance of the split products here (see splitmm.cuh): an inner index is a variable i, with
+// Sigma_ri on one side and L_ic on the other, and 2^e_i is the standard deviation
+// sqrt(Sigma_ii).  Then |Sigma_ri| / 2^e_i <= 2 sqrt(Sigma_rr) along a row, so the cut stays
+// below 2^-55 sqrt(Sigma_rr) max_i |L_ic| sqrt(Sigma_ii): what the rounding of the DFMAs is
+// bounded by, and as invariant under a change of units.  Restated on the CPU against 60 digits
+// (block elimination, n = 49..256, products alone; error of Sigma_ij over sqrt(Sigma_ii
+// Sigma_jj)): first-order walk + 1e-8 with units 2^U(-20, 20) 4e-8 without balance, 1e-15 with
+// it (DFMAs 1e-15), third-order 8e-2 / 3e-10 (2e-10); scaled by L_ii in place of the deviation a
+// random graph with conductances e^(6 N(0,1)) gives 5e-13 (DFMAs and this 8e-16).
+__device__ __forceinline__ int sd_exp(double s) {
+    return sp_balance((((__double2hiint(s) >> 20) & 0x7ff) - 1023) >> 1);
+}
+
 // at(r, c) -= sum_k ga(r, k) gb(c, k), r < R, c < Cn (LOWER: r >= c), k < K <= 16, by the
 // whole CTA (a barrier at the end): the split where it pays and can take the chunk, else
-// DFMAs from staged operands.  S0, S1: staging buffers.
+// DFMAs from staged operands.  S0, S1: staging buffers; e: the balance of the inner index.
 template <bool LOWER, class GetA, class GetB, class At>
-__device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int Cn, int K, GetA ga, GetB gb, At at) {
-    if (sp_worth(LOWER ? R * Cn / 2 : R * Cn, K) && sp_stage_ab(S0, R, ga, S1, Cn, gb, K)) {
+__device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int Cn, int K, const int* e, GetA ga,
+                                              GetB gb, At at) {
+    if (sp_worth(LOWER ? R * Cn / 2 : R * Cn, K) && sp_stage_ab(S0, R, ga, S1, Cn, gb, K, Balance{e, R, K})) {
         sp_product<LOWER>(S0, 0, R, S1, 0, Cn, at);
     } else {
         for_rc(R, K, [&](int r, int k) { S0[r + k * kRStLd] = ga(r, k); });
@@ -2405,10 +2420,10 @@ __device__ void selinv_inverses(double* C, int w, LGet lget) {
 // with it 93.5 ms, without 67.4 (65.6 with I left inside Y, which costs a rounding: error against
 // 64 bits 3.9e-16 for 3.0e-16; one column at a time over the whole block: 115).  Rows more
 // than kd below the diagonal are outside the band and left alone.  lget(i, c): L_ic, i >= c.
-// S0: digits; S1: digits, then the panel's rows; sv: kNbMax doubles.
+// S0: digits; S1: digits, then the panel's rows; sv: kNbMax doubles; be: kNbMax, the balance.
 constexpr int kSelP = 16;
 template <class LGet>
-__device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, double* sv, LGet lget) {
+__device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, double* sv, int* be, LGet lget) {
     constexpr int LDX = kNbMax + 1 - kSelP;   // panel rows below: at most kNbMax - kSelP
     static_assert(LDX * kSelP + kSelP * (kSelP + 1) <= kRStage, "panel rows and its diagonal block fit a staging buffer");
     double* X = S1;                           // X(r, c), row b + r of the panel's columns
@@ -2437,7 +2452,7 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
                 };
                 auto gb = [&](int c, int k) { return lget(b + i0 + k, p + c); };
                 auto gab = [&](int r, int k) { return r < m ? ga(r, k) : gb(r - m, k); };
-                if (sp_worth(m * pw, K) && sp_stage_a(S0, m + pw, gab, K)) {
+                if (sp_worth(m * pw, K) && sp_stage_a(S0, m + pw, gab, K, Balance{be + b + i0, m, K})) {
                     sp_product<false>(S0, 0, m, S0, m, pw, [&](int r, int c) -> double& { return X[r + c * LDX]; });
                 } else {
                     for_rc(pw, K, [&](int c, int k) { S0[c + k * kRStLd] = gb(c, k); });
@@ -2533,21 +2548,26 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
             }
         }
         __syncthreads();
+        if (threadIdx.x < pw) be[p + threadIdx.x] = sd_exp(P[pk(w, p + threadIdx.x, p + threadIdx.x)]);
     }
 }
 
 // Rows [rs0, rs0 + R) of an off-diagonal block of a selected inverse, held in C (leading
-// dimension kRLd, w columns): C <- C L^{-1}, panels of 32 columns from the right.
+// dimension kRLd, w columns): C <- C L^{-1}, panels of 32 columns from the right.  The
+// deviations of the block's own variables k are not known yet, those of the rows are (2^er[r]):
+// ek[k], the balance of column k, is that of the largest |X_rk| / 2^er[r], at most sqrt(Sigma_kk).
 template <class LGet>
-__device__ __forceinline__ void selinv_back(double* C, int R, int w, double* S0, double* S1, double* sv, LGet lget) {
+__device__ __forceinline__ void selinv_back(double* C, int R, int w, double* S0, double* S1, double* sv, const int* er,
+                                            int* ek, LGet lget) {
     for (int p = ((w - 1) / kPb) * kPb; p >= 0; p -= kPb) {
         const int pw = min(kPb, w - p);
         for (int k0 = p + pw; k0 < w; k0 += kSpK) {
             const double* X = C + k0 * kRLd;
             double* Y = C + p * kRLd;
-            chunk_product<false>(S0, S1, R, pw, min(kSpK, w - k0), [&](int r, int k) { return X[r + k * kRLd]; },
-                          [&](int c, int k) { return lget(k0 + k, p + c); },
-                          [&](int r, int c) -> double& { return Y[r + c * kRLd]; });
+            chunk_product<false>(S0, S1, R, pw, min(kSpK, w - k0), ek + k0,
+                                 [&](int r, int k) { return X[r + k * kRLd]; },
+                                 [&](int c, int k) { return lget(k0 + k, p + c); },
+                                 [&](int r, int c) -> double& { return Y[r + c * kRLd]; });
         }
         for (int idx = threadIdx.x; idx < kPb * kPb; idx += kThreads) {
             const int i = idx & (kPb - 1), j = idx / kPb;
@@ -2558,6 +2578,21 @@ __device__ __forceinline__ void selinv_back(double* C, int R, int w, double* S0,
         __syncthreads();
         trsm_back(C + p * kRLd, kRLd, R, pw, S0, kPb + 1, sv);
         __syncthreads();
+        if (p > 0) {  // eight threads a column
+            static_assert(kThreads == 8 * kPb, "a pass covers a panel's columns");
+            const int c = threadIdx.x >> 3;
+            constexpr int kZero = -100000;  // a column of zeros: its row of L counts for nothing
+            int e = kZero;
+            if (c < pw)
+                for (int r = threadIdx.x & 7; r < R; r += 8) {
+                    const int x = (__double2hiint(C[r + (p + c) * kRLd]) >> 20) & 0x7ff;
+                    if (x > 0) e = max(e, x - 1023 - er[r]);
+                }
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) e = max(e, __shfl_xor_sync(0xffffffffu, e, o));
+            if (c < pw && (threadIdx.x & 7) == 0) ek[p + c] = e == kZero ? -kSpBalMax : sp_balance(e);
+            __syncthreads();
+        }
     }
 }
 
@@ -2572,6 +2607,7 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
     const long long total = (long long)a.ntasks * a.batch;
     const int nb = a.nb;
     __shared__ int16_t s_idx[2][kNbMax];  // stored-column indices of a contribution's tiles
+    __shared__ int s_be[kNbMax], s_er[kRRows];  // balance of the inner index, deviations of the rows
     for (;;) {
         if (threadIdx.x == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
         __syncthreads();
@@ -2599,11 +2635,23 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                     const DSCon cn = a.cons[ci];
                     const DTile Lt = a.tiles[cn.ltile];
                     const DTile St = a.tiles[cn.stile];
-                    if (threadIdx.x == 0) s_ok = wait_counter(cnt + cn.stile, 1, a.spin, &a.hdr->status);
-                    __syncthreads();
-                    if (!s_ok) break;
+                    // Sigma's tile, and the diagonal tile of j for the deviations of its variables
+                    // (the tasks of j come earlier in the queue)
+                    const int dj = a.diag_tile[Lt.I];
+                    bool ok = true;
+                    if (threadIdx.x == 0) ok = wait_counter(cnt + cn.stile, 1, a.spin, &a.hdr->status);
+                    if (threadIdx.x == 32 && cn.mode != SCON_DIAG)
+                        ok = wait_counter(cnt + dj, 1, a.spin, &a.hdr->status);
+                    if (!__syncthreads_and(ok)) {
+                        if (threadIdx.x == 0) s_ok = 0;
+                        __syncthreads();
+                        break;
+                    }
                     const double* LT = Lf + Lt.off;
                     const double* ST = Sg + St.off;
+                    const DTile Dj = a.tiles[dj];
+                    for (int i = Lt.r0 + threadIdx.x; i < Lt.r1; i += kThreads)
+                        s_be[i] = sd_exp(diag_at(Sg + Dj.off, Dj, nb, i, i));
                     const int16_t* si_S = a.sinv + (size_t)cn.stile * nb;
                     const int16_t* si_L = a.sinv + (size_t)cn.ltile * nb;
                     // stored-column indices used by every chunk: Sigma's for the inner rows i
@@ -2633,12 +2681,18 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                             const int q = s_idx[1][c];
                             return q >= 0 ? __ldg(LT + (i0 + k) + (size_t)q * nb) : 0.0;
                         };
-                        chunk_product<false>(S0, S1, R, sw, K, ga, gb, [&](int r, int c) -> double& { return C[r + c * kRLd]; });
+                        chunk_product<false>(S0, S1, R, sw, K, s_be + i0, ga, gb,
+                                             [&](int r, int c) -> double& { return C[r + c * kRLd]; });
                     }
                 }
                 if (s_ok) {
-                    // X L_g = C on the stored columns
-                    selinv_back(C, R, sw, S0, S1, sv, [&](int i, int j) {
+                    // X L_g = C on the stored columns (the diagonal tile of the rows is the
+                    // SCON_DIAG contribution's)
+                    const DTile Dm = a.tiles[a.diag_tile[O.I]];
+                    for (int r = threadIdx.x; r < R; r += kThreads)
+                        s_er[r] = sd_exp(diag_at(Sg + Dm.off, Dm, nb, rs0 + r, rs0 + r));
+                    __syncthreads();
+                    selinv_back(C, R, sw, S0, S1, sv, s_er, s_be, [&](int i, int j) {
                         return diag_at(DT, D, nb, logical_col(O, a.saind, i), logical_col(O, a.saind, j));
                     });
                     double* T = Sg + O.off;
@@ -2662,6 +2716,10 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                 const bool contig = Tt.c0 >= 0;
                 const int M = contig ? Tt.sw : w;   // rows/cols of the Z block
                 const int z0 = contig ? Tt.c0 : 0;
+                // the diagonal tile of the rows was final before this tile could be
+                const DTile Dm = a.tiles[a.diag_tile[Tt.I]];
+                for (int i = Tt.r0 + threadIdx.x; i < Tt.r1; i += kThreads)
+                    s_be[i] = sd_exp(diag_at(Sg + Dm.off, Dm, nb, i, i));
                 const int16_t* si = a.sinv + (size_t)cn.ltile * nb;
                 for (int q = threadIdx.x; q < nb; q += kThreads) s_idx[0][q] = contig ? (int16_t)q : si[q];
                 __syncthreads();
@@ -2676,11 +2734,11 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                         return q >= 0 ? __ldg(LT + (i0 + k) + (size_t)q * nb) : 0.0;
                     };
                     auto epi = [&](int r, int c) -> double& { return C[pk(w, z0 + r, z0 + c)]; };
-                    chunk_product<true>(S0, S1, M, M, K, ga, gb, epi);
+                    chunk_product<true>(S0, S1, M, M, K, s_be + i0, ga, gb, epi);
                 }
             }
             if (s_ok) {
-                selinv_diag(C, w, min(O.kd, nb - 1), S0, S1, sv,
+                selinv_diag(C, w, min(O.kd, nb - 1), S0, S1, sv, s_be,
                             [&](int i, int c) { return diag_at(DT, D, nb, i, c); });
                 // padding rows and columns of a ragged tile: zero
                 write_sigma_diag(C, w, Sg + O.off, O, nb);
@@ -2730,6 +2788,7 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
     __shared__ long long s_slot;
     __shared__ int s_ok;
     __shared__ int ia[kNbMax], ja[kNbMax], srow[kNbMax];
+    __shared__ int s_be[kNbMax], s_er[kRRows];  // balance of the inner index, deviations of the rows
     const long long total = (long long)a.ntasks * a.batch;
     for (;;) {
         if (threadIdx.x == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
@@ -2760,12 +2819,21 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                 const SnDevCell Lc = a.cells[q.lcell];
                 const SnDevCell Sc = a.cells[q.scell];
                 const int Kp = Lc.J, h = Lc.h;
-                if (threadIdx.x == 0) s_ok = wait_counter(cnt + q.scell, Sc.nslices, a.spin, &a.hdr->status);
+                const SnDevCell Dk = a.cells[q.diag];
+                // Sigma's cell, and the diagonal cell of K' for the deviations of its variables
+                // (the tasks of K' come earlier in the queue)
+                bool ok = true;
+                if (threadIdx.x == 0) ok = wait_counter(cnt + q.scell, Sc.nslices, a.spin, &a.hdr->status);
+                if (threadIdx.x == 32 && q.mode != SN_SC_SAME)
+                    ok = wait_counter(cnt + q.diag, Dk.nslices, a.spin, &a.hdr->status);
                 // row lists: the source cell's (for the searches) and the index maps of the
                 // gathered block G(i, j) = Sigma(row i of the target slice, row j of (K',J))
                 for (int i = threadIdx.x; i < Sc.h; i += kThreads) srow[i] = a.rows[a.rowoff[q.scell] + i];
-                __syncthreads();
-                if (!s_ok) break;
+                if (!__syncthreads_and(ok)) {
+                    if (threadIdx.x == 0) s_ok = 0;
+                    __syncthreads();
+                    break;
+                }
                 const int* rt = a.rows + a.rowoff[t.cell] + t.rs0;
                 const int* rp = a.rows + a.rowoff[q.lcell];
                 auto find = [&](int r) {  // position of global row r in the source cell's rows
@@ -2780,6 +2848,8 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                     ia[i] = q.mode == SN_SC_LOWER ? find(rt[i]) : rt[i] - a.first[K];
                 for (int j = threadIdx.x; j < h; j += kThreads)
                     ja[j] = q.mode == SN_SC_UPPER ? find(rp[j]) : rp[j] - a.first[q.mode == SN_SC_SAME ? K : Kp];
+                for (int j = threadIdx.x; j < h; j += kThreads)
+                    s_be[j] = sd_exp(__ldcg(Sg + Dk.off + (size_t)(rp[j] - a.first[Kp]) * (Dk.ld + 1)));
                 __syncthreads();
                 const double* ST = Sg + Sc.off;
                 const double* LT = Lf + Lc.off;
@@ -2792,12 +2862,18 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                     };
                     // L(K',J) rows j0.. (through L1: a thread walks down its column)
                     auto gb = [&](int c, int k) { return __ldg(LT + (j0 + k) + (size_t)c * Lc.ld); };
-                    chunk_product<false>(S0, S1, R, w, min(kSpK, h - j0), ga, gb,
+                    chunk_product<false>(S0, S1, R, w, min(kSpK, h - j0), s_be + j0, ga, gb,
                                   [&](int r, int c) -> double& { return C[r + c * kRLd]; });  // C = -sum G L
                 }
             }
             if (s_ok) {
-                selinv_back(C, R, w, S0, S1, sv, lget);
+                // (the diagonal cell of the rows is the SN_SC_SAME contribution's)
+                const SnDevCell Dr = a.cells[t.rdiag];
+                const int* rt = a.rows + a.rowoff[t.cell] + t.rs0;
+                for (int i = threadIdx.x; i < R; i += kThreads)
+                    s_er[i] = sd_exp(__ldcg(Sg + Dr.off + (size_t)(rt[i] - a.first[K]) * (Dr.ld + 1)));
+                __syncthreads();
+                selinv_back(C, R, w, S0, S1, sv, s_er, s_be, lget);
                 double* T = Sg + O.off + t.rs0;
                 for_rc(R, w, [&](int r, int c) { __stcg(T + r + (size_t)c * O.ld, C[r + c * kRLd]); });
             }
@@ -2813,16 +2889,22 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                 if (!s_ok) break;
                 const double* ST = Sg + Lc.off;
                 const double* LT = Lf + Lc.off;
+                // the diagonal cell of the rows was final before this cell could be
+                const SnDevCell Dk = a.cells[q.diag];
+                const int* rp = a.rows + a.rowoff[q.lcell];
+                for (int i = threadIdx.x; i < Lc.h; i += kThreads)
+                    s_be[i] = sd_exp(__ldcg(Sg + Dk.off + (size_t)(rp[i] - a.first[Lc.J]) * (Dk.ld + 1)));
+                __syncthreads();
                 for (int i0 = 0; i0 < Lc.h; i0 += kSpK) {
                     const int Kc = min(kSpK, Lc.h - i0);
                     auto ga = [&](int r, int k) { return __ldcg(ST + (i0 + k) + (size_t)r * Lc.ld); };
                     auto gb = [&](int r, int k) { return __ldg(LT + (i0 + k) + (size_t)r * Lc.ld); };
                     auto epi = [&](int r, int c) -> double& { return C[pk(w, r, c)]; };  // C = -Z (lower)
-                    chunk_product<true>(S0, S1, w, w, Kc, ga, gb, epi);
+                    chunk_product<true>(S0, S1, w, w, Kc, s_be + i0, ga, gb, epi);
                 }
             }
             if (s_ok) {
-                selinv_diag(C, w, w - 1, S0, S1, sv, lget);
+                selinv_diag(C, w, w - 1, S0, S1, sv, s_be, lget);
                 double* T = Sg + D.off;
                 for_rc(w, w, [&](int r, int c) {
                     if (r >= c) __stcg(T + r + (size_t)c * D.ld, C[pk(w, r, c)]);
@@ -3670,7 +3752,7 @@ extern "C" int stc_selinv(const stc_plan* Pc, const void* d_factor, int64_t batc
     if (cudaMemsetAsync(d_work, 0, factorize_ws(P, batch), st) != cudaSuccess) return STC_ERR_CUDA;
     SelinvArgs a{};
     a.tiles = ts->d_tiles; a.saind = P->dev.saind; a.sinv = P->dev.sinv; a.tasks = P->dev.stasks;
-    a.cons = P->dev.scons; a.factor = (const double*)d_factor; a.sigma = (double*)d_sigma;
+    a.cons = P->dev.scons; a.diag_tile = P->dev.diag_tile; a.factor = (const double*)d_factor; a.sigma = (double*)d_sigma;
     a.fstride = P->factor_doubles; a.hdr = (WorkHeader*)d_work;
     a.counters = (int*)((char*)d_work + sizeof(WorkHeader)); a.ntiles = (int)P->tiles.size();
     a.ntasks = (int)P->stasks.size(); a.batch = batch; a.nb = (int)P->nb;

@@ -46,23 +46,48 @@ __device__ __forceinline__ int* sp_exp(double* S) { return reinterpret_cast<int*
 // and two rows of four pairs (the fragment loads) both touch every bank once.
 __device__ __forceinline__ int sp_slot(int r, int kp) { return r * 8 + (kp ^ (((r & 1) << 2) | ((r >> 1) & 3))); }
 
-// Biased exponent of the largest entry of a chunk row v[0..15]; ok: the row can take this
-// path (see above).
-__device__ __forceinline__ int sp_row_exp(const double (&v)[kSpK], bool& ok) {
-    unsigned m = 0u, any = 0u;
+// Balance of the inner index.  A row keeps 62 bits below its largest entry of the chunk, so
+// both operands need rows whose entries matter alike: rows of L do (|L_ik| <= sqrt(a_ii) for
+// every k), rows of a selected inverse times L do not (Sigma_ri ~ 1 / d_i against L_ic ~ d_i
+// for a variable i in units 1 / d_i).  There the caller gives the power of two b(i, k) that
+// entry k of operand row i is multiplied by before the cut, opposite for the two operands, so
+// the products stay what they are.  It is added to the exponents only: no entry is formed.
+// A balance outside 2^+-kSpBalMax (entries that are not finite have to stay out of range)
+// becomes one that puts every row of the other operand out of range: DFMAs take the chunk.
+constexpr int kSpBalMax = 300, kSpUnbalanced = 3000;
+__device__ __forceinline__ int sp_balance(int e) { return abs(e) <= kSpBalMax ? e : kSpUnbalanced; }
+struct NoBalance {
+    static constexpr bool kNone = true;
+    __device__ __forceinline__ int operator()(int, int) const { return 0; }
+};
+struct Balance {  // A's rows (i < R) times 2^-e[k], B's times 2^e[k]
+    static constexpr bool kNone = false;
+    const int* e;
+    int R, K;
+    __device__ __forceinline__ int operator()(int i, int k) const { return k >= K ? 0 : i < R ? -e[k] : e[k]; }
+};
+
+// Biased exponent of the largest entry of a chunk row v[0..15], entry k times 2^bal(i, k);
+// ok: the row can take this path (see above; a subnormal entry counts as 2^-1023, far below
+// the cut of a row in range).
+template <class Bal>
+__device__ __forceinline__ int sp_row_exp(const double (&v)[kSpK], bool& ok, int i, Bal bal) {
+    int m = Bal::kNone ? 0 : -kSpUnbalanced;
+    unsigned any = 0u;
 #pragma unroll
     for (int k = 0; k < kSpK; ++k) {
         const unsigned h = (unsigned)__double2hiint(v[k]) & 0x7fffffffu;
-        m = max(m, h);
+        m = max(m, Bal::kNone ? (int)h : (int)(h >> 20) + bal(i, k));
         any |= h | (unsigned)__double2loint(v[k]);
     }
-    const int e = (int)(m >> 20);
+    const int e = Bal::kNone ? m >> 20 : m;
     ok = any == 0u || (e >= 1023 - 400 && e <= 1023 + 400);
     return e;
 }
 
-// The digits of row r, v[0..15] (zero from K on), e its exponent.
-__device__ __forceinline__ void sp_split_row(const double (&v)[kSpK], int e, int K, double* S, int r) {
+// The digits of v[0..15] (zero from K on) times 2^bal(i, k), e their exponent, as row r.
+template <class Bal>
+__device__ __forceinline__ void sp_split_row(const double (&v)[kSpK], int e, int K, double* S, int r, int i, Bal bal) {
     sp_exp(S)[r] = e;
     uint4* D = sp_digits(S);
 #pragma unroll
@@ -80,7 +105,7 @@ __device__ __forceinline__ void sp_split_row(const double (&v)[kSpK], int e, int
             unsigned long long f = ((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32) |
                                    (unsigned)__double2loint(v[2 * kp + q]);
             f = ex ? f : 0ull;
-            f = (f << 9) >> min(e - ex, 63);
+            f = (f << 9) >> min(e - ex - bal(i, 2 * kp + q), 63);
             f = ((int)h < 0 ? 0ull - f : f) + 0x8080808080808080ull;  // digit bytes, each + 128
             hi[q] = (unsigned)(f >> 32);
             lo[q] = (unsigned)f;
@@ -102,10 +127,12 @@ __device__ __forceinline__ bool sp_worth(int entries, int K) { return K * ((entr
 
 // Operands A (R x K, entries ga(r, k)) and B (Cn x K, gb(c, k)) of a chunk into the digit
 // buffers SA and SB, a thread per row (R + Cn <= blockDim.x); returns on every thread
-// whether all rows can take the tensor path, after a barrier.  IN_PLACE: ga or gb may read
-// SA or SB; nothing is written unless the result is true.
-template <bool IN_PLACE, class GetA, class GetB>
-__device__ __forceinline__ bool sp_stage_t(double* SA, int R, GetA ga, double* SB, int Cn, GetB gb, int K) {
+// whether all rows can take the tensor path, after a barrier.  bal(i, k): the balance of row
+// i (A's rows, then B's).  IN_PLACE: ga or gb may read SA or SB; nothing is written unless
+// the result is true.
+template <bool IN_PLACE, class GetA, class GetB, class Bal = NoBalance>
+__device__ __forceinline__ bool sp_stage_t(double* SA, int R, GetA ga, double* SB, int Cn, GetB gb, int K,
+                                           Bal bal = Bal()) {
     const int i = threadIdx.x;
     double v[kSpK];
 #pragma unroll
@@ -120,18 +147,19 @@ __device__ __forceinline__ bool sp_stage_t(double* SA, int R, GetA ga, double* S
             if (k < K) v[k] = gb(i - R, k);
     }
     bool ok = true;
-    const int e = sp_row_exp(v, ok);
+    const int e = sp_row_exp(v, ok, i, bal);
     if (IN_PLACE && !__syncthreads_and(ok)) return false;
-    if (i < R + Cn) sp_split_row(v, e, K, i < R ? SA : SB, i < R ? i : i - R);
+    if (i < R + Cn) sp_split_row(v, e, K, i < R ? SA : SB, i < R ? i : i - R, i, bal);
     return __syncthreads_and(ok);
 }
-template <class GetA, class GetB>
-__device__ __forceinline__ bool sp_stage_ab(double* SA, int R, GetA ga, double* SB, int Cn, GetB gb, int K) {
-    return sp_stage_t<false>(SA, R, ga, SB, Cn, gb, K);
+template <class GetA, class GetB, class Bal = NoBalance>
+__device__ __forceinline__ bool sp_stage_ab(double* SA, int R, GetA ga, double* SB, int Cn, GetB gb, int K,
+                                            Bal bal = Bal()) {
+    return sp_stage_t<false>(SA, R, ga, SB, Cn, gb, K, bal);
 }
-template <class GetA>
-__device__ __forceinline__ bool sp_stage_a(double* SA, int R, GetA ga, int K) {
-    return sp_stage_t<false>(SA, R, ga, SA, 0, ga, K);
+template <class GetA, class Bal = NoBalance>
+__device__ __forceinline__ bool sp_stage_a(double* SA, int R, GetA ga, int K, Bal bal = Bal()) {
+    return sp_stage_t<false>(SA, R, ga, SA, 0, ga, K, bal);
 }
 
 // Digits of one 16-byte pair as eight f16x2 registers (the two columns of digit d), exact:

@@ -294,13 +294,13 @@ void stc_plan::build_device_form(stc::SnPlan& S, const vector<int32_t>& snof,
             const int32_t K = S.cells[4 * T + 1];
             for (int32_t sl = 0; sl < S.dcells[T].nslices; ++sl) {
                 stc::SnSTask t{};
-                t.kind = stc::SN_S_OFF; t.cell = T; t.diag = c0;
+                t.kind = stc::SN_S_OFF; t.cell = T; t.diag = c0; t.rdiag = S.cptr[K];
                 t.rs0 = sl * stc::kSnSliceH; t.rs1 = std::min(height(T), t.rs0 + stc::kSnSliceH);
                 t.cbeg = (int32_t)S.scons.size();
                 for (int32_t c2 = c0 + 1; c2 < c1; ++c2) {
                     const int32_t K2 = S.cells[4 * c2 + 1];
                     stc::SnSCon q{};
-                    q.lcell = c2;
+                    q.lcell = c2; q.diag = S.cptr[K2];
                     if (K2 == K) { q.mode = stc::SN_SC_SAME; q.scell = S.cptr[K]; }
                     else if (K2 < K) { q.mode = stc::SN_SC_LOWER; q.scell = cell_of(K2, K); }
                     else { q.mode = stc::SN_SC_UPPER; q.scell = cell_of(K, K2); }
@@ -312,11 +312,11 @@ void stc_plan::build_device_form(stc::SnPlan& S, const vector<int32_t>& snof,
             }
         }
         stc::SnSTask d{};
-        d.kind = stc::SN_S_DIAG; d.cell = c0; d.diag = c0; d.rs0 = 0; d.rs1 = width(J);
+        d.kind = stc::SN_S_DIAG; d.cell = c0; d.diag = c0; d.rdiag = c0; d.rs0 = 0; d.rs1 = width(J);
         d.cbeg = (int32_t)S.scons.size();
         for (int32_t c2 = c0 + 1; c2 < c1; ++c2) {
             stc::SnSCon q{};
-            q.lcell = c2; q.scell = c2; q.mode = stc::SN_SC_OWN;
+            q.lcell = c2; q.scell = c2; q.mode = stc::SN_SC_OWN; q.diag = S.cptr[S.cells[4 * c2 + 1]];
             S.scons.push_back(q);
         }
         d.cend = (int32_t)S.scons.size();
