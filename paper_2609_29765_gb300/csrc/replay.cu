@@ -2375,8 +2375,16 @@ __device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int
 // The inverses W = L_pp^{-1} of the 16 x 16 diagonal blocks of a w x w triangle (w <=
 // kSelWMax) behind the packed triangle in C, panel q at C + w (w + 1) / 2 + 272 q, entry
 // (i, l) at i + 17 l: they need L only and are made before the first wait.  A column per lane
-// of a half-warp.
+// of a half-warp.  The place behind a panel's first column holds 1 where products with W may
+// be used, |W| |L_pp| having no row sum above kSelCond (the units of the variables cancel in
+// it), else 0.  Products against the recurrence, restated on the CPU against 60 digits on 340
+// walks, grids and covariance kernels with ridges of every size: largest ratio of the errors
+// 3.4 up to 64 (2 to 3 already at 1: one more rounding of 1 / L), 1.8 up to 128, 7 up to 1,000,
+// 2e4 beyond.  The panels of the spatio-temporal precisions and FEM operators have 2 to 31, a
+// first-order walk's 31; 64 gradients at n = 4,020 take as long with 16 as with 32, with 4
+// 1.4 ms more of 30.
 constexpr int kSelWMax = 112;
+constexpr double kSelCond = 16.0;
 static_assert(kSelWMax * (kSelWMax + 1) / 2 + (kSelWMax / 16) * 272 <= kRCbuf, "the inverses fit behind the triangle");
 template <class LGet>
 __device__ void selinv_inverses(double* C, int w, LGet lget) {
@@ -2389,7 +2397,7 @@ __device__ void selinv_inverses(double* C, int w, LGet lget) {
     __syncthreads();
     const int l = threadIdx.x & 15, q = threadIdx.x >> 4;  // np <= 7 < 16 half-warps
     if (q < ((np + 1) & ~1)) {
-        const double* M = Wb + min(q, np - 1) * 272;
+        double* M = Wb + min(q, np - 1) * 272;
         double x[16];
 #pragma unroll
         for (int i = 0; i < 16; ++i) {
@@ -2398,10 +2406,28 @@ __device__ void selinv_inverses(double* C, int w, LGet lget) {
             for (int k = 0; k < i; ++k) t = fma(-M[i + 17 * k], x[k], t);
             x[i] = t / M[i + 17 * i];
         }
-        __syncwarp();
-        if (q < np)
+        double s0 = 0.0, s1 = 0.0;  // row l of |L_pp|
 #pragma unroll
-            for (int i = 0; i < 16; ++i) Wb[q * 272 + i + 17 * l] = i >= l ? x[i] : 0.0;
+        for (int k = 0; k < 16; k += 2) {
+            s0 += fabs(M[l + 17 * k]);
+            s1 += fabs(M[l + 17 * (k + 1)]);
+        }
+        __syncwarp();
+        if (q < np) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) M[i + 17 * l] = i >= l ? x[i] : 0.0;
+            M[16 + 17 * l] = s0 + s1;
+        }
+        __syncwarp();
+        double c0 = 0.0, c1 = 0.0;  // row l of |W| |L_pp|
+#pragma unroll
+        for (int k = 0; k < 16; k += 2) {
+            c0 = fma(fabs(M[l + 17 * k]), M[16 + 17 * k], c0);
+            c1 = fma(fabs(M[l + 17 * (k + 1)]), M[16 + 17 * (k + 1)], c1);
+        }
+        const unsigned far = __ballot_sync(0xffffffffu, !(c0 + c1 <= kSelCond)) >> (threadIdx.x & 16);
+        __syncwarp();
+        if (q < np && l == 0) M[16] = (far & 0xffffu) ? 0.0 : 1.0;
     }
     __syncthreads();
 }
@@ -2415,11 +2441,15 @@ __device__ void selinv_inverses(double* C, int w, LGet lget) {
 // panel's own 16 x 16 block the products with those rows.  With Z' the panel's part of Z then
 // and W = L_pp^{-1}, that block is Sigma_pp = W^T W + W^T Y W, Y = -L_pp^T Z', whose lower
 // triangle needs only that of Z': four products of an entry per thread, W made before the task's
-// first wait (w <= kSelWMax, where it fits beside the block).  Wider blocks take the element
-// recurrence on one warp, 18 FP64 instructions (1,150 clocks) a column: 16 bands of n = 50,000
-// with it 93.5 ms, without 67.4 (65.6 with I left inside Y, which costs a rounding: error against
-// 64 bits 3.9e-16 for 3.0e-16; one column at a time over the whole block: 115).  Rows more
-// than kd below the diagonal are outside the band and left alone.  lget(i, c): L_ic, i >= c.
+// first wait (w <= kSelWMax, where it fits beside the block).  L_pp^T and W multiply the rounding
+// of Z', which the recurrence, using each finished entry in the next, does not: with a random
+// walk of order 3 + 1e-8 an error of 1.5e-7 over sqrt(Sigma_ii Sigma_jj) for 2e-10.  So only
+// panels whose |W| |L_pp| stays small (kSelCond) take the products; the others and wider blocks
+// take the element recurrence on one warp, 18 FP64 instructions (1,150 clocks) a column: 16
+// bands of n = 50,000 with it 93.5 ms, without 67.4 (65.6 with I left inside Y, which costs a
+// rounding: error against 64 bits 3.9e-16 for 3.0e-16; one column at a time over the whole
+// block: 115).  Rows more than kd below the diagonal are outside the band and left alone.
+// lget(i, c): L_ic, i >= c.
 // S0: digits; S1: digits, then the panel's rows; sv: kNbMax doubles; be: kNbMax, the balance.
 constexpr int kSelP = 16;
 template <class LGet>
@@ -2493,11 +2523,11 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
             }
         }
         __syncthreads();
-        if (w <= kSelWMax) {
+        const double* W = P + w * (w + 1) / 2 + (p / kSelP) * 272;
+        if (w <= kSelWMax && W[16] != 0.0) {
             // Sigma_pp = W^T W + W^T (Y W), Y = -L_pp^T Z' (P holds -Z'): products of an entry
             // per thread, Y and Y W in the rows' buffer.  W^T W apart, its largest term last:
             // the terms of 1/L^2, which dominate, are rounded once
-            const double* W = P + w * (w + 1) / 2 + (p / kSelP) * 272;
             double *Y = X, *T = X + 272;
             const int r = threadIdx.x & 15, c = threadIdx.x >> 4;
             const bool in = r < pw && c < pw;

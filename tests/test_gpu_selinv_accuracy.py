@@ -102,3 +102,49 @@ def test_units(name, units, route):
     else:
         u = np.random.default_rng(n).integers(-int(e), int(e) + 1, size=n).astype(float)
     _check(Ap, Ai, Ax, kw.pop("nb"), route, d=np.exp2(u), **kw)
+
+
+# ---- intrinsic fields and covariance kernels with a small ridge: ill-conditioned panels ----
+def _dense_lower(A, bw=None):
+    import scipy.sparse as sp
+    A = np.where(np.abs(np.subtract.outer(np.arange(len(A)), np.arange(len(A)))) <= (len(A) if bw is None else bw), A, 0.0)
+    return I.lower_csc(sp.csc_matrix(A))
+
+
+def _walk(n, order, ridge):
+    D = np.eye(n)
+    for _ in range(order):
+        D = np.diff(D, axis=0)
+    return D.T @ D + ridge * np.eye(n)
+
+
+def _kernel(n, f, ridge):
+    r = np.abs(np.subtract.outer(np.arange(n), np.arange(n))).astype(float)
+    return f(r) + ridge * np.eye(n)
+
+
+def _matern(r, length=20.0):
+    s = np.sqrt(5.0) * r / length
+    return (1.0 + s + s * s / 3.0) * np.exp(-s)
+
+
+RIDGED = {
+    "walk of order 1 + 1e-8": lambda: (_walk(96, 1, 1e-8), 1),
+    "walk of order 2 + 1e-8": lambda: (_walk(96, 2, 1e-8), 2),
+    "walk of order 3 + 1e-8": lambda: (_walk(96, 3, 1e-8), 3),
+    "Matern 5/2, range 20, + 1e-8": lambda: (_kernel(96, _matern, 1e-8), None),
+    "squared exponential, range 3, + 1e-8": lambda: (_kernel(96, lambda r: np.exp(-r * r / 18.0), 1e-8), None),
+    "squared exponential, range 3, + 1e-10": lambda: (_kernel(96, lambda r: np.exp(-r * r / 18.0), 1e-10), None),
+}
+
+
+# blocks up to 112 columns with and without the panels' inverses; in other units, too
+@pytest.mark.parametrize("route", ROUTES)
+@pytest.mark.parametrize("nb", [32, 64, 128])
+@pytest.mark.parametrize("units", [0, 30])
+@pytest.mark.parametrize("name", list(RIDGED))
+def test_ridged(name, units, nb, route):
+    A, bw = RIDGED[name]()
+    Ap, Ai, Ax = _dense_lower(A, bw)
+    u = np.random.default_rng(nb).integers(-units, units + 1, size=len(A)).astype(float)
+    _check(Ap, Ai, Ax, nb, route, d=np.exp2(u), ordering="natural")
