@@ -2346,17 +2346,19 @@ __device__ __forceinline__ double sym_at(const double* T, const DTile& d, int nb
 // Sigma_jj)): first-order walk + 1e-8 with units 2^U(-20, 20) 4e-8 without balance, 1e-15 with
 // it (DFMAs 1e-15), third-order 8e-2 / 3e-10 (2e-10); scaled by L_ii in place of the deviation a
 // random graph with conductances e^(6 N(0,1)) gives 5e-13 (DFMAs and this 8e-16).
+static_assert(kNbMax <= kThreads && kNbMax % kSpK == 0, "a thread per inner row; a chunk's balances in range");
 __device__ __forceinline__ int sd_exp(double s) {
     return sp_balance((((__double2hiint(s) >> 20) & 0x7ff) - 1023) >> 1);
 }
 
 // at(r, c) -= sum_k ga(r, k) gb(c, k), r < R, c < Cn (LOWER: r >= c), k < K <= 16, by the
 // whole CTA (a barrier at the end): the split where it pays and can take the chunk, else
-// DFMAs from staged operands.  S0, S1: staging buffers; e: the balance of the inner index.
+// DFMAs from staged operands.  S0, S1: staging buffers; e: the balance of the inner index,
+// late: written since the last barrier.
 template <bool LOWER, class GetA, class GetB, class At>
-__device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int Cn, int K, const int* e, GetA ga,
-                                              GetB gb, At at) {
-    if (sp_worth(LOWER ? R * Cn / 2 : R * Cn, K) && sp_stage_ab(S0, R, ga, S1, Cn, gb, K, Balance{e, R, K})) {
+__device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int Cn, int K, const int* e, bool late,
+                                              GetA ga, GetB gb, At at) {
+    if (sp_worth(LOWER ? R * Cn / 2 : R * Cn, K) && sp_stage_ab(S0, R, ga, S1, Cn, gb, K, Balance{e, R, K, late})) {
         sp_product<LOWER>(S0, 0, R, S1, 0, Cn, at);
     } else {
         for_rc(R, K, [&](int r, int k) { S0[r + k * kRStLd] = ga(r, k); });
@@ -2482,7 +2484,7 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
                 };
                 auto gb = [&](int c, int k) { return lget(b + i0 + k, p + c); };
                 auto gab = [&](int r, int k) { return r < m ? ga(r, k) : gb(r - m, k); };
-                if (sp_worth(m * pw, K) && sp_stage_a(S0, m + pw, gab, K, Balance{be + b + i0, m, K})) {
+                if (sp_worth(m * pw, K) && sp_stage_a(S0, m + pw, gab, K, Balance{be + b + i0, m, K, false})) {
                     sp_product<false>(S0, 0, m, S0, m, pw, [&](int r, int c) -> double& { return X[r + c * LDX]; });
                 } else {
                     for_rc(pw, K, [&](int c, int k) { S0[c + k * kRStLd] = gb(c, k); });
@@ -2594,7 +2596,7 @@ __device__ __forceinline__ void selinv_back(double* C, int R, int w, double* S0,
         for (int k0 = p + pw; k0 < w; k0 += kSpK) {
             const double* X = C + k0 * kRLd;
             double* Y = C + p * kRLd;
-            chunk_product<false>(S0, S1, R, pw, min(kSpK, w - k0), ek + k0,
+            chunk_product<false>(S0, S1, R, pw, min(kSpK, w - k0), ek + k0, false,
                                  [&](int r, int k) { return X[r + k * kRLd]; },
                                  [&](int c, int k) { return lget(k0 + k, p + c); },
                                  [&](int r, int c) -> double& { return Y[r + c * kRLd]; });
@@ -2637,7 +2639,8 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
     const long long total = (long long)a.ntasks * a.batch;
     const int nb = a.nb;
     __shared__ int16_t s_idx[2][kNbMax];  // stored-column indices of a contribution's tiles
-    __shared__ int s_be[kNbMax], s_er[kRRows];  // balance of the inner index, deviations of the rows
+    __shared__ __align__(16) int s_be[kNbMax];  // balance of the inner index
+    __shared__ int s_er[kRRows];                          // deviations of the rows, see sd_exp
     for (;;) {
         if (threadIdx.x == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
         __syncthreads();
@@ -2661,27 +2664,19 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                 const int R = min(kRRows, t.r1 - rs0);
                 for_rc(R, sw, [&](int r, int c) { C[r + c * kRLd] = 0.0; });
                 __syncthreads();
-                for (int ci = t.cbeg; ci < t.cend; ++ci) {
+                // the newest block (the first listed) last: its deviations come latest
+                for (int ci = t.cend - 1; ci >= t.cbeg; --ci) {
                     const DSCon cn = a.cons[ci];
                     const DTile Lt = a.tiles[cn.ltile];
                     const DTile St = a.tiles[cn.stile];
                     // Sigma's tile, and the diagonal tile of j for the deviations of its variables
                     // (the tasks of j come earlier in the queue)
                     const int dj = a.diag_tile[Lt.I];
+                    const DTile Dj = a.tiles[dj];
                     bool ok = true;
                     if (threadIdx.x == 0) ok = wait_counter(cnt + cn.stile, 1, a.spin, &a.hdr->status);
                     if (threadIdx.x == 32 && cn.mode != SCON_DIAG)
                         ok = wait_counter(cnt + dj, 1, a.spin, &a.hdr->status);
-                    if (!__syncthreads_and(ok)) {
-                        if (threadIdx.x == 0) s_ok = 0;
-                        __syncthreads();
-                        break;
-                    }
-                    const double* LT = Lf + Lt.off;
-                    const double* ST = Sg + St.off;
-                    const DTile Dj = a.tiles[dj];
-                    for (int i = Lt.r0 + threadIdx.x; i < Lt.r1; i += kThreads)
-                        s_be[i] = sd_exp(diag_at(Sg + Dj.off, Dj, nb, i, i));
                     const int16_t* si_S = a.sinv + (size_t)cn.stile * nb;
                     const int16_t* si_L = a.sinv + (size_t)cn.ltile * nb;
                     // stored-column indices used by every chunk: Sigma's for the inner rows i
@@ -2690,7 +2685,16 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                         s_idx[0][q] = si_S[q];
                         s_idx[1][q] = q < sw ? si_L[logical_col(O, a.saind, q)] : (int16_t)-1;
                     }
-                    __syncthreads();
+                    if (!__syncthreads_and(ok)) {
+                        if (threadIdx.x == 0) s_ok = 0;
+                        __syncthreads();
+                        break;
+                    }
+                    const double* LT = Lf + Lt.off;
+                    const double* ST = Sg + St.off;
+                    const int ri = Lt.r0 + kThreads - 1 - threadIdx.x;
+                    if (sp_worth(R * sw, kSpK) && ri < Lt.r1)
+                        s_be[ri - Lt.r0] = sd_exp(diag_at(Sg + Dj.off, Dj, nb, ri, ri));
                     for (int i0 = Lt.r0; i0 < Lt.r1; i0 += kSpK) {
                         const int K = min(kSpK, Lt.r1 - i0);
                         // Sigma(m, j): output rows contiguous; Sigma(j, m)^T: inner rows contiguous
@@ -2711,17 +2715,19 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                             const int q = s_idx[1][c];
                             return q >= 0 ? __ldg(LT + (i0 + k) + (size_t)q * nb) : 0.0;
                         };
-                        chunk_product<false>(S0, S1, R, sw, K, s_be + i0, ga, gb,
+                        chunk_product<false>(S0, S1, R, sw, K, s_be + (i0 - Lt.r0), i0 == Lt.r0, ga, gb,
                                              [&](int r, int c) -> double& { return C[r + c * kRLd]; });
                     }
                 }
                 if (s_ok) {
                     // X L_g = C on the stored columns (the diagonal tile of the rows is the
-                    // SCON_DIAG contribution's)
-                    const DTile Dm = a.tiles[a.diag_tile[O.I]];
-                    for (int r = threadIdx.x; r < R; r += kThreads)
-                        s_er[r] = sd_exp(diag_at(Sg + Dm.off, Dm, nb, rs0 + r, rs0 + r));
-                    __syncthreads();
+                    // SCON_DIAG contribution's; one panel has no products to balance)
+                    if (sw > kPb) {
+                        const DTile Dm = a.tiles[a.diag_tile[O.I]];
+                        for (int r = threadIdx.x; r < R; r += kThreads)
+                            s_er[r] = sd_exp(diag_at(Sg + Dm.off, Dm, nb, rs0 + r, rs0 + r));
+                        __syncthreads();
+                    }
                     selinv_back(C, R, sw, S0, S1, sv, s_er, s_be, [&](int i, int j) {
                         return diag_at(DT, D, nb, logical_col(O, a.saind, i), logical_col(O, a.saind, j));
                     });
@@ -2738,21 +2744,21 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
             for (int ci = t.cbeg; ci < t.cend; ++ci) {
                 const DSCon cn = a.cons[ci];
                 const DTile Tt = a.tiles[cn.ltile];
+                const DTile Dm = a.tiles[a.diag_tile[Tt.I]];
+                const bool contig = Tt.c0 >= 0;
+                const int M = contig ? Tt.sw : w;   // rows/cols of the Z block
+                const int z0 = contig ? Tt.c0 : 0;
+                const int16_t* si = a.sinv + (size_t)cn.ltile * nb;
                 if (threadIdx.x == 0) s_ok = wait_counter(cnt + cn.stile, 1, a.spin, &a.hdr->status);
+                for (int q = threadIdx.x; q < nb; q += kThreads) s_idx[0][q] = contig ? (int16_t)q : si[q];
                 __syncthreads();
                 if (!s_ok) break;
                 const double* LT = Lf + Tt.off;
                 const double* ST = Sg + Tt.off;
-                const bool contig = Tt.c0 >= 0;
-                const int M = contig ? Tt.sw : w;   // rows/cols of the Z block
-                const int z0 = contig ? Tt.c0 : 0;
                 // the diagonal tile of the rows was final before this tile could be
-                const DTile Dm = a.tiles[a.diag_tile[Tt.I]];
-                for (int i = Tt.r0 + threadIdx.x; i < Tt.r1; i += kThreads)
-                    s_be[i] = sd_exp(diag_at(Sg + Dm.off, Dm, nb, i, i));
-                const int16_t* si = a.sinv + (size_t)cn.ltile * nb;
-                for (int q = threadIdx.x; q < nb; q += kThreads) s_idx[0][q] = contig ? (int16_t)q : si[q];
-                __syncthreads();
+                const int ri = Tt.r0 + kThreads - 1 - threadIdx.x;
+                if (sp_worth(M * M / 2, kSpK) && ri < Tt.r1)
+                    s_be[ri - Tt.r0] = sd_exp(diag_at(Sg + Dm.off, Dm, nb, ri, ri));
                 for (int i0 = Tt.r0; i0 < Tt.r1; i0 += kSpK) {
                     const int K = min(kSpK, Tt.r1 - i0);
                     auto ga = [&](int r, int k) {
@@ -2764,7 +2770,7 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                         return q >= 0 ? __ldg(LT + (i0 + k) + (size_t)q * nb) : 0.0;
                     };
                     auto epi = [&](int r, int c) -> double& { return C[pk(w, z0 + r, z0 + c)]; };
-                    chunk_product<true>(S0, S1, M, M, K, s_be + i0, ga, gb, epi);
+                    chunk_product<true>(S0, S1, M, M, K, s_be + (i0 - Tt.r0), i0 == Tt.r0, ga, gb, epi);
                 }
             }
             if (s_ok) {
@@ -2818,7 +2824,8 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
     __shared__ long long s_slot;
     __shared__ int s_ok;
     __shared__ int ia[kNbMax], ja[kNbMax], srow[kNbMax];
-    __shared__ int s_be[kNbMax], s_er[kRRows];  // balance of the inner index, deviations of the rows
+    __shared__ __align__(16) int s_be[kNbMax];  // balance of the inner index
+    __shared__ int s_er[kRRows];                          // deviations of the rows, see sd_exp
     const long long total = (long long)a.ntasks * a.batch;
     for (;;) {
         if (threadIdx.x == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
@@ -2844,12 +2851,15 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
             const int K = O.J;
             for_rc(R, w, [&](int r, int c) { C[r + c * kRLd] = 0.0; });
             __syncthreads();
-            for (int ci = t.cbeg; ci < t.cend; ++ci) {
+            // the newest supernode (the first listed) last: its deviations come latest
+            for (int ci = t.cend - 1; ci >= t.cbeg; --ci) {
                 const SnSCon q = a.cons[ci];
                 const SnDevCell Lc = a.cells[q.lcell];
                 const SnDevCell Sc = a.cells[q.scell];
                 const int Kp = Lc.J, h = Lc.h;
                 const SnDevCell Dk = a.cells[q.diag];
+                const int* rt = a.rows + a.rowoff[t.cell] + t.rs0;
+                const int* rp = a.rows + a.rowoff[q.lcell];
                 // Sigma's cell, and the diagonal cell of K' for the deviations of its variables
                 // (the tasks of K' come earlier in the queue)
                 bool ok = true;
@@ -2859,13 +2869,16 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                 // row lists: the source cell's (for the searches) and the index maps of the
                 // gathered block G(i, j) = Sigma(row i of the target slice, row j of (K',J))
                 for (int i = threadIdx.x; i < Sc.h; i += kThreads) srow[i] = a.rows[a.rowoff[q.scell] + i];
+                const int ri = kThreads - 1 - threadIdx.x;  // the row whose balance this thread makes
+                const bool mine = sp_worth(R * w, kSpK) && ri < h;
+                const int rc = mine ? rp[ri] - a.first[Kp] : 0;
                 if (!__syncthreads_and(ok)) {
                     if (threadIdx.x == 0) s_ok = 0;
                     __syncthreads();
                     break;
                 }
-                const int* rt = a.rows + a.rowoff[t.cell] + t.rs0;
-                const int* rp = a.rows + a.rowoff[q.lcell];
+                double sii = 0.0;
+                if (mine) sii = __ldcg(Sg + Dk.off + (size_t)rc * (Dk.ld + 1));
                 auto find = [&](int r) {  // position of global row r in the source cell's rows
                     int lo = 0, hi = Sc.h;
                     while (lo < hi) {
@@ -2878,9 +2891,8 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                     ia[i] = q.mode == SN_SC_LOWER ? find(rt[i]) : rt[i] - a.first[K];
                 for (int j = threadIdx.x; j < h; j += kThreads)
                     ja[j] = q.mode == SN_SC_UPPER ? find(rp[j]) : rp[j] - a.first[q.mode == SN_SC_SAME ? K : Kp];
-                for (int j = threadIdx.x; j < h; j += kThreads)
-                    s_be[j] = sd_exp(__ldcg(Sg + Dk.off + (size_t)(rp[j] - a.first[Kp]) * (Dk.ld + 1)));
                 __syncthreads();
+                if (mine) s_be[ri] = sd_exp(sii);
                 const double* ST = Sg + Sc.off;
                 const double* LT = Lf + Lc.off;
                 for (int j0 = 0; j0 < h; j0 += kSpK) {
@@ -2892,17 +2904,20 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                     };
                     // L(K',J) rows j0.. (through L1: a thread walks down its column)
                     auto gb = [&](int c, int k) { return __ldg(LT + (j0 + k) + (size_t)c * Lc.ld); };
-                    chunk_product<false>(S0, S1, R, w, min(kSpK, h - j0), s_be + j0, ga, gb,
+                    chunk_product<false>(S0, S1, R, w, min(kSpK, h - j0), s_be + j0, j0 == 0, ga, gb,
                                   [&](int r, int c) -> double& { return C[r + c * kRLd]; });  // C = -sum G L
                 }
             }
             if (s_ok) {
-                // (the diagonal cell of the rows is the SN_SC_SAME contribution's)
-                const SnDevCell Dr = a.cells[t.rdiag];
-                const int* rt = a.rows + a.rowoff[t.cell] + t.rs0;
-                for (int i = threadIdx.x; i < R; i += kThreads)
-                    s_er[i] = sd_exp(__ldcg(Sg + Dr.off + (size_t)(rt[i] - a.first[K]) * (Dr.ld + 1)));
-                __syncthreads();
+                // (the diagonal cell of the rows is the SN_SC_SAME contribution's; one panel has
+                // no products to balance)
+                if (w > kPb) {
+                    const SnDevCell Dr = a.cells[t.rdiag];
+                    const int* rt = a.rows + a.rowoff[t.cell] + t.rs0;
+                    for (int i = threadIdx.x; i < R; i += kThreads)
+                        s_er[i] = sd_exp(__ldcg(Sg + Dr.off + (size_t)(rt[i] - a.first[K]) * (Dr.ld + 1)));
+                    __syncthreads();
+                }
                 selinv_back(C, R, w, S0, S1, sv, s_er, s_be, lget);
                 double* T = Sg + O.off + t.rs0;
                 for_rc(R, w, [&](int r, int c) { __stcg(T + r + (size_t)c * O.ld, C[r + c * kRLd]); });
@@ -2914,23 +2929,24 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
             for (int ci = t.cbeg; ci < t.cend; ++ci) {
                 const SnSCon q = a.cons[ci];
                 const SnDevCell Lc = a.cells[q.lcell];
+                const SnDevCell Dk = a.cells[q.diag];
+                const int* rp = a.rows + a.rowoff[q.lcell];
                 if (threadIdx.x == 0) s_ok = wait_counter(cnt + q.scell, Lc.nslices, a.spin, &a.hdr->status);
+                const int ri = kThreads - 1 - threadIdx.x;  // the row whose balance this thread makes
+                const bool mine = sp_worth(w * w / 2, kSpK) && ri < Lc.h;
+                const int rc = mine ? rp[ri] - a.first[Lc.J] : 0;
                 __syncthreads();
                 if (!s_ok) break;
                 const double* ST = Sg + Lc.off;
                 const double* LT = Lf + Lc.off;
                 // the diagonal cell of the rows was final before this cell could be
-                const SnDevCell Dk = a.cells[q.diag];
-                const int* rp = a.rows + a.rowoff[q.lcell];
-                for (int i = threadIdx.x; i < Lc.h; i += kThreads)
-                    s_be[i] = sd_exp(__ldcg(Sg + Dk.off + (size_t)(rp[i] - a.first[Lc.J]) * (Dk.ld + 1)));
-                __syncthreads();
+                if (mine) s_be[ri] = sd_exp(__ldcg(Sg + Dk.off + (size_t)rc * (Dk.ld + 1)));
                 for (int i0 = 0; i0 < Lc.h; i0 += kSpK) {
                     const int Kc = min(kSpK, Lc.h - i0);
                     auto ga = [&](int r, int k) { return __ldcg(ST + (i0 + k) + (size_t)r * Lc.ld); };
                     auto gb = [&](int r, int k) { return __ldg(LT + (i0 + k) + (size_t)r * Lc.ld); };
                     auto epi = [&](int r, int c) -> double& { return C[pk(w, r, c)]; };  // C = -Z (lower)
-                    chunk_product<true>(S0, S1, w, w, Kc, s_be + i0, ga, gb, epi);
+                    chunk_product<true>(S0, S1, w, w, Kc, s_be + i0, i0 == 0, ga, gb, epi);
                 }
             }
             if (s_ok) {

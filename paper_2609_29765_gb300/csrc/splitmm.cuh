@@ -57,17 +57,24 @@ __device__ __forceinline__ int sp_slot(int r, int kp) { return r * 8 + (kp ^ (((
 constexpr int kSpBalMax = 300, kSpUnbalanced = 3000;
 __device__ __forceinline__ int sp_balance(int e) { return abs(e) <= kSpBalMax ? e : kSpUnbalanced; }
 struct NoBalance {
-    static constexpr bool kNone = true;
-    __device__ __forceinline__ int operator()(int, int) const { return 0; }
+    static constexpr bool kNone = true, late = false;
 };
 struct Balance {  // A's rows (i < R) times 2^-e[k], B's times 2^e[k]
     static constexpr bool kNone = false;
-    const int* e;
+    const int* e;  // 16 readable values from a 16-byte boundary on, those from K on unused
     int R, K;
-    __device__ __forceinline__ int operator()(int i, int k) const { return k >= K ? 0 : i < R ? -e[k] : e[k]; }
+    bool late;  // e was written since the last barrier (the same for the whole CTA)
 };
+// The balances of columns 4 g .. 4 g + 3 in row i.
+__device__ __forceinline__ void sp_bal4(const Balance& b, int i, int g, int (&s)[4]) {
+    const int4 x = reinterpret_cast<const int4*>(b.e)[g];
+    const int v[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) s[q] = 4 * g + q >= b.K ? 0 : i < b.R ? -v[q] : v[q];
+}
+__device__ __forceinline__ void sp_bal4(const NoBalance&, int, int, int (&s)[4]) { s[0] = s[1] = s[2] = s[3] = 0; }
 
-// Biased exponent of the largest entry of a chunk row v[0..15], entry k times 2^bal(i, k);
+// Biased exponent of the largest entry of a chunk row v[0..15], balanced as operand row i;
 // ok: the row can take this path (see above; a subnormal entry counts as 2^-1023, far below
 // the cut of a row in range).
 template <class Bal>
@@ -75,17 +82,22 @@ __device__ __forceinline__ int sp_row_exp(const double (&v)[kSpK], bool& ok, int
     int m = Bal::kNone ? 0 : -kSpUnbalanced;
     unsigned any = 0u;
 #pragma unroll
-    for (int k = 0; k < kSpK; ++k) {
-        const unsigned h = (unsigned)__double2hiint(v[k]) & 0x7fffffffu;
-        m = max(m, Bal::kNone ? (int)h : (int)(h >> 20) + bal(i, k));
-        any |= h | (unsigned)__double2loint(v[k]);
+    for (int g = 0; g < kSpK / 4; ++g) {
+        int s[4];
+        sp_bal4(bal, i, g, s);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const unsigned h = (unsigned)__double2hiint(v[4 * g + q]) & 0x7fffffffu;
+            m = max(m, Bal::kNone ? (int)h : (int)(h >> 20) + s[q]);
+            any |= h | (unsigned)__double2loint(v[4 * g + q]);
+        }
     }
     const int e = Bal::kNone ? m >> 20 : m;
     ok = any == 0u || (e >= 1023 - 400 && e <= 1023 + 400);
     return e;
 }
 
-// The digits of v[0..15] (zero from K on) times 2^bal(i, k), e their exponent, as row r.
+// The digits of v[0..15] (zero from K on), balanced as operand row i, e their exponent, as row r.
 template <class Bal>
 __device__ __forceinline__ void sp_split_row(const double (&v)[kSpK], int e, int K, double* S, int r, int i, Bal bal) {
     sp_exp(S)[r] = e;
@@ -96,6 +108,8 @@ __device__ __forceinline__ void sp_split_row(const double (&v)[kSpK], int e, int
             D[sp_slot(r, kp)] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
             continue;
         }
+        int s[4];
+        sp_bal4(bal, i, kp >> 1, s);
         unsigned hi[2], lo[2];
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
@@ -105,7 +119,7 @@ __device__ __forceinline__ void sp_split_row(const double (&v)[kSpK], int e, int
             unsigned long long f = ((unsigned long long)((h & 0xfffffu) | 0x100000u) << 32) |
                                    (unsigned)__double2loint(v[2 * kp + q]);
             f = ex ? f : 0ull;
-            f = (f << 9) >> min(e - ex - bal(i, 2 * kp + q), 63);
+            f = (f << 9) >> min(e - ex - s[2 * (kp & 1) + q], 63);
             f = ((int)h < 0 ? 0ull - f : f) + 0x8080808080808080ull;  // digit bytes, each + 128
             hi[q] = (unsigned)(f >> 32);
             lo[q] = (unsigned)f;
@@ -127,8 +141,8 @@ __device__ __forceinline__ bool sp_worth(int entries, int K) { return K * ((entr
 
 // Operands A (R x K, entries ga(r, k)) and B (Cn x K, gb(c, k)) of a chunk into the digit
 // buffers SA and SB, a thread per row (R + Cn <= blockDim.x); returns on every thread
-// whether all rows can take the tensor path, after a barrier.  bal(i, k): the balance of row
-// i (A's rows, then B's).  IN_PLACE: ga or gb may read SA or SB; nothing is written unless
+// whether all rows can take the tensor path, after a barrier.  bal: the balance of the inner
+// index.  IN_PLACE: ga or gb may read SA or SB; nothing is written unless
 // the result is true.
 template <bool IN_PLACE, class GetA, class GetB, class Bal = NoBalance>
 __device__ __forceinline__ bool sp_stage_t(double* SA, int R, GetA ga, double* SB, int Cn, GetB gb, int K,
@@ -146,6 +160,7 @@ __device__ __forceinline__ bool sp_stage_t(double* SA, int R, GetA ga, double* S
         for (int k = 0; k < kSpK; ++k)
             if (k < K) v[k] = gb(i - R, k);
     }
+    if (!Bal::kNone && bal.late) __syncthreads();  // the balance was written while the rows were loaded
     bool ok = true;
     const int e = sp_row_exp(v, ok, i, bal);
     if (IN_PLACE && !__syncthreads_and(ok)) return false;
