@@ -261,6 +261,8 @@ struct SnSolveNode {   // one supernode as the solve sees it
     int32_t roff;      // its rows below the diagonal block in the row lists
     int32_t kbeg, kend;  // children
     int32_t chunk, nchunk;  // its chunks (at least one)
+    int32_t parent;    // in the elimination tree, -1 for a root
+    int32_t pad;
 };
 struct SnPlan {
     std::vector<int32_t> first;

@@ -2049,6 +2049,11 @@ __global__ void __launch_bounds__(kThreads, 2) sn_replay_kernel(const __grid_con
 // Backward step J: z_J = L_JJ^{-T} (y_J - L_below^T z_below), z scattered to x = P^T z.  A
 // step waits for its children (its parent) only and reads its panel once as one dense block;
 // rows below beyond kSnSolveRows are tasks of their own, so a wide panel takes several SMs.
+// Chains run in groups of `inflight` (sn_inflight), which share the places of the update
+// vectors and partials: a step waits until the reader of the previous group's chain in its
+// place is done (an earlier task of the queue).  A group's backward steps alternate with the
+// next group's forward steps, so where one has few steps left to run, near the roots, the
+// other has many.
 // What bounds it: the path through the tree, per level a diagonal substitution and one
 // chunk (256 x 128 FMAs on one SM's FP64 pipe, 8 us).  Gathering every cell of a row
 // supernode one by one, in J order, took 58.2 ms at n = 180,020 (now 5.7),
@@ -2061,13 +2066,43 @@ struct SnSolveArgs {
     const double* b;           // [chains][n]
     double* x;                 // [chains][n]
     double* y;                 // workspace [chains][n]
-    double* u;                 // workspace [chains][nu]
-    double* part;              // workspace [chains][npart]
+    double* u;                 // workspace [inflight][nu]
+    double* part;              // workspace [inflight][npart]
     int* flags;                // workspace [chains][2 nchunks + 2 nsn]
     WorkHeader* hdr;
     long long chains, nrhs, n, nu, npart, spin;
+    long long inflight;        // chains of a group
     int nsn, nchunks;
 };
+
+// Queue slot -> chain group (returned), direction, and position among the group's steps of
+// that direction: F_0, then B_(g-1) and F_g in turn, then B of the last group.
+__device__ __forceinline__ long long sn_solve_slot(long long slot, long long nchunks, long long chains, long long inflight,
+                                                   bool* fwd, long long* sl) {
+    const long long ng = (chains + inflight - 1) / inflight;
+    const long long h = nchunks * inflight, hl = nchunks * (chains - (ng - 1) * inflight);  // steps of a group, of the last
+    const long long first = ng > 1 ? h : hl;
+    if (slot < first) {
+        *fwd = true;
+        *sl = slot;
+        return 0;
+    }
+    if (ng == 1) {
+        *fwd = false;
+        *sl = slot - first;
+        return 0;
+    }
+    const long long s = slot - h, g = min(s / (2 * h), ng - 2), r = s - g * 2 * h;  // B_g and F_(g+1)
+    const long long both = g < ng - 2 ? h : hl;
+    if (r < 2 * both) {
+        *fwd = r & 1;
+        *sl = r >> 1;
+        return *fwd ? g + 1 : g;
+    }
+    *fwd = false;
+    *sl = r < h + hl ? r - hl : r - (h + hl);
+    return r < h + hl ? ng - 2 : ng - 1;
+}
 
 // v <- M^{-1} v (forward) or M^{-T} v (backward), M the unit lower w x w triangle packed in
 // Ls (pk layout), panels of 32: warp 0 solves a panel's triangle, the other rows (columns)
@@ -2114,24 +2149,27 @@ __global__ void __launch_bounds__(kThreads, 2) sn_solve_kernel(SnSolveArgs a) {
     __shared__ double red[kThreads];
     __shared__ long long s_slot;
     const int T = blockDim.x, tid = threadIdx.x;
-    const long long half = (long long)a.nchunks * a.chains, total = 2 * half;
+    const long long total = 2LL * a.nchunks * a.chains;
     for (;;) {
         if (tid == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
         __syncthreads();
         const long long slot = s_slot;
         bool ok = __syncthreads_and(*(volatile int*)&a.hdr->status == STC_OK);
         if (slot >= total) break;
-        const bool fwd = slot < half;
-        const long long sl = fwd ? slot : slot - half;
-        const int32_t* tk = (fwd ? a.fwd : a.bwd) + 2 * (sl / a.chains);
+        bool fwd;
+        long long sl;
+        const long long grp = sn_solve_slot(slot, a.nchunks, a.chains, a.inflight, &fwd, &sl);
+        const long long ch0 = grp * a.inflight, cg = min(a.inflight, a.chains - ch0);
+        const int32_t* tk = (fwd ? a.fwd : a.bwd) + 2 * (sl / cg);
         const int J = tk[0], q = tk[1];
-        const long long ch = sl % a.chains;
+        const long long place = sl % cg, ch = ch0 + place;
         const SnSolveNode d = a.nodes[J];
         const double* P = a.factor + (ch / a.nrhs) * a.fstride + d.off;
         double* y = a.y + ch * a.n;
-        double* u = a.u + ch * a.nu;
-        double* part = a.part + ch * a.npart + d.poff;
-        int* fchunk = a.flags + ch * (2LL * a.nchunks + 2LL * a.nsn);  // forward chunks done
+        double* u = a.u + place * a.nu;
+        double* part = a.part + place * a.npart + d.poff;
+        const long long nflags = 2LL * a.nchunks + 2LL * a.nsn;
+        int* fchunk = a.flags + ch * nflags;                           // forward chunks done
         int* bchunk = fchunk + a.nchunks;                              // backward chunks done
         int* yflag = bchunk + a.nchunks;                               // y_J in place
         int* zflag = yflag + a.nsn;                                    // z_J in place
@@ -2153,6 +2191,12 @@ __global__ void __launch_bounds__(kThreads, 2) sn_solve_kernel(SnSolveArgs a) {
                 for (int z = tid; z < c.nchunk && ok; z += T) ok = wait_counter(fchunk + c.chunk + z, 1, a.spin, &a.hdr->status);
             }
             if (q > 0 && tid == 0 && ok) ok = wait_counter(yflag + J, 1, a.spin, &a.hdr->status);
+            if (grp > 0 && d.parent >= 0 && ok) {
+                // J's update vector of the previous group's chain: read by its parent's chunks
+                const SnSolveNode& p = a.nodes[d.parent];
+                const int* prev = fchunk - a.inflight * nflags + p.chunk;
+                for (int z = tid; z < p.nchunk && ok; z += T) ok = wait_counter(prev + z, 1, a.spin, &a.hdr->status);
+            }
             for (int r = tid; r < kSnSolveRows; r += T) us[r] = 0.0;
             ok = __syncthreads_and(ok);
             if (ok) {
@@ -2229,6 +2273,9 @@ __global__ void __launch_bounds__(kThreads, 2) sn_solve_kernel(SnSolveArgs a) {
             if (tid == 0 && ok) {
                 if (R > 0) ok = wait_counter(zflag + a.chunk_own[d.chunk + q], 1, a.spin, &a.hdr->status);
                 if (ok && q == 0) ok = wait_counter(yflag + J, 1, a.spin, &a.hdr->status);
+                // the partials of the previous group's chain: read by its first chunk
+                if (ok && q > 0 && grp > 0)
+                    ok = wait_counter(zflag + J - a.inflight * nflags, 1, a.spin, &a.hdr->status);
             }
             ok = __syncthreads_and(ok);
             if (ok) {
@@ -3302,18 +3349,31 @@ size_t counters_per_item(const stc_plan* P) { return is_sn(P) ? P->supernodal().
 size_t factorize_ws(const stc_plan* P, int64_t batch) {
     return sizeof(WorkHeader) + (size_t)batch * counters_per_item(P) * sizeof(int);
 }
+// Chains of the supernodal solve that are in flight together, each with update vectors and
+// backward partials of its own (17.8 MB at n = 180,020, where x has 1.4): as many as
+// kSnSolveBytes hold, kSnSolveChains at least.  At n = 180,020 with 16 / all in flight: 16
+// right-hand sides 23 ms, 64 91 / 79 ms, 256 361 / 274 ms and 0.7 / 4.9 GB.
+constexpr size_t kSnSolveBytes = 256u << 20;
+constexpr int64_t kSnSolveChains = 16;
+int64_t sn_inflight(const SnPlan& S, int64_t chains) {
+    const size_t per = std::max<size_t>(1, (size_t)(S.nu + S.npart) * sizeof(double));
+    return std::min<int64_t>(chains, std::max<int64_t>(kSnSolveChains, (int64_t)(kSnSolveBytes / per)));
+}
 // solve: step flags per chain (tile routes: one per forward and backward step; supernodal:
 // one per forward and backward chunk and two per supernode) and a y vector per chain;
-// supernodal: also the update vectors and backward partials of each chain
+// supernodal: also the update vectors and backward partials of the chains in flight
 size_t solve_flags(const stc_plan* P, int64_t chains) {
     size_t steps = 2 * (size_t)P->nt;
     if (is_sn(P)) steps = 2 * (size_t)P->supernodal().nchunks + 2 * (size_t)P->supernodal().nsn();
     return ((size_t)chains * steps * sizeof(int) + 255) / 256 * 256;
 }
 size_t solve_ws(const stc_plan* P, int64_t chains) {
-    size_t ylen = (size_t)(P->nt * P->nb);
-    if (is_sn(P)) ylen = (size_t)(P->n + P->supernodal().nu + P->supernodal().npart);
-    return sizeof(WorkHeader) + solve_flags(P, chains) + (size_t)chains * ylen * sizeof(double);
+    size_t len = (size_t)chains * P->nt * P->nb;
+    if (is_sn(P)) {
+        const SnPlan& S = P->supernodal();
+        len = (size_t)chains * P->n + (size_t)sn_inflight(S, chains) * (S.nu + S.npart);
+    }
+    return sizeof(WorkHeader) + solve_flags(P, chains) + len * sizeof(double);
 }
 
 int32_t pick_slices_impl(stc_plan* P, int64_t batch, int sms) {
@@ -3389,7 +3449,8 @@ int sn_solve(stc_plan* P, const void* d_factor, int64_t batch, int64_t nrhs, con
     a.flags = (int*)((char*)d_work + sizeof(WorkHeader));
     a.y = (double*)((char*)d_work + sizeof(WorkHeader) + flags);
     a.u = a.y + chains * P->n;
-    a.part = a.u + chains * Sp.nu;
+    a.inflight = sn_inflight(Sp, chains);
+    a.part = a.u + a.inflight * Sp.nu;
     a.chains = chains; a.nrhs = nrhs; a.nsn = Sp.nsn(); a.nchunks = Sp.nchunks; a.n = P->n; a.nu = Sp.nu;
     a.npart = Sp.npart;
     a.spin = P->opt.spin_limit > 0 ? P->opt.spin_limit : kDefaultSpin;

@@ -474,6 +474,7 @@ void stc::sn_build_solve(stc::SnPlan& S) {
     for (int32_t J = 0; J < nsn; ++J) {
         S.snodes[J].kbeg = nkids[J];
         S.snodes[J].kend = nkids[J + 1];
+        S.snodes[J].parent = parent[J];
         if (parent[J] >= 0) S.skids[at[parent[J]]++] = J;
     }
     S.srel.resize(uo);
