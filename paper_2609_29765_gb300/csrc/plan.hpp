@@ -303,9 +303,12 @@ struct SnPlan {
     std::vector<int32_t> srel;         // per below row: its position in the parent's rows
     std::vector<int32_t> schunk_own;   // per chunk: row supernode that owns its first row
     std::vector<int32_t> sfwd, sbwd;   // queue order, two per task: supernode, chunk
+    std::vector<int32_t> rowbeg, rowcells;  // per row supernode: its cells (J, I), I < J, ascending
     int64_t nu = 0, npart = 0;         // doubles of the update vectors, of the backward partials
     int32_t nchunks = 0;
     int32_t wmax = 0;                  // widest supernode
+    // modelled microseconds of the solve by rows and by the tree: longest path, work of a chain
+    double rows_path = 0.0, rows_work = 0.0, tree_path = 0.0, tree_work = 0.0;
     int32_t nsn() const { return (int32_t)first.size() - 1; }
     // item layout of the supernodal route: the arena, then one logdet partial per supernode
     int64_t poff() const { return (arena + 31) / 32 * 32; }
@@ -334,6 +337,7 @@ struct SnDev {
     int32_t* cell_rowoff = nullptr;
     SnSolveNode* snodes = nullptr;
     int32_t *skids = nullptr, *srel = nullptr, *schunk_own = nullptr, *sfwd = nullptr, *sbwd = nullptr;
+    int32_t *cptr = nullptr, *rowbeg = nullptr, *rowcells = nullptr;
     int32_t* order = nullptr;       // task of each queue position (sn_queue_order)
     int device = -1;
 };

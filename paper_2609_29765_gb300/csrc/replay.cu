@@ -23,6 +23,7 @@
 #include <functional>
 #include <queue>
 #include <climits>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <stdexcept>
@@ -2104,24 +2105,40 @@ __device__ __forceinline__ long long sn_solve_slot(long long slot, long long nch
     return r < h + hl ? ng - 2 : ng - 1;
 }
 
-// v <- M^{-1} v (forward) or M^{-T} v (backward), M the unit lower w x w triangle packed in
-// Ls (pk layout), panels of 32: warp 0 solves a panel's triangle, the other rows (columns)
+// v <- M^{-1} v (forward) or M^{-T} v (backward), M the unit lower w x w triangle in Ls, (r, c)
+// at ix(r, c), panels of 32: warp 0 solves a panel's triangle, the other rows (columns)
 // are then updated by a thread each.
-template <bool BACK>
-__device__ __forceinline__ void sn_tri_solve(double* v, const double* Ls, int w) {
+template <bool BACK, bool PRELOAD, class Ix>
+__device__ __forceinline__ void sn_tri_solve(double* v, const double* Ls, int w, Ix ix) {
     const int lane = threadIdx.x & 31;
     const int np = (w + 31) / 32;
     for (int qi = 0; qi < np; ++qi) {
         const int p = BACK ? (np - 1 - qi) * 32 : qi * 32, pw = min(32, w - p);
         if (threadIdx.x < 32) {
             double vi = lane < pw ? v[p + lane] : 0.0;
+            if (PRELOAD) {
+                // this lane's row (column) of the triangle first, so that a step of the chain is
+                // a shuffle and an FMA
+                double m[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j) {
+                    const bool live = BACK ? lane < j && j < pw : lane > j && lane < pw;
+                    m[j] = live ? Ls[BACK ? ix(p + j, p + lane) : ix(p + lane, p + j)] : 0.0;
+                }
+#pragma unroll
+                for (int jj = 0; jj < 32; ++jj) {
+                    const int j = BACK ? 31 - jj : jj;
+                    if (j < pw) vi = fma(-m[j], __shfl_sync(0xffffffffu, vi, j), vi);
+                }
+            } else {
 #pragma unroll 8
-            for (int jj = 0; jj < pw; ++jj) {
-                const int j = BACK ? pw - 1 - jj : jj;
-                const bool live = BACK ? lane < j : (lane > j && lane < pw);
-                const double m = live ? Ls[BACK ? pk(w, p + j, p + lane) : pk(w, p + lane, p + j)] : 0.0;
-                const double yj = __shfl_sync(0xffffffffu, vi, j);
-                if (live) vi = fma(-m, yj, vi);
+                for (int jj = 0; jj < pw; ++jj) {
+                    const int j = BACK ? pw - 1 - jj : jj;
+                    const bool live = BACK ? lane < j : (lane > j && lane < pw);
+                    const double m = live ? Ls[BACK ? ix(p + j, p + lane) : ix(p + lane, p + j)] : 0.0;
+                    const double yj = __shfl_sync(0xffffffffu, vi, j);
+                    if (live) vi = fma(-m, yj, vi);
+                }
             }
             if (lane < pw) v[p + lane] = vi;
         }
@@ -2131,10 +2148,10 @@ __device__ __forceinline__ void sn_tri_solve(double* v, const double* Ls, int w)
             double s0 = v[r], s1 = 0.0;
             int l = 0;
             for (; l + 1 < pw; l += 2) {
-                s0 = fma(-Ls[BACK ? pk(w, p + l, r) : pk(w, r, p + l)], v[p + l], s0);
-                s1 = fma(-Ls[BACK ? pk(w, p + l + 1, r) : pk(w, r, p + l + 1)], v[p + l + 1], s1);
+                s0 = fma(-Ls[BACK ? ix(p + l, r) : ix(r, p + l)], v[p + l], s0);
+                s1 = fma(-Ls[BACK ? ix(p + l + 1, r) : ix(r, p + l + 1)], v[p + l + 1], s1);
             }
-            if (l < pw) s0 = fma(-Ls[BACK ? pk(w, p + l, r) : pk(w, r, p + l)], v[p + l], s0);
+            if (l < pw) s0 = fma(-Ls[BACK ? ix(p + l, r) : ix(r, p + l)], v[p + l], s0);
             v[r] = s0 + s1;
         }
         __syncthreads();
@@ -2149,6 +2166,7 @@ __global__ void __launch_bounds__(kThreads, 2) sn_solve_kernel(SnSolveArgs a) {
     __shared__ double red[kThreads];
     __shared__ long long s_slot;
     const int T = blockDim.x, tid = threadIdx.x;
+    const auto packed = [&](int w) { return [w](int r, int c) { return pk(w, r, c); }; };
     const long long total = 2LL * a.nchunks * a.chains;
     for (;;) {
         if (tid == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
@@ -2217,7 +2235,7 @@ __global__ void __launch_bounds__(kThreads, 2) sn_solve_kernel(SnSolveArgs a) {
                     __syncthreads();
                 }
                 if (q == 0) {
-                    sn_tri_solve<false>(v, Ls, w);
+                    sn_tri_solve<false, false>(v, Ls, w, packed(w));
                     for (int i = tid; i < w; i += T) {
                         v[i] *= sdinv[i];
                         __stcg(y + d.first + i, v[i]);
@@ -2322,7 +2340,7 @@ __global__ void __launch_bounds__(kThreads, 2) sn_solve_kernel(SnSolveArgs a) {
                         v[i] = (__ldcg(y + d.first + i) - s) * sdinv[i];
                     }
                     __syncthreads();
-                    sn_tri_solve<true>(v, Ls, w);
+                    sn_tri_solve<true, false>(v, Ls, w, packed(w));
                     for (int i = tid; i < w; i += T) {
                         __stcg(y + d.first + i, v[i]);
                         a.x[ch * a.n + a.perm[d.first + i]] = v[i];
@@ -2349,6 +2367,143 @@ __global__ void fp64_probe_kernel(double* out, long long iters, double a, double
 #pragma unroll
     for (int i = 0; i < 8; ++i) s += c[i];
     out[blockIdx.x * (long long)blockDim.x + threadIdx.x] = s;
+}
+
+// The same solve with every step gathering from the cells of its row supernode one by one:
+// y_J = L_JJ^{-1} ((P b)_J - sum_I L_(J,I) y_I), z_J = L_JJ^{-T} (y_J - sum_K L_(K,J)^T z_K).
+// Only the newest cell's product lies between two steps of a chain of supernodes, where the
+// tree solve has a whole panel's; where the tree is wide a row has too many cells.  sn_by_rows
+// chooses.
+struct SnRowSolveArgs {
+    const SnDevCell* cells;
+    const int32_t* cptr;       // cells of column supernode J: [cptr[J], cptr[J+1]), diagonal first
+    const int32_t* rowbeg;     // cells of row supernode J: rowcells[rowbeg[J] .. rowbeg[J+1])
+    const int32_t* rowcells;
+    const int32_t *rows, *rowoff, *first, *perm;
+    const double* factor;
+    long long fstride;
+    const double* b;           // [chains][n]
+    double* x;                 // [chains][n]
+    double* y;                 // workspace [chains][n]
+    int* done;                 // workspace [chains][2 nsn]: y_J, z_J in place
+    WorkHeader* hdr;
+    long long chains, nrhs, n, spin;
+    int nsn, ldt;
+};
+
+__global__ void __launch_bounds__(kThreads, 2) sn_row_solve_kernel(SnRowSolveArgs a) {
+    extern __shared__ __align__(16) double smem[];
+    double* Ls = smem;                              // unit triangle of the diagonal block, odd columns
+    const auto ix = [&](int r, int c) { return r + c * a.ldt; };
+    __shared__ double v[kNbMax], sdinv[kNbMax], ys[kNbMax], part[kNbMax];
+    __shared__ int s_ok;
+    __shared__ long long s_slot;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const long long total = 2LL * a.nsn * a.chains;
+    for (;;) {
+        if (tid == 0) {
+            s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
+            s_ok = *(volatile int*)&a.hdr->status == STC_OK;
+        }
+        __syncthreads();
+        const long long slot = s_slot;
+        bool ok = s_ok;
+        __syncthreads();
+        if (slot >= total) break;
+        const int ti = (int)(slot / a.chains);
+        const long long ch = slot % a.chains;
+        const bool fwd = ti < a.nsn;
+        const int J = fwd ? ti : 2 * a.nsn - 1 - ti;
+        const double* F = a.factor + (ch / a.nrhs) * a.fstride;
+        double* y = a.y + ch * a.n;
+        int *ydone = a.done + ch * 2LL * a.nsn, *zdone = ydone + a.nsn;
+        const SnDevCell D = a.cells[a.cptr[J]];
+        const int w = D.w, c0 = a.first[J];
+        // thread 0 waits for *flag; every thread gets the outcome
+        const auto wait = [&](const int* flag) {
+            if (tid == 0) s_ok = wait_counter(flag, 1, a.spin, &a.hdr->status);
+            __syncthreads();
+            return (bool)s_ok;
+        };
+        if (ok) {
+            // diagonal block before any wait
+            const double* P = F + D.off;
+            for (int c = tid; c < w; c += kThreads) sdinv[c] = 1.0 / __ldg(P + c + (size_t)c * D.ld);
+            __syncthreads();
+            for (int c = warp; c < w; c += kThreads / 32)
+                for (int r = c + 1 + lane; r < w; r += 32) Ls[ix(r, c)] = __ldg(P + r + (size_t)c * D.ld) * sdinv[c];
+            if (fwd) {
+                for (int r = tid; r < w; r += kThreads) v[r] = a.b[ch * a.n + a.perm[c0 + r]];
+                for (int q = a.rowbeg[J]; q < a.rowbeg[J + 1] && ok; ++q) {  // ascending I
+                    const SnDevCell T = a.cells[a.rowcells[q]];
+                    const int* rows = a.rows + a.rowoff[a.rowcells[q]];
+                    const int cI = a.first[T.I];
+                    if (!(ok = wait(ydone + T.I))) break;
+                    for (int k = tid; k < T.w; k += kThreads) ys[k] = __ldcg(y + cI + k);
+                    __syncthreads();
+                    // two threads per row (T.h <= 128), halves of the inner range
+                    const int i = tid >> 1, hf = tid & 1;
+                    double s0 = 0.0, s1 = 0.0;
+                    if (i < T.h) {
+                        const double* Lr = F + T.off + i;
+                        int k = hf;
+                        for (; k + 2 < T.w; k += 4) {
+                            s0 = fma(__ldcg(Lr + (size_t)k * T.ld), ys[k], s0);
+                            s1 = fma(__ldcg(Lr + (size_t)(k + 2) * T.ld), ys[k + 2], s1);
+                        }
+                        if (k < T.w) s0 = fma(__ldcg(Lr + (size_t)k * T.ld), ys[k], s0);
+                    }
+                    double t = s0 + s1;
+                    t += __shfl_xor_sync(0xffffffffu, t, 1);
+                    if (i < T.h && hf == 0) v[rows[i] - c0] -= t;
+                    __syncthreads();
+                }
+            } else {
+                ok = wait(ydone + J);
+                if (ok)
+                    for (int r = tid; r < w; r += kThreads) v[r] = __ldcg(y + c0 + r);
+                for (int q = a.cptr[J + 1] - 1; q > a.cptr[J] && ok; --q) {  // last first
+                    const SnDevCell T = a.cells[q];
+                    const int* rows = a.rows + a.rowoff[q];
+                    if (!(ok = wait(zdone + T.J))) break;
+                    for (int i = tid; i < T.h; i += kThreads) ys[i] = __ldcg(y + rows[i]);
+                    __syncthreads();
+                    for (int k = warp; k < T.w; k += kThreads / 32) {
+                        const double* Lc = F + T.off + (size_t)k * T.ld;
+                        double t = 0.0;
+                        for (int i = lane; i < T.h; i += 32) t = fma(__ldcg(Lc + i), ys[i], t);
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
+                        if (lane == 0) part[k] = t;
+                    }
+                    __syncthreads();
+                    for (int k = tid; k < T.w; k += kThreads) v[k] -= part[k];
+                    __syncthreads();
+                }
+            }
+            if (ok) {
+                __syncthreads();
+                if (!fwd) {
+                    for (int i = tid; i < w; i += kThreads) v[i] *= sdinv[i];
+                    __syncthreads();
+                    if (w > 32) sn_tri_solve<true, true>(v, Ls, w, ix);
+                    else sn_tri_solve<true, false>(v, Ls, w, ix);
+                } else {
+                    if (w > 32) sn_tri_solve<false, true>(v, Ls, w, ix);
+                    else sn_tri_solve<false, false>(v, Ls, w, ix);
+                }
+                for (int i = tid; i < w; i += kThreads) {
+                    const double t = fwd ? v[i] * sdinv[i] : v[i];
+                    __stcg(y + c0 + i, t);
+                    if (!fwd) a.x[ch * a.n + a.perm[c0 + i]] = t;
+                }
+            }
+        }
+        __threadfence();
+        __syncthreads();
+        // (after a failed wait too, so that nothing waits for this task)
+        if (tid == 0) red_release_add((fwd ? ydone : zdone) + J, 1);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -3102,6 +3257,9 @@ int device_info(int* dev, int* sms) {
         if (cudaFuncSetAttribute(sn_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(kRPacked * sizeof(double))) != cudaSuccess)
             return STC_ERR_CUDA;
+        if (cudaFuncSetAttribute(sn_row_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)(kLdc * kNbMax * sizeof(double))) != cudaSuccess)
+            return STC_ERR_CUDA;
         if (cudaFuncSetAttribute(sn_selinv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRSmemBytes) !=
             cudaSuccess)
             return STC_ERR_CUDA;
@@ -3130,7 +3288,7 @@ void free_dev(stc_plan* P) {
         if (p) cudaFree(p);
     d = DevPlanArrays{};
     SnDev& q = P->sndev;
-    void* sptrs[] = {q.cells, q.tasks, q.upds, q.maps, q.first, q.value_map, q.csc_map, q.fill_src, q.stasks, q.scons, q.rows, q.cell_rowoff, q.order,
+    void* sptrs[] = {q.cells, q.tasks, q.upds, q.maps, q.first, q.value_map, q.csc_map, q.fill_src, q.stasks, q.scons, q.rows, q.cell_rowoff, q.order, q.cptr, q.rowbeg, q.rowcells,
                      q.snodes, q.skids, q.srel, q.schunk_own, q.sfwd, q.sbwd};
     for (void* p : sptrs)
         if (p) cudaFree(p);
@@ -3281,6 +3439,11 @@ int ensure_sn_impl(stc_plan* P, int dev) {
     if ((rc = upload(&d.schunk_own, S.schunk_own))) return rc;
     if ((rc = upload(&d.sfwd, S.sfwd))) return rc;
     if ((rc = upload(&d.sbwd, S.sbwd))) return rc;
+    if ((rc = upload(&d.cptr, S.cptr))) return rc;
+    if ((rc = upload(&d.rowbeg, S.rowbeg))) return rc;
+    std::vector<int32_t> rowcells = S.rowcells;
+    if (rowcells.empty()) rowcells.push_back(0);
+    if ((rc = upload(&d.rowcells, rowcells))) return rc;
     if ((rc = upload(&d.order, sn_queue_order(S, kSnQueueCtas)))) return rc;
     d.device = dev;
     return STC_OK;
@@ -3432,6 +3595,19 @@ int sn_factorize_scattered(stc_plan* P, int64_t batch, void* d_factor, void* d_w
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
 
+// Which of the two supernodal solves takes `chains` chains: by the modelled time of each, its
+// longest path and its work spread over the CTAs that it keeps busy (microseconds, see
+// sn_build_solve).  Measured, rows / tree: one chain on a band (n = 20,000, half-bandwidth 200)
+// 8.9 / 11.1 ms, half-bandwidth 20 10.2 / 14.6, a random pattern (n = 1,000, RCM) 0.70 / 1.64, a
+// 120 x 120 grid under RCM 7.0 / 12.2, but a grid of 32 x 32 under ND 0.22 / 0.14 and n = 22,520
+// spatio-temporal 3.7 / 1.0; 256 chains on that random pattern 12.4 / 8.4, 1,024 on a band
+// (n = 3,000, half-bandwidth 8) 9.5 / 3.2.
+double sn_model(double path, double work) { return std::cbrt(path * path * path + work * work * work); }
+bool sn_by_rows(const SnPlan& S, double chains) {
+    return sn_model(S.rows_path, chains * S.rows_work / 170.0) <
+           0.9 * sn_model(S.tree_path, chains * S.tree_work / (S.wmax <= 32 ? 780.0 : 200.0));
+}
+
 int sn_solve(stc_plan* P, const void* d_factor, int64_t batch, int64_t nrhs, const double* d_b, double* d_x,
              void* d_work, void* stream, int dev, int sms) {
     int rc;
@@ -3441,8 +3617,26 @@ int sn_solve(stc_plan* P, const void* d_factor, int64_t batch, int64_t nrhs, con
     cudaStream_t st = S(stream);
     const size_t flags = solve_flags(P, chains);
     if (cudaMemsetAsync(d_work, 0, sizeof(WorkHeader) + flags, st) != cudaSuccess) return STC_ERR_CUDA;
-    SnSolveArgs a{};
     const SnDev& d = P->sndev;
+    const size_t tri = (size_t)Sp.wmax * (Sp.wmax + 1) / 2 * sizeof(double);
+    if (sn_by_rows(Sp, (double)chains)) {
+        SnRowSolveArgs a{};
+        a.cells = d.cells; a.cptr = d.cptr; a.rowbeg = d.rowbeg; a.rowcells = d.rowcells; a.rows = d.rows;
+        a.rowoff = d.cell_rowoff; a.first = d.first; a.perm = P->dev.perm; a.factor = (const double*)d_factor;
+        a.fstride = Sp.item_doubles(); a.b = d_b; a.x = d_x; a.hdr = (WorkHeader*)d_work;
+        a.done = (int*)((char*)d_work + sizeof(WorkHeader));
+        a.y = (double*)((char*)d_work + sizeof(WorkHeader) + flags);
+        a.chains = chains; a.nrhs = nrhs; a.n = P->n; a.nsn = Sp.nsn();
+        a.ldt = Sp.wmax | 1;
+        a.spin = P->opt.spin_limit > 0 ? P->opt.spin_limit : kDefaultSpin;
+        // one CTA per SM where the path decides (a band, n = 20,000, half-bandwidth 20: 10.2 ms, two
+        // 11.4), two where the work does (64 chains, half-bandwidth 200: 11.5 / 9.9 ms)
+        const bool two = chains * Sp.rows_work / 100.0 > Sp.rows_path;
+        sn_row_solve_kernel<<<grid_of(P, two ? 2LL * sms : (long long)sms, 2LL * a.nsn * chains), kThreads,
+                              (size_t)a.ldt * Sp.wmax * sizeof(double), st>>>(a);
+        return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
+    }
+    SnSolveArgs a{};
     a.nodes = d.snodes; a.kids = d.skids; a.rel = d.srel; a.chunk_own = d.schunk_own; a.fwd = d.sfwd; a.bwd = d.sbwd;
     a.rows = d.rows; a.perm = P->dev.perm; a.factor = (const double*)d_factor; a.fstride = Sp.item_doubles();
     a.b = d_b; a.x = d_x; a.hdr = (WorkHeader*)d_work;
@@ -3457,9 +3651,8 @@ int sn_solve(stc_plan* P, const void* d_factor, int64_t batch, int64_t nrhs, con
     const long long total = 2LL * a.nchunks * chains;
     // narrow supernodes: CTAs of two warps, eight per SM (a step is then mostly latency)
     const bool narrow = Sp.wmax <= 32;
-    const size_t sm = (size_t)Sp.wmax * (Sp.wmax + 1) / 2 * sizeof(double);
     const int grid = grid_of(P, narrow ? 8LL * sms : 2LL * sms, total);
-    sn_solve_kernel<<<grid, narrow ? 64 : kThreads, sm, st>>>(a);
+    sn_solve_kernel<<<grid, narrow ? 64 : kThreads, tri, st>>>(a);
     return cudaGetLastError() == cudaSuccess ? STC_OK : STC_ERR_CUDA;
 }
 

@@ -16,13 +16,18 @@ def _stcov():
     return Ap, Ai, I.stcov_values((1.3, 0.6, 0.4), 12, 12, 12, 5), dict(coords=coords)
 
 
-def _band():  # 310 rows below a panel: two chunks, so backward partials
-    return (*I.band(1500, 310, seed=4), dict(ordering="natural"))
+def _blocks():  # dense blocks tied by border rows: panels of two chunks, so backward partials
+    import scipy.sparse as sp
+    rng = np.random.default_rng(4)
+    blocks, size, border = 16, 420, 60
+    A = sp.block_diag([rng.uniform(-1, 1, (size, size)) / size for _ in range(blocks)], format="csc")
+    B = sp.csc_matrix(rng.uniform(-1, 1, (border, blocks * size)) / size)
+    M = sp.bmat([[A + A.T, B.T], [B, sp.csc_matrix((border, border))]], format="csc")
+    return (*I.lower_csc(M + sp.diags(1.0 + np.asarray(abs(M).sum(axis=0)).ravel())), dict(ordering="natural"))
 
 
 # chains far beyond one group, the last group not full, by value sets and by right-hand sides
-@pytest.mark.parametrize("make", [_stcov, _band])
-@pytest.mark.parametrize("batch,nrhs", [(1, 10001), (3, 3333)])
+@pytest.mark.parametrize("make,batch,nrhs", [(_stcov, 1, 10001), (_stcov, 3, 3333), (_blocks, 1, 3001), (_blocks, 3, 999)])
 def test_groups(make, batch, nrhs):
     from paper_2609_29765_gb300.api import Plan
     Ap, Ai, Ax, kw = make()
