@@ -2589,6 +2589,9 @@ __device__ __forceinline__ void chunk_product(double* S0, double* S1, int R, int
 // 1.4 ms more of 30.
 constexpr int kSelWMax = 112;
 constexpr double kSelCond = 16.0;
+// Whether a block's task makes them: not for one panel with nothing to wait for, where they
+// take as long as the recurrence (n = 1: 48 us a call with them, 26 without).
+__device__ __forceinline__ bool selinv_inverts(int w, bool waits) { return w <= kSelWMax && (w > 16 || waits); }
 static_assert(kSelWMax * (kSelWMax + 1) / 2 + (kSelWMax / 16) * 272 <= kRCbuf, "the inverses fit behind the triangle");
 template <class LGet>
 __device__ void selinv_inverses(double* C, int w, LGet lget) {
@@ -2654,10 +2657,11 @@ __device__ void selinv_inverses(double* C, int w, LGet lget) {
 // rounding: error against 64 bits 3.9e-16 for 3.0e-16; one column at a time over the whole
 // block: 115).  Rows more than kd below the diagonal are outside the band and left alone.
 // lget(i, c): L_ic, i >= c.
-// S0: digits; S1: digits, then the panel's rows; sv: kNbMax doubles; be: kNbMax, the balance.
+// inv: the inverses are there.  S0: digits; S1: digits, then the panel's rows; sv: kNbMax
+// doubles; be: kNbMax, the balance.
 constexpr int kSelP = 16;
 template <class LGet>
-__device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, double* sv, int* be, LGet lget) {
+__device__ void selinv_diag(double* P, int w, int kd, bool inv, double* S0, double* S1, double* sv, int* be, LGet lget) {
     constexpr int LDX = kNbMax + 1 - kSelP;   // panel rows below: at most kNbMax - kSelP
     static_assert(LDX * kSelP + kSelP * (kSelP + 1) <= kRStage, "panel rows and its diagonal block fit a staging buffer");
     double* X = S1;                           // X(r, c), row b + r of the panel's columns
@@ -2728,7 +2732,7 @@ __device__ void selinv_diag(double* P, int w, int kd, double* S0, double* S1, do
         }
         __syncthreads();
         const double* W = P + w * (w + 1) / 2 + (p / kSelP) * 272;
-        if (w <= kSelWMax && W[16] != 0.0) {
+        if (inv && W[16] != 0.0) {
             // Sigma_pp = W^T W + W^T (Y W), Y = -L_pp^T Z' (P holds -Z'): products of an entry
             // per thread, Y and Y W in the rows' buffer.  W^T W apart, its largest term last:
             // the terms of 1/L^2, which dominate, are rounded once
@@ -2941,7 +2945,8 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
         } else if (t.kind == TASK_SDIAG && s_ok) {
             const int w = O.sw;
             for (int e = threadIdx.x; e < w * (w + 1) / 2; e += kThreads) C[e] = 0.0;
-            if (w <= kSelWMax) selinv_inverses(C, w, [&](int i, int c) { return diag_at(DT, D, nb, i, c); });
+            const bool inv = selinv_inverts(w, t.cend > t.cbeg);
+            if (inv) selinv_inverses(C, w, [&](int i, int c) { return diag_at(DT, D, nb, i, c); });
             __syncthreads();
             for (int ci = t.cbeg; ci < t.cend; ++ci) {
                 const DSCon cn = a.cons[ci];
@@ -2976,7 +2981,7 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
                 }
             }
             if (s_ok) {
-                selinv_diag(C, w, min(O.kd, nb - 1), S0, S1, sv, s_be,
+                selinv_diag(C, w, min(O.kd, nb - 1), inv, S0, S1, sv, s_be,
                             [&](int i, int c) { return diag_at(DT, D, nb, i, c); });
                 // padding rows and columns of a ragged tile: zero
                 write_sigma_diag(C, w, Sg + O.off, O, nb);
@@ -3126,7 +3131,8 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
             }
         } else if (t.kind == SN_S_DIAG && s_ok) {
             for (int e = threadIdx.x; e < w * (w + 1) / 2; e += kThreads) C[e] = 0.0;
-            if (w <= kSelWMax) selinv_inverses(C, w, lget);
+            const bool inv = selinv_inverts(w, t.cend > t.cbeg);
+            if (inv) selinv_inverses(C, w, lget);
             __syncthreads();
             for (int ci = t.cbeg; ci < t.cend; ++ci) {
                 const SnSCon q = a.cons[ci];
@@ -3152,7 +3158,7 @@ __global__ void __launch_bounds__(kThreads, 2) sn_selinv_kernel(SnSelinvArgs a) 
                 }
             }
             if (s_ok) {
-                selinv_diag(C, w, w - 1, S0, S1, sv, s_be, lget);
+                selinv_diag(C, w, w - 1, inv, S0, S1, sv, s_be, lget);
                 double* T = Sg + D.off;
                 for_rc(w, w, [&](int r, int c) {
                     if (r >= c) __stcg(T + r + (size_t)c * D.ld, C[pk(w, r, c)]);
