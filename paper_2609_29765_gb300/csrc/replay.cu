@@ -2396,19 +2396,14 @@ __global__ void __launch_bounds__(kThreads, 2) sn_row_solve_kernel(SnRowSolveArg
     double* Ls = smem;                              // unit triangle of the diagonal block, odd columns
     const auto ix = [&](int r, int c) { return r + c * a.ldt; };
     __shared__ double v[kNbMax], sdinv[kNbMax], ys[kNbMax], part[kNbMax];
-    __shared__ int s_ok;
     __shared__ long long s_slot;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const long long total = 2LL * a.nsn * a.chains;
     for (;;) {
-        if (tid == 0) {
-            s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
-            s_ok = *(volatile int*)&a.hdr->status == STC_OK;
-        }
+        if (tid == 0) s_slot = (long long)atomicAdd(&a.hdr->head, 1ULL);
         __syncthreads();
         const long long slot = s_slot;
-        bool ok = s_ok;
-        __syncthreads();
+        bool ok = __syncthreads_and(*(volatile int*)&a.hdr->status == STC_OK);
         if (slot >= total) break;
         const int ti = (int)(slot / a.chains);
         const long long ch = slot % a.chains;
@@ -2421,9 +2416,9 @@ __global__ void __launch_bounds__(kThreads, 2) sn_row_solve_kernel(SnRowSolveArg
         const int w = D.w, c0 = a.first[J];
         // thread 0 waits for *flag; every thread gets the outcome
         const auto wait = [&](const int* flag) {
-            if (tid == 0) s_ok = wait_counter(flag, 1, a.spin, &a.hdr->status);
-            __syncthreads();
-            return (bool)s_ok;
+            bool done = true;
+            if (tid == 0) done = wait_counter(flag, 1, a.spin, &a.hdr->status);
+            return (bool)__syncthreads_and(done);
         };
         if (ok) {
             // diagonal block before any wait
