@@ -3515,10 +3515,11 @@ size_t factorize_ws(const stc_plan* P, int64_t batch) {
 }
 // Chains of the supernodal solve that are in flight together, each with update vectors and
 // backward partials of its own (17.8 MB at n = 180,020, where x has 1.4): as many as
-// kSnSolveBytes hold, kSnSolveChains at least.  At n = 180,020 with 16 / all in flight: 16
-// right-hand sides 23 ms, 64 91 / 79 ms, 256 361 / 274 ms and 0.7 / 4.9 GB.
+// kSnSolveBytes hold, kSnSolveChains at least.  At n = 180,020 with 16 / 32 / 64 / all in
+// flight: 16 right-hand sides 23 ms, 64 91 / 84 / 79 / 79 ms, 256 361 / 333 / 307 / 274 ms and
+// 0.7 / 1.0 / 1.5 / 4.9 GB.
 constexpr size_t kSnSolveBytes = 256u << 20;
-constexpr int64_t kSnSolveChains = 16;
+constexpr int64_t kSnSolveChains = 32;
 int64_t sn_inflight(const SnPlan& S, int64_t chains) {
     const size_t per = std::max<size_t>(1, (size_t)(S.nu + S.npart) * sizeof(double));
     return std::min<int64_t>(chains, std::max<int64_t>(kSnSolveChains, (int64_t)(kSnSolveBytes / per)));

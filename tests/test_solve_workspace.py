@@ -14,6 +14,6 @@ def test_workspace_per_chain(dims):
     # from some number of chains on, a chain more is one vector of n and its step flags: four
     # ints a supernode or chunk at most, and there are no more of those than 3 n / 4
     assert P.workspace_bytes(40000) - P.workspace_bytes(20000) <= 20000 * (8 * n + 12 * n)
-    # 256 MB at most, or 16 chains
+    # 256 MB at most, or 32 chains
     one = P.workspace_bytes(1)
-    assert P.workspace_bytes(40000) <= 40000 * 20 * n + max(16 * one, 256 << 20) + 4096
+    assert P.workspace_bytes(40000) <= 40000 * 20 * n + max(32 * one, 256 << 20) + 4096
