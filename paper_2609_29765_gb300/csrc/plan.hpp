@@ -122,8 +122,8 @@ struct DUpd {
 
 // Selected inverse (Takahashi recurrence on the tile map), walked in reverse order.
 //   TASK_SOFF  Sigma_mk = -(sum_j Sigma_(m,j) L_jk) L_kk^{-1} on the stored columns of (m,k)
-//   TASK_SDIAG Sigma_kk from Z = sum_j Sigma_jk^T L_jk and the element recurrence inside
-//              the diagonal tile
+//   TASK_SDIAG Sigma_kk from Z = sum_j Sigma_jk^T L_jk, the diagonal tile by 16-column
+//              panels
 enum : int32_t { TASK_SOFF = 0, TASK_SDIAG = 1 };
 enum : int32_t { SCON_MJ = 0, SCON_JM = 1, SCON_DIAG = 2, SCON_OWN = 3 };
 
@@ -233,8 +233,8 @@ struct SnDevUpd {
 // L(K',J)) L_JJ^{-1}; the Sigma block comes from the diagonal cell of K (K' = K), from
 // the cell (K,K') of supernode K' (K' < K) or transposed from the cell (K',K) of K
 // (K' > K), rows located by searching the source cell's row list.  A diagonal task forms
-// Z = sum over J's cells of Sigma(K',J)^T L(K',J) and runs the element recurrence inside
-// the diagonal block.
+// Z = sum over J's cells of Sigma(K',J)^T L(K',J) and finishes the diagonal block by
+// 16-column panels.
 enum : int32_t { SN_S_OFF = 0, SN_S_DIAG = 1 };
 enum : int32_t { SN_SC_SAME = 0, SN_SC_LOWER = 1, SN_SC_UPPER = 2, SN_SC_OWN = 3 };
 struct SnSTask {

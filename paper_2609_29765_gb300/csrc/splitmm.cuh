@@ -1,23 +1,32 @@
-// splitmm.cuh -- FP64 tile products on the tensor cores by an error-free split.
+// splitmm.cuh -- FP64 tile products on the tensor cores by a split into digits.
 //
 // sm_103a has no FP64 tensor kind worth using (DMMA shares the 2-DFMA/clk/SM FP64 pipe),
-// so C -= A B^T is formed from exact integer products (the error-free transformation of
-// Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012): each operand row of a
-// 16-column chunk is scaled by a power of two to 62-bit fixed point, cut into eight
+// so C -= A B^T is formed from integer products of digits (after the error-free
+// transformation of Ozaki, Ogita, Oishi and Rump, Numer. Algorithms 59, 2012): each operand
+// row of a 16-column chunk is scaled by a power of two to 62-bit fixed point, cut into eight
 // balanced base-256 digits, and the digit pairs (i, j), i + j <= 7, are multiplied by
 // mma.sync f16 with f32 accumulators, one accumulator per i + j.  A digit is at most 128
 // in magnitude, so a sum over 16 columns and 8 pairs stays below 2^21 and every f32 sum
-// is exact.  The eight sums are put together in integers (one rounding to 2^-58 of the
-// largest product the rows allow), rounded to a double and subtracted from C: two
-// roundings per 16 columns where sixteen fused multiply-adds made sixteen.
+// is exact.  The eight sums are put together in integers, rounded to a double and subtracted
+// from C.
+//
+// What is exact and what is not: the sums of the 36 pairs are.  An entry more than 2^9 below
+// its row's largest of the chunk loses its last bits (truncated), one 2^62 below all of them;
+// the 28 pairs beyond are left out; the sum is rounded twice.  All of it is at most 2^-53 of
+// (largest of A's row) x (largest of B's row) per chunk, with digits of one sign throughout;
+// with the digits of ordinary data about 2^-58.  That is relative to the row maxima, not to
+// sum |a_k b_k| as the roundings of FMAs are.  For rows of L over the same columns it is what
+// the factorization's error is measured in (|L_ik| <= sqrt(a_ii), units of the variables scale
+// whole rows); products of other operands have to be balanced first (Balance below).
 //
 // What bounds it: 36 tensor products per FP64 product at 605 TFLOP/s (mma.sync f16,
 // measured) are 16.8 TFLOP/s of FP64 work against 1.26 on the DFMA pipe; the split, the
 // digit expansion and the epilogue issue about as long as the tensor pipe runs.  Measured,
-// supernodal route: one factorization at n = 180,020 517 -> 251 ms, a 48^3 FEM operator
-// 180 -> 98 ms, 16 sets at n = 22,520 95 -> 57 ms, and the products and their staging no
-// more than 37 % of the CTAs' time (the rest waits for other tasks).  Tile routes: 64 bands
-// (n = 50,000, half-bandwidth 200) 178 -> 89 ms with the 16-column panels of POTRF and TRSM.
+// supernodal route: one factorization at n = 180,020 517 -> 251 ms by the products alone
+// (107 with two CTAs per SM and the scheduled queue), a 48^3 FEM operator 180 -> 98 (33) ms,
+// 16 sets at n = 22,520 95 -> 57 (35) ms; of the CTAs' time at n = 180,020 the products then
+// take 55 %, their staging 17 %.  Tile routes: 64 bands (n = 50,000, half-bandwidth 200)
+// 178 -> 89 ms with the 16-column panels of POTRF and TRSM.
 //
 // Rows whose largest entry is not finite or lies outside 2^[-400, 400] (where the scale
 // arithmetic could leave the exponent range), and rows of subnormals, are reported by the

@@ -16,7 +16,7 @@ def _bordered(blocks, size, border):
     """Dense blocks tied by dense border rows: chains of panels with up to size + border rows
     below, and a root with cells of every panel."""
     rng = np.random.default_rng(size)
-    A = sp.block_diag([rng.uniform(-1, 1, (size, size)) / size for _ in range(blocks)], format="csc")
+    A = sp.block_diag([sp.csc_matrix(rng.uniform(-1, 1, (size, size)) / size) for _ in range(blocks)], format="csc")
     B = sp.csc_matrix(rng.uniform(-1, 1, (border, blocks * size)) / size)
     M = sp.bmat([[A + A.T, B.T], [B, sp.csc_matrix((border, border))]], format="csc")
     M = M + sp.diags(1.0 + np.asarray(abs(M).sum(axis=0)).ravel())

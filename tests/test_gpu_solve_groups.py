@@ -20,7 +20,7 @@ def _blocks():  # dense blocks tied by border rows: panels of two chunks, so bac
     import scipy.sparse as sp
     rng = np.random.default_rng(4)
     blocks, size, border = 16, 420, 60
-    A = sp.block_diag([rng.uniform(-1, 1, (size, size)) / size for _ in range(blocks)], format="csc")
+    A = sp.block_diag([sp.csc_matrix(rng.uniform(-1, 1, (size, size)) / size) for _ in range(blocks)], format="csc")
     B = sp.csc_matrix(rng.uniform(-1, 1, (border, blocks * size)) / size)
     M = sp.bmat([[A + A.T, B.T], [B, sp.csc_matrix((border, border))]], format="csc")
     return (*I.lower_csc(M + sp.diags(1.0 + np.asarray(abs(M).sum(axis=0)).ravel())), dict(ordering="natural"))
