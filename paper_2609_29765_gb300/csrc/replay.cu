@@ -6,8 +6,8 @@
 // GB300 notes that shape this file:
 //  * FP64 runs at 2 DFMA/clk/SM (1.26 TFLOP/s; mma.sync.m8n8k4.f64 shares that pipe and is
 //    no faster), a dependent DFMA takes 64-70 clocks of a warp whatever its active lanes.  So
-//    the tile products of any size go to the tensor cores as exact integer products of split
-//    operands (splitmm.cuh), small ones are one entry per thread, and POTRF, TRSM and the
+//    the tile products of any size go to the tensor cores as integer products of operands
+//    split into digits (splitmm.cuh), small ones are one entry per thread, and POTRF, TRSM and the
 //    solves, which are chains, are laid out for few dependent FP64 instructions.  Tiles live
 //    in shared memory.
 //  * One persistent kernel per call walks the whole DAG of every batch item: CTAs take
@@ -575,7 +575,7 @@ constexpr int kM16 = kP16 + 1;  // leading dimension of a panel's 16 x 16 unit t
 // last step is folded into the column M_rj = u_rj / d_j (third-order Householder iteration
 // from the hardware estimate, e = 1 - d y0, 1 / d = y0 (1 + e + e^2 + ...)), and the 16
 // square roots come at the end side by side: 11,400 clocks alone, 17,100 with a reciprocal
-// square root per pivot.  A block with a pivot outside [2^-991, 2^992) (an integer test: a
+// square root per pivot.  A block with a pivot outside [2^-991, 2^989) (an integer test: a
 // double comparison is an FP64 instruction too) is done again one column at a time.
 __device__ int potrf_diag16(double* P, int nb, int p, int pw, double* M, double* inv) {
     const int lane = threadIdx.x & 31, r = lane >> 1, h = lane & 1;
@@ -2507,9 +2507,8 @@ __global__ void __launch_bounds__(kThreads, 2) sn_row_solve_kernel(SnRowSolveArg
 // one persistent kernel walking block columns in reverse order with per-tile counters.
 // Off-diagonal tile:  Sigma_mk = -(sum_j Sigma_(m,j) L_jk) L_kk^{-1}  (stored columns of
 // (m,k); entries the symbolic factor proves zero are never read by structural outputs).
-// Diagonal tile: Z = sum_j Sigma_jk^T L_jk, then column c = w-1..0 of the tile:
-//   Sigma_rc = (-Z_rc - sum_{i>c} L_ic Sigma_ri) / L_cc          (r > c)
-//   Sigma_cc = 1/L_cc^2 + (-Z_cc - sum_{i>c} L_ic Sigma_ic) / L_cc
+// Diagonal tile: Z = sum_j Sigma_jk^T L_jk, then the tile by 16-column panels (selinv_diag).
+// Its products are split with the inner index balanced by the variables' deviations (sd_exp).
 // ---------------------------------------------------------------------------
 struct SelinvArgs {
     const DTile* tiles;
@@ -2536,9 +2535,10 @@ __device__ __forceinline__ double sym_at(const double* T, const DTile& d, int nb
 
 // Balance of the split products here (see splitmm.cuh): an inner index is a variable i, with
 // Sigma_ri on one side and L_ic on the other, and 2^e_i is the standard deviation
-// sqrt(Sigma_ii).  Then |Sigma_ri| / 2^e_i <= 2 sqrt(Sigma_rr) along a row, so the cut stays
-// below 2^-55 sqrt(Sigma_rr) max_i |L_ic| sqrt(Sigma_ii): what the rounding of the DFMAs is
-// bounded by, and as invariant under a change of units.  Restated on the CPU against 60 digits
+// sqrt(Sigma_ii) within a factor of 2.  Then |Sigma_ri| / 2^e_i <= 2 sqrt(Sigma_rr) along a
+// row, so the error of a chunk stays below 2^-52 (ordinary data: 2^-57) of sqrt(Sigma_rr)
+// max_i |L_ic| sqrt(Sigma_ii): what the rounding of DFMAs is bounded by, and as invariant
+// under a change of units.  Restated on the CPU against 60 digits
 // (block elimination, n = 49..256, products alone; error of Sigma_ij over sqrt(Sigma_ii
 // Sigma_jj)): first-order walk + 1e-8 with units 2^U(-20, 20) 4e-8 without balance, 1e-15 with
 // it (DFMAs 1e-15), third-order 8e-2 / 3e-10 (2e-10); scaled by L_ii in place of the deviation a
@@ -2996,8 +2996,8 @@ __global__ void __launch_bounds__(kThreads, 2) selinv_kernel(SelinvArgs a) {
 // with Sigma(rows_K, rows_K') read from the diagonal cell of K (K' = K), from the cell
 // (K,K') of supernode K' (K' < K) or transposed from the cell (K',K) of K (K' > K), each
 // row located by a search of the source cell's row list.  Diagonal task: C = -Z,
-// Z = sum over J's cells of Sigma(K',J)^T L(K',J), then the element recurrence inside the
-// diagonal block (as for a diagonal tile).
+// Z = sum over J's cells of Sigma(K',J)^T L(K',J), then the diagonal block by 16-column
+// panels (as for a diagonal tile).
 // ---------------------------------------------------------------------------
 struct SnSelinvArgs {
     const SnDevCell* cells;
@@ -3579,8 +3579,9 @@ void fill_sn(SnArgs& a, const stc_plan* P, void* d_factor, int* counters, int32_
     a.spin = P->opt.spin_limit > 0 ? P->opt.spin_limit : kDefaultSpin;
 }
 
-// Supernodal factorization: the persistent kernel over (task, item) slots, every item of
-// a task in lockstep (the left-looking task order is topological).
+// Supernodal factorization: the persistent kernel over (task, item) slots, every item of a
+// task in lockstep.  No wait can deadlock because a task comes behind every task whose cells
+// it reads: in the order of sn_queue_order, and in the stored left-looking one.
 int sn_factorize_scattered(stc_plan* P, int64_t batch, void* d_factor, void* d_work, int32_t* d_info, void* stream,
                            int dev, int sms) {
     int rc;
