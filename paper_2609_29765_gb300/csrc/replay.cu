@@ -2072,15 +2072,14 @@ struct SnSolveArgs {
     int* flags;                // workspace [chains][2 nchunks + 2 nsn]
     WorkHeader* hdr;
     long long chains, nrhs, n, nu, npart, spin;
-    long long inflight;        // chains of a group
+    long long inflight, groups;  // chains of a group, groups
     int nsn, nchunks;
 };
 
-// Queue slot -> chain group (returned), direction, and position among the group's steps of
+// Queue slot -> chain group of the ng (returned), direction, and position among the group's steps of
 // that direction: F_0, then B_(g-1) and F_g in turn, then B of the last group.
 __device__ __forceinline__ long long sn_solve_slot(long long slot, long long nchunks, long long chains, long long inflight,
-                                                   bool* fwd, long long* sl) {
-    const long long ng = (chains + inflight - 1) / inflight;
+                                                   long long ng, bool* fwd, long long* sl) {
     const long long h = nchunks * inflight, hl = nchunks * (chains - (ng - 1) * inflight);  // steps of a group, of the last
     const long long first = ng > 1 ? h : hl;
     if (slot < first) {
@@ -2176,7 +2175,7 @@ __global__ void __launch_bounds__(kThreads, 2) sn_solve_kernel(SnSolveArgs a) {
         if (slot >= total) break;
         bool fwd;
         long long sl;
-        const long long grp = sn_solve_slot(slot, a.nchunks, a.chains, a.inflight, &fwd, &sl);
+        const long long grp = sn_solve_slot(slot, a.nchunks, a.chains, a.inflight, a.groups, &fwd, &sl);
         const long long ch0 = grp * a.inflight, cg = min(a.inflight, a.chains - ch0);
         const int32_t* tk = (fwd ? a.fwd : a.bwd) + 2 * (sl / cg);
         const int J = tk[0], q = tk[1];
@@ -3647,6 +3646,7 @@ int sn_solve(stc_plan* P, const void* d_factor, int64_t batch, int64_t nrhs, con
     a.y = (double*)((char*)d_work + sizeof(WorkHeader) + flags);
     a.u = a.y + chains * P->n;
     a.inflight = sn_inflight(Sp, chains);
+    a.groups = (chains + a.inflight - 1) / a.inflight;
     a.part = a.u + a.inflight * Sp.nu;
     a.chains = chains; a.nrhs = nrhs; a.nsn = Sp.nsn(); a.nchunks = Sp.nchunks; a.n = P->n; a.nu = Sp.nu;
     a.npart = Sp.npart;
